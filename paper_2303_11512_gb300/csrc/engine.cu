@@ -52,7 +52,7 @@ void op_apply(mgmlmc_hier* h, int l, const typename CT<R>::T* x, typename CT<R>:
 
 template <typename R>
 void sap_sweep(mgmlmc_hier* h, int l, const typename CT<R>::T* f, typename CT<R>::T* x, int nrhs,
-               const int* active, void* x16) {
+               const int* active, void* x16, bool zero) {
   const LevelData& L = h->lv[l];
   cudaStream_t st = h->ctx->stream;
   if (sizeof(R) == 8 && !L.sap64_ok) throw Error(MGMLMC_ERR_INVALID_ARG, "FP64 SAP inverse not built at this level");
@@ -72,7 +72,7 @@ void sap_sweep(mgmlmc_hier* h, int l, const typename CT<R>::T* f, typename CT<R>
   for (int color = 0; color < 2; ++color) {
     if (l == 0)
       sap_half_fine<R>(st, links_of<R>(L), (R)L.diag, L.side, L.sap_bs, sapinv_of<R>(L), f, x, color, nrhs, active,
-                       sizeof(R) == 4 && L.sapinv32_t);
+                       sizeof(R) == 4 && L.sapinv32_t, !zero ? SAP_X : color == 0 ? SAP_ZERO : SAP_OTHER);
     else
       sap_half_coarse<R>(st, st_of<R>(L), L.side, L.dof, L.sap_bs, sapinv_of<R>(L), f, x, color, nrhs, active);
   }
@@ -111,9 +111,11 @@ void vcycle(mgmlmc_hier* h, int l, const typename CT<R>::T* r, typename CT<R>::T
     if (h->use_tc(l) && tc_block_selected(L.tc_bf, L.side, nrhs))
       e16 = h->work("vc_e16", l, sizeof(uint32_t) * L.n * nrhs);
   }
-  vzero<C>(st, e, L.n, nrhs);
+  // the fine smoother starts from zero without reading e; its two colours then write every site
+  const bool lazy_zero = l == 0 && L.sap_bs == 4 && h->prm.pre_smooth > 0;
+  if (!lazy_zero) vzero<C>(st, e, L.n, nrhs);
   if (e16) MG_CUDA(cudaMemsetAsync(e16, 0, sizeof(uint32_t) * L.n * nrhs, st));
-  for (int s = 0; s < h->prm.pre_smooth; ++s) sap_sweep<R>(h, l, r, e, nrhs, active, e16);
+  for (int s = 0; s < h->prm.pre_smooth; ++s) sap_sweep<R>(h, l, r, e, nrhs, active, e16, lazy_zero && s == 0);
   bool done = false;
   if constexpr (sizeof(R) == 4) {
     if (h->use_tc(l)) {  // res = r - D e on the tensor cores (preconditioner accuracy)
@@ -135,8 +137,8 @@ void vcycle(mgmlmc_hier* h, int l, const typename CT<R>::T* r, typename CT<R>::T
   for (int s = 0; s < h->prm.post_smooth; ++s) sap_sweep<R>(h, l, r, e, nrhs, active, e16);
 }
 
-template void sap_sweep<float>(mgmlmc_hier*, int, const float2*, float2*, int, const int*, void*);
-template void sap_sweep<double>(mgmlmc_hier*, int, const double2*, double2*, int, const int*, void*);
+template void sap_sweep<float>(mgmlmc_hier*, int, const float2*, float2*, int, const int*, void*, bool);
+template void sap_sweep<double>(mgmlmc_hier*, int, const double2*, double2*, int, const int*, void*, bool);
 template void op_apply<float>(mgmlmc_hier*, int, const float2*, float2*, const float2*, int, const int*);
 template void op_apply<double>(mgmlmc_hier*, int, const double2*, double2*, const double2*, int, const int*);
 template void vcycle<float>(mgmlmc_hier*, int, const float2*, float2*, int, const int*);

@@ -12,6 +12,9 @@
 //   (1 + sigma_1) x = h (1,  1),  h = x0 + x1
 //   (1 - sigma_2) x = h (1, -i),  h = x0 + i x1
 //   (1 + sigma_2) x = h (1,  i),  h = x0 - i x1
+#include <algorithm>
+#include <type_traits>
+
 #include "ops.cuh"
 
 namespace mg {
@@ -229,41 +232,290 @@ void fine_block_matrices(cudaStream_t st, const double2* l64, double diag, int L
 }
 
 // ---- SAP half sweep on the fine level ----------------------------------------
-// One CTA per block of the colour; the block inverse is staged in shared memory
-// once and applied to all right-hand sides in groups of G.
-template <typename R, int BS, bool TRANS>
-__global__ void __launch_bounds__(256) k_sap_fine(const typename CT<R>::T* __restrict__ lk, R diag, int L,
-                                                  const typename CT<R>::T* __restrict__ inv,
-                                                  const typename CT<R>::T* __restrict__ f,
-                                                  typename CT<R>::T* __restrict__ x, int color, int nrhs,
-                                                  const int* __restrict__ active) {
+// x_B += D_BB^{-1} (f - D x)_B on the blocks of one colour.  `known` says what of x is read: all of it (SAP_X),
+// nothing (SAP_ZERO: x counts as zero, the first half sweep of a cycle), or the other colour only (SAP_OTHER: x
+// counts as zero on this colour, the second half sweep).
+
+__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
+}
+__device__ __forceinline__ void cp_async8(void* dst, const void* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
+}
+
+// FP32, 4 x 4 blocks.  An item is one block; blockIdx.y picks the tile of RG right-hand sides, which a CTA keeps.
+// Two warps per CTA and one shared-memory stage (21 KB at RG = 16, ten CTAs per SM, each in another phase):
+//   fetch     f on the block, x on the block and on the 16 sites around it, the inverse, all by cp.async
+//   residual  lane = rhs, consecutive sites per thread: f - D x replaces f in place
+//   product   inv_B r: a thread owns two sites (4 complex rows) times NR = RG / 8 rhs
+// What bounds it: the bytes that shared memory returns to registers (128 a clock and SM; 48 bytes for 32 FMAs in the
+// product), then DRAM (390 MB at L = 512, 32 rhs: f and x come as whole 128-byte lines although a colour uses every
+// other 64 bytes).  Half sweep at L = 512: 100 us with 32 rhs, 56 with 16, 37 with 8.  Measured at 32 rhs and left:
+// loads to registers at the start of an item 147 us (global latency); one row and 8 rhs per thread (72 bytes for 32
+// FMAs) 130 us whatever the occupancy, prefetch depth or packing of the FMAs.  The sums run over the columns in order.
+template <int RG>
+struct SapF {
+  static constexpr int RP = RG + 1;  // padded row: 8 sites of one rhs hit distinct banks in the final update
+  float4 f[16 * RG];
+  float4 x[32 * RP];    // block sites, then the sites around it: -x, +x (by row), -t, +t (by column)
+  float2 inv[32 * 32];  // transposed: row j holds column j of the inverse
+  float2 lx[20];        // x links of sites (row, -1 .. 3)
+  float2 lt[20];        // t links of sites (-1 .. 3, column)
+};
+
+template <int RG>
+__global__ void __launch_bounds__(64) k_sap_fine4_fp32(const float2* __restrict__ lk, float diag, int L,
+                                                       const float2* __restrict__ inv, const float2* __restrict__ f,
+                                                       float2* __restrict__ x, int color, int nrhs, int nitems,
+                                                       int known, const int* __restrict__ active) {
+  constexpr int RP = SapF<RG>::RP, T = 64, NR = RG / 8, RSTEP = T / (4 * RG) ? T / (4 * RG) : 1;
+  constexpr int RTH = T / 4 < RG ? T / 4 : RG;  // rhs that the CTA's threads fetch at once
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  SapF<RG>& s = *reinterpret_cast<SapF<RG>*>(smem_raw);
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int nbx = L / 4, half = nbx / 2, r0 = blockIdx.y * RG;
+  const size_t n = 2 * (size_t)L * L;
+  const unsigned live_mask =
+      __ballot_sync(0xffffffffu, lane < RG && r0 + lane < nrhs && !(active && !active[r0 + lane]));
+  // fetch: site fj of row fi + RSTEP m of rhs frr + RTH k (64 consecutive bytes per rhs and row)
+  const int fj = tid & 3, frr = (tid >> 2) % RTH, fi = (tid >> 2) / RTH;
+  const int g = tid & 7, rg = tid >> 3;  // row group and rhs group of the product
+  for (int item = blockIdx.x; item < nitems; item += gridDim.x) {
+    const int BT = item / half, t0 = 4 * BT, x0 = 4 * (2 * (item - BT * half) + ((BT + color) & 1));
+    const int tm = t0 == 0 ? L - 1 : t0 - 1, tp = t0 + 4 == L ? 0 : t0 + 4;
+    const int xm = x0 == 0 ? L - 1 : x0 - 1, xp = x0 + 4 == L ? 0 : x0 + 4;
+    {
+      const char* I = reinterpret_cast<const char*>(inv + (size_t)(BT * nbx + x0 / 4) * 1024);
+#pragma unroll
+      for (int q = 0; q < 512 / T; ++q)
+        cp_async16(reinterpret_cast<char*>(s.inv) + (tid + q * T) * 16, I + (tid + q * T) * 16);
+      if (tid < 20) {
+        const int i = tid / 5, j = tid - 5 * i;
+        cp_async8(&s.lx[tid], lk + 2 * ((t0 + i) * L + (j ? x0 + j - 1 : xm)));
+      } else if (tid >= 32 && tid < 52) {
+        const int i = (tid - 32) >> 2, j = tid & 3;
+        cp_async8(&s.lt[tid - 32], lk + 2 * ((i ? t0 + i - 1 : tm) * L + x0 + j) + 1);
+      }
+#pragma unroll
+      for (int k = 0; k < RG / RTH; ++k) {
+        const int rr = frr + RTH * k;
+        if (!((live_mask >> rr) & 1)) continue;
+        const float2* frow = f + (size_t)(r0 + rr) * n;
+        const float2* xrow = x + (size_t)(r0 + rr) * n;
+#pragma unroll
+        for (int m = 0; m < 4 / RSTEP; ++m) {
+          const int i = fi + RSTEP * m, q = 4 * i + fj;
+          const int site = (t0 + i) * L + x0 + fj;
+          cp_async16(&s.f[q * RG + rr], frow + 2 * site);
+          if (known == SAP_X) cp_async16(&s.x[q * RP + rr], xrow + 2 * site);
+          if (known != SAP_ZERO) {
+            const int edge = i == 0 ? (t0 + fj) * L + xm : i == 1 ? (t0 + fj) * L + xp : (i == 2 ? tm : tp) * L + x0 + fj;
+            cp_async16(&s.x[(16 + q) * RP + rr], xrow + 2 * edge);
+          }
+        }
+      }
+      asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;" ::: "memory");
+    }
+    __syncthreads();
+    if (known != SAP_ZERO) {
+      constexpr int SPT = 16 * RG / T;  // sites per thread: consecutive ones
+      const int rr = tid % RG, j0 = (tid / RG) * SPT;
+      float2 a0, a1;
+      auto at = [&](int k) {
+        const float4 v = k >= 16 || known == SAP_X ? s.x[k * RP + rr] : make_float4(0.f, 0.f, 0.f, 0.f);
+        a0 = make_float2(v.x, v.y);
+        a1 = make_float2(v.z, v.w);
+      };
+#pragma unroll
+      for (int q = 0; q < SPT; ++q) {
+        const int j = j0 + q, jx = j & 3, jt = j >> 2;
+        at(j);
+        float2 o0 = cscale(a0, diag), o1 = cscale(a1, diag);
+        {
+          at(jx < 3 ? j + 1 : 20 + jt);
+          const float2 u = cmul(s.lx[5 * jt + jx + 1], csub(a0, a1));
+          o0 = cadd(o0, u);
+          o1 = csub(o1, u);
+        }
+        {
+          at(jx > 0 ? j - 1 : 16 + jt);
+          const float2 u = cmulc(s.lx[5 * jt + jx], cadd(a0, a1));
+          o0 = cadd(o0, u);
+          o1 = cadd(o1, u);
+        }
+        {
+          at(jt < 3 ? j + 4 : 28 + jx);
+          const float2 u = cmul(s.lt[4 * jt + 4 + jx], cadd(a0, cmuli(a1)));
+          o0 = cadd(o0, u);
+          o1 = cadd(o1, cmulmi(u));
+        }
+        {
+          at(jt > 0 ? j - 4 : 24 + jx);
+          const float2 u = cmulc(s.lt[4 * jt + jx], cadd(a0, cmulmi(a1)));
+          o0 = cadd(o0, u);
+          o1 = cadd(o1, cmuli(u));
+        }
+        const float4 fv = s.f[j * RG + rr];
+        s.f[j * RG + rr] = make_float4(fv.x - o0.x, fv.y - o0.y, fv.z - o1.x, fv.w - o1.y);
+      }
+      __syncthreads();
+    }
+    float2 acc[4][NR];
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+      for (int b = 0; b < NR; ++b) acc[a][b] = make_float2(0.f, 0.f);
+#pragma unroll 2
+    for (int j = 0; j < 16; ++j) {
+      float4 v[NR];
+#pragma unroll
+      for (int b = 0; b < NR; ++b) v[b] = s.f[j * RG + rg * NR + b];
+#pragma unroll
+      for (int sp = 0; sp < 2; ++sp) {
+        const float4* mi = reinterpret_cast<const float4*>(s.inv + (2 * j + sp) * 32);
+        const float4 m0 = mi[g], m1 = mi[8 + g];  // rows 2g, 2g + 1 and 16 + 2g, 17 + 2g
+#pragma unroll
+        for (int b = 0; b < NR; ++b) {
+          const float2 w = sp ? make_float2(v[b].z, v[b].w) : make_float2(v[b].x, v[b].y);
+          acc[0][b] = cfma(make_float2(m0.x, m0.y), w, acc[0][b]);
+          acc[1][b] = cfma(make_float2(m0.z, m0.w), w, acc[1][b]);
+          acc[2][b] = cfma(make_float2(m1.x, m1.y), w, acc[2][b]);
+          acc[3][b] = cfma(make_float2(m1.z, m1.w), w, acc[3][b]);
+        }
+      }
+    }
+    const int site = (t0 + (g >> 2)) * L + x0 + (g & 3);
+    float2* xo = x + (size_t)(r0 + rg * NR) * n;
+#pragma unroll
+    for (int b = 0; b < NR; ++b) {
+      const int rr = rg * NR + b;
+      if ((live_mask >> rr) & 1) {
+        if (known == SAP_X) {
+          const float4 p = s.x[g * RP + rr], q = s.x[(8 + g) * RP + rr];
+          acc[0][b] = cadd(make_float2(p.x, p.y), acc[0][b]);
+          acc[1][b] = cadd(make_float2(p.z, p.w), acc[1][b]);
+          acc[2][b] = cadd(make_float2(q.x, q.y), acc[2][b]);
+          acc[3][b] = cadd(make_float2(q.z, q.w), acc[3][b]);
+        }
+        st_sp(xo + (size_t)b * n, site, acc[0][b], acc[1][b]);
+        st_sp(xo + (size_t)b * n, site + 2 * L, acc[2][b], acc[3][b]);
+      }
+    }
+    __syncthreads();  // the stage is refilled next
+  }
+}
+
+// FP64, 4 x 4 blocks: bound by the FP64 units (two FMAs a clock and SM).  The blocks of one colour do not couple, so
+// with E the hops that leave the block x_B + D_BB^{-1} (f - D x)_B = D_BB^{-1} (f - E x)_B: the hops inside the block
+// and the old x_B drop out.  One CTA of two warps per block, tiles of RG right-hand sides; a thread owns two sites
+// (4 complex rows) times RG / 8 rhs.
+template <int RG>
+__global__ void __launch_bounds__(64) k_sap_fine4_fp64(const double2* __restrict__ lk, int L,
+                                                       const double2* __restrict__ inv, const double2* __restrict__ f,
+                                                       double2* __restrict__ x, int color, int nrhs, int known,
+                                                       const int* __restrict__ active) {
+  constexpr int BD = 32, IS = BD + 1, RS = RG + 1, NR = RG / 8;
+  __shared__ double2 sinv[BD * IS];  // transposed
+  __shared__ double2 sres[BD * RS];
+  const int tid = threadIdx.x;
+  const int nbx = L / 4, half = nbx / 2;
+  const int BT = blockIdx.x / half;
+  const int BX = 2 * (blockIdx.x - BT * half) + ((BT + color) & 1);
+  const double2* I = inv + (size_t)(BT * nbx + BX) * BD * BD;
+#pragma unroll 4
+  for (int e = tid; e < BD * BD; e += 64) sinv[(e % BD) * IS + e / BD] = I[e];
+  const size_t n = 2 * (size_t)L * L;
+  const int g = tid & 7, rg = tid >> 3;  // row group and rhs group of the product
+  for (int r0 = blockIdx.y * RG; r0 < nrhs; r0 += gridDim.y * RG) {
+#pragma unroll 4
+    for (int q = tid; q < 16 * RG; q += 64) {
+      const int jx = q & 3, rr = (q >> 2) % RG, jt = (q >> 2) / RG;
+      const int rhs = r0 + rr;
+      if (rhs < nrhs && !(active && !active[rhs])) {
+        const int t = 4 * BT + jt, xx = 4 * BX + jx, s = t * L + xx;
+        const double2* X = x + rhs * n;
+        double2 o0, o1, a0, a1;
+        ld_sp(f + rhs * n, s, o0, o1);
+        if (known != SAP_ZERO && (jx == 0 || jx == 3)) {  // (1 -+ sigma_1) hop out of the block
+          const int s2 = jx == 3 ? (xx == L - 1 ? s + 1 - L : s + 1) : (xx == 0 ? s + L - 1 : s - 1);
+          ld_sp(X, s2, a0, a1);
+          const double2 w = jx == 3 ? __ldg(lk + 2 * s) : cconj(__ldg(lk + 2 * s2));
+          const double sg = jx == 3 ? -1.0 : 1.0;
+          const double2 u = cmul(w, cadd(a0, cscale(a1, sg)));
+          o0 = csub(o0, u);
+          o1 = csub(o1, cscale(u, sg));
+        }
+        if (known != SAP_ZERO && (jt == 0 || jt == 3)) {  // (1 -+ sigma_2) hop
+          const int s2 = jt == 3 ? (t == L - 1 ? xx : s + L) : (t == 0 ? s + L * (L - 1) : s - L);
+          ld_sp(X, s2, a0, a1);
+          const double2 w = jt == 3 ? __ldg(lk + 2 * s + 1) : cconj(__ldg(lk + 2 * s2 + 1));
+          const double sg = jt == 3 ? 1.0 : -1.0;
+          const double2 u = cmul(w, cadd(a0, cscale(cmuli(a1), sg)));
+          o0 = csub(o0, u);
+          o1 = cadd(o1, cscale(cmuli(u), sg));
+        }
+        const int j = 4 * jt + jx;
+        sres[(2 * j) * RS + rr] = o0;
+        sres[(2 * j + 1) * RS + rr] = o1;
+      }
+    }
+    __syncthreads();
+    double2 acc[4][NR];
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+      for (int b = 0; b < NR; ++b) acc[a][b] = make_double2(0, 0);
+#pragma unroll 4
+    for (int j = 0; j < BD; ++j) {
+      const double2* mi = sinv + j * IS;
+      const double2 m[4] = {mi[2 * g], mi[2 * g + 1], mi[16 + 2 * g], mi[17 + 2 * g]};
+      double2 v[NR];
+#pragma unroll
+      for (int b = 0; b < NR; ++b) v[b] = sres[j * RS + rg * NR + b];
+#pragma unroll
+      for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int b = 0; b < NR; ++b) acc[a][b] = cfma(m[a], v[b], acc[a][b]);
+    }
+#pragma unroll
+    for (int b = 0; b < NR; ++b) {
+      const int rhs = r0 + rg * NR + b;
+      if (rhs < nrhs && !(active && !active[rhs])) {
+        double2* X = x + rhs * n;
+        const int s = (4 * BT + (g >> 2)) * L + 4 * BX + (g & 3);
+        st_sp(X, s, acc[0][b], acc[1][b]);
+        st_sp(X, s + 2 * L, acc[2][b], acc[3][b]);
+      }
+    }
+    __syncthreads();
+  }
+}
+
+// 2 x 2 blocks (8 unknowns; mg_params.sap_block_fine = 2): one CTA per block, one thread per (row, rhs)
+template <typename R>
+__global__ void __launch_bounds__(256) k_sap_fine2(const typename CT<R>::T* __restrict__ lk, R diag, int L,
+                                                   const typename CT<R>::T* __restrict__ inv, bool inv_t,
+                                                   const typename CT<R>::T* __restrict__ f,
+                                                   typename CT<R>::T* __restrict__ x, int color, int nrhs,
+                                                   const int* __restrict__ active) {
   typedef typename CT<R>::T C;
-  constexpr int NS = BS * BS;      // sites per block
-  constexpr int BD = 2 * NS;       // dof per block
-  constexpr int G = 256 / NS;      // rhs per group (one thread per site and rhs in the residual phase)
-  __shared__ C sinv[BD * BD];      // transposed: sinv[j * BD + i] = inv[i][j] (conflict-free over i)
+  constexpr int NS = 4, BD = 8, G = 64;
+  __shared__ C sinv[BD * BD];  // sinv[j * BD + i] = inv[i][j]
   __shared__ C sres[G * BD];
-  const int nbx = L / BS;
-  const int half = nbx / 2;
-  const int k = blockIdx.x;
-  const int BT = k / half;
-  const int BX = 2 * (k % half) + ((BT + color) & 1);
-  const int blk = BT * nbx + BX;
-  const C* I = inv + (size_t)blk * BD * BD;
-  if (TRANS)  // stored transposed already: a straight, conflict-free copy
-    for (int e = threadIdx.x; e < BD * BD; e += blockDim.x) sinv[e] = I[e];
-  else
-    for (int e = threadIdx.x; e < BD * BD; e += blockDim.x) sinv[(e % BD) * BD + e / BD] = I[e];
-  const int V = L * L;
-  const size_t n = 2 * (size_t)V;
+  const int nbx = L / 2, half = nbx / 2;
+  const int BT = blockIdx.x / half;
+  const int BX = 2 * (blockIdx.x - BT * half) + ((BT + color) & 1);
+  const C* I = inv + (size_t)(BT * nbx + BX) * BD * BD;
+  for (int e = threadIdx.x; e < BD * BD; e += blockDim.x) sinv[inv_t ? e : (e % BD) * BD + e / BD] = I[e];
+  const size_t n = 2 * (size_t)L * L;
   for (int r0 = 0; r0 < nrhs; r0 += G) {
     __syncthreads();
-    // residual of the block sites
-    for (int q = threadIdx.x; q < G * NS; q += blockDim.x) {
-      const int g = q / NS, j = q % NS;
-      const int rhs = r0 + g;
+    {
+      const int q = threadIdx.x, g = q / NS, j = q % NS, rhs = r0 + g;
       if (rhs < nrhs && !(active && !active[rhs])) {
-        const int s = (BT * BS + j / BS) * L + BX * BS + (j % BS);
+        const int s = (BT * 2 + j / 2) * L + BX * 2 + (j % 2);
         C o0, o1, f0, f1;
         wilson_site<R>(lk, diag, L, x + rhs * n, s, o0, o1);
         ld_sp(f + rhs * n, s, f0, f1);
@@ -273,14 +525,12 @@ __global__ void __launch_bounds__(256) k_sap_fine(const typename CT<R>::T* __res
     }
     __syncthreads();
     for (int q = threadIdx.x; q < G * BD; q += blockDim.x) {
-      const int g = q / BD, i = q % BD;
-      const int rhs = r0 + g;
+      const int g = q / BD, i = q % BD, rhs = r0 + g;
       if (rhs < nrhs && !(active && !active[rhs])) {
         C acc = czero<C>();
-#pragma unroll 8
+#pragma unroll
         for (int j = 0; j < BD; ++j) acc = cfma(sinv[j * BD + i], sres[g * BD + j], acc);
-        const int js = i >> 1;
-        const int s = (BT * BS + js / BS) * L + BX * BS + (js % BS);
+        const int js = i >> 1, s = (BT * 2 + js / 2) * L + BX * 2 + (js % 2);
         C* px = x + rhs * n + 2 * s + (i & 1);
         *px = cadd(*px, acc);
       }
@@ -291,28 +541,57 @@ __global__ void __launch_bounds__(256) k_sap_fine(const typename CT<R>::T* __res
 template <typename R>
 void sap_half_fine(cudaStream_t st, const typename CT<R>::T* links, R diag, int L, int bs,
                    const typename CT<R>::T* inv, const typename CT<R>::T* f, typename CT<R>::T* x, int color,
-                   int nrhs, const int* active, bool inv_transposed) {
+                   int nrhs, const int* active, bool inv_transposed, int known) {
   MG_CHECK_ARG(bs == 4 || bs == 2, "fine SAP block side must be 2 or 4");
+  if (nrhs <= 0) return;
   const int nb = (L / bs) * (L / bs) / 2;
-  // per block and rhs: x, f read and x written on the block (bd complex each); inverse once per block
+  // per block and rhs: f and the surrounding x read, x written on the block (bd complex each); inverse once per block
   const double bd = 2.0 * bs * bs, cs = sizeof(typename CT<R>::T), ar = act_rhs(nrhs);
-  const double bytes = nb * (ar * 3 * bd * cs + bd * bd * cs);
-  const double flops = nb * ar * (bs * bs * 56.0 + 8.0 * bd * bd);
-  if (bs == 4 && inv_transposed)
-    MG_LAUNCH_W(bytes, flops, (k_sap_fine<R, 4, true>), nb, 256, 0, st, links, diag, L, inv, f, x, color, nrhs, active);
-  else if (bs == 4)
-    MG_LAUNCH_W(bytes, flops, (k_sap_fine<R, 4, false>), nb, 256, 0, st, links, diag, L, inv, f, x, color, nrhs,
+  const double bytes = nb * (ar * (known == SAP_ZERO ? 2 : 3) * bd * cs + bd * bd * cs);
+  const double flops = nb * ar * ((known == SAP_ZERO ? 0.0 : bs * bs * 56.0) + 8.0 * bd * bd);
+  if (bs == 2) {
+    MG_CHECK_ARG(known == SAP_X, "2 x 2 blocks read all of x");
+    MG_LAUNCH_W(bytes, flops, k_sap_fine2<R>, nb, 256, 0, st, links, diag, L, inv, inv_transposed, f, x, color, nrhs,
                 active);
-  else if (inv_transposed)
-    MG_LAUNCH_W(bytes, flops, (k_sap_fine<R, 2, true>), nb, 256, 0, st, links, diag, L, inv, f, x, color, nrhs, active);
-  else
-    MG_LAUNCH_W(bytes, flops, (k_sap_fine<R, 2, false>), nb, 256, 0, st, links, diag, L, inv, f, x, color, nrhs,
-                active);
+    return;
+  }
+  if constexpr (sizeof(R) == 4) {
+    MG_CHECK_ARG(inv_transposed, "the FP32 fine smoother reads transposed block inverses");
+    int dev = 0, nsm = 152;
+    MG_CUDA(cudaGetDevice(&dev));
+    MG_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+    // tile of right-hand sides: 8 where that takes the batch, else 16.  A tile of 32 needs fewer reads of the
+    // inverse per FMA but leaves 6 CTAs per SM instead of 10: 115 us against 100 at L = 512, 32 rhs.
+    auto go = [&](auto rg) {
+      constexpr int RG = decltype(rg)::value, sm = (int)sizeof(SapF<RG>), per_sm = std::min(16, 227 * 1024 / (sm + 1024));
+      const int ntile = (nrhs + RG - 1) / RG;
+      const dim3 grid(std::max(1, std::min(nb, (nsm * per_sm + ntile - 1) / ntile)), ntile);
+      ensure_max_smem((const void*)k_sap_fine4_fp32<RG>, sm);
+      MG_LAUNCH_W(bytes, flops, k_sap_fine4_fp32<RG>, grid, 64, sm, st, links, diag, L, inv, f, x, color, nrhs, nb,
+                  known, active);
+    };
+    if (nrhs <= 8)
+      go(std::integral_constant<int, 8>());
+    else
+      go(std::integral_constant<int, 16>());
+  } else {
+    // lattices with few blocks spread the tiles of a batch over blockIdx.y; those with many keep the inverse in
+    // shared memory across the tiles
+    auto go = [&](auto rg) {
+      constexpr int RG = decltype(rg)::value;
+      const dim3 grid(nb, nb >= 4096 ? 1 : cdiv(nrhs, RG));
+      MG_LAUNCH_W(bytes, flops, k_sap_fine4_fp64<RG>, grid, 64, 0, st, links, L, inv, f, x, color, nrhs, known, active);
+    };
+    if (nrhs <= 8)
+      go(std::integral_constant<int, 8>());
+    else
+      go(std::integral_constant<int, 16>());
+  }
 }
 template void sap_half_fine<float>(cudaStream_t, const float2*, float, int, int, const float2*, const float2*,
-                                   float2*, int, int, const int*, bool);
+                                   float2*, int, int, const int*, bool, int);
 template void sap_half_fine<double>(cudaStream_t, const double2*, double, int, int, const double2*,
-                                    const double2*, double2*, int, int, const int*, bool);
+                                    const double2*, double2*, int, int, const int*, bool, int);
 
 // out[b][j][i] = (float) in[b][i][j] for nb blocks of bd x bd
 __global__ void k_blocks_to_fp32_transposed(const double2* __restrict__ in, int nb, int bd, float2* __restrict__ out) {

@@ -1,0 +1,73 @@
+"""Kernels at the edges of their tiles (remainders of the right-hand-side and row tiles, smallest lattices), against
+the CPU oracle.  Tolerances are relative to the largest reference entry and stated from the arithmetic: FP64 kernels
+a few hundred roundings of 1.1e-16 (1e-12 where block inverses enter), FP32 ones of 6e-8."""
+import numpy as np
+import pytest
+
+from oracle import multigrid as omg
+from oracle import schwinger as osch
+from synthetic import gauge
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+
+@pytest.fixture(scope="module")
+def api():
+    import __graft_entry__ as g
+    g.build()
+    from paper_2303_11512_gb300 import api
+    return api
+
+
+@pytest.fixture(scope="module")
+def ctx(api):
+    c = api.Context()
+    yield c
+    for h, _ in _HIER.values():
+        h.close()
+    _HIER.clear()
+    c.close()
+
+
+_HIER = {}
+
+
+def hierarchy(api, ctx, L, **kw):
+    """(GPU hierarchy, oracle hierarchy) of one interacting field without bootstrap rounds."""
+    key = (L, tuple(sorted(kw.items())))
+    if key not in _HIER:
+        U = gauge.links(gauge.field(L, 3.0, 0, sweeps=60))
+        par = dict(ntv=4, setup_sweeps=2, seed=3, tensor_cores=0, pre_smooth=1, post_smooth=1)
+        par.update(kw)
+        h = api.mg_setup(ctx, torch.from_numpy(U).cuda(), L, -0.05, **par)
+        H = omg.Hierarchy(osch.dirac_sparse(U, -0.05), L, ntv=par["ntv"], setup_sweeps=2, seed=3)
+        _HIER[key] = (h, H)
+    return _HIER[key]
+
+
+def relerr(a, b):
+    return float(np.abs(np.asarray(a) - b).max() / np.abs(b).max())
+
+
+def vecs(n, k, seed, dtype):
+    rs = np.random.default_rng(seed)
+    return (rs.standard_normal((k, n)) + 1j * rs.standard_normal((k, n))).astype(dtype)
+
+
+@pytest.mark.parametrize("prec,tol", [("FP64", 1e-12), ("FP32", 2e-5)])
+@pytest.mark.parametrize("L,nrhs", [(16, 1), (16, 8), (16, 9), (16, 17), (32, 33)])
+def test_fine_smoother_and_cycle_tiles(api, ctx, L, nrhs, prec, tol):
+    """Fine SAP sweeps from a given x and, through the V-cycle, from zero: rhs tiles of 8 and 16 and their remainders
+    (one 4 x 4 block solve amplifies roundings by its condition, about 10, over at most 4 half sweeps)."""
+    h, H = hierarchy(api, ctx, L)
+    dt = np.complex128 if prec == "FP64" else np.complex64
+    f, x = vecs(H.n[0], nrhs, 1, dt), vecs(H.n[0], nrhs, 2, dt)
+    ref = H.sap(0).sweep(f.T.astype(complex), x.T.astype(complex)).T
+    xd = torch.from_numpy(x).cuda()
+    h.smooth(0, torch.from_numpy(f).cuda(), xd, getattr(api, prec), 1)
+    assert relerr(xd.cpu().numpy(), ref) < tol
+    xd.fill_(float("nan"))  # the cycle starts from zero whatever the output buffer holds
+    h.vcycle(0, torch.from_numpy(f).cuda(), xd, getattr(api, prec))
+    assert relerr(xd.cpu().numpy(), H.vcycle(0, f.T, 1, 1).T) < 10 * tol
