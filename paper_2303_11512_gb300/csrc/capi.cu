@@ -47,12 +47,16 @@ int mgmlmc_ctx_create(void* stream, mgmlmc_ctx** out) {
   if (!c) return MGMLMC_ERR_OOM;
   c->stream = (cudaStream_t)stream;
   if (cudaGetDevice(&c->device) != cudaSuccess ||
-      cudaMallocHost((void**)&c->pinned, 64) != cudaSuccess) {
+      cudaMallocHost((void**)&c->pinned, 64 * sizeof(int) + 64) != cudaSuccess ||
+      cudaEventCreateWithFlags(&c->flag_event[0], cudaEventDisableTiming) != cudaSuccess ||
+      cudaEventCreateWithFlags(&c->flag_event[1], cudaEventDisableTiming) != cudaSuccess) {
     cudaGetLastError();
+    if (c->flag_event[0]) cudaEventDestroy(c->flag_event[0]);
+    if (c->pinned) cudaFreeHost(c->pinned);
     delete c;
     return MGMLMC_ERR_CUDA;
   }
-  c->pinned_d = reinterpret_cast<double*>(c->pinned + 8);
+  c->pinned_d = reinterpret_cast<double*>(c->pinned + 64);
   *out = c;
   return MGMLMC_OK;
 }
@@ -61,6 +65,7 @@ void mgmlmc_ctx_destroy(mgmlmc_ctx* ctx) {
   if (!ctx) return;
   cudaStreamSynchronize(ctx->stream);
   if (ctx->pinned) cudaFreeHost(ctx->pinned);
+  for (cudaEvent_t e : ctx->flag_event) cudaEventDestroy(e);
   delete ctx;
 }
 

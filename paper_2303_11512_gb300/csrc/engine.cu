@@ -184,71 +184,6 @@ __global__ void k_gm_cycle(const double* __restrict__ beta2, int* act, int* cact
   atomicAdd(count, 1);
 }
 
-__global__ void k_gm_arnoldi(int j, int m, int nrhs, const double2* __restrict__ h1, const double2* __restrict__ h2,
-                             const double* __restrict__ hn2, double* hn, double2* H, double* cs, double2* sn,
-                             double2* g, int* iact, int* kvec, int* its, const double* __restrict__ bnorm,
-                             double tol, int maxit, int* count) {
-  const int r = blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= nrhs || !iact[r]) return;
-  double2 col[65];
-  for (int i = 0; i <= j; ++i) col[i] = cadd(h1[(size_t)i * nrhs + r], h2[(size_t)i * nrhs + r]);
-  const double hh = sqrt(hn2[r]);
-  col[j + 1] = make_double2(hh, 0);
-  for (int i = 0; i < j; ++i) {
-    const double c = cs[(size_t)i * nrhs + r];
-    const double2 s = sn[(size_t)i * nrhs + r];
-    const double2 a = col[i], b = col[i + 1];
-    col[i] = cadd(cscale(a, c), cmul(s, b));
-    col[i + 1] = csub(cscale(b, c), cmulc(s, a));
-  }
-  // new rotation zeroing col[j+1]
-  const double2 a = col[j], b = col[j + 1];
-  const double na = sqrt(a.x * a.x + a.y * a.y), nb = sqrt(b.x * b.x + b.y * b.y);
-  double c;
-  double2 s, rr;
-  if (na == 0.0) {
-    c = 0.0; s = make_double2(1, 0); rr = b;
-  } else {
-    const double t = sqrt(na * na + nb * nb);
-    const double2 ph = make_double2(a.x / na, a.y / na);
-    c = na / t;
-    s = cscale(cmul(ph, cconj(b)), 1.0 / t);
-    rr = cscale(ph, t);
-  }
-  cs[(size_t)j * nrhs + r] = c;
-  sn[(size_t)j * nrhs + r] = s;
-  col[j] = rr;
-  for (int i = 0; i <= j; ++i) H[((size_t)i * m + j) * nrhs + r] = col[i];
-  const double2 gj = g[(size_t)j * nrhs + r];
-  g[(size_t)(j + 1) * nrhs + r] = cneg(cmulc(s, gj));
-  g[(size_t)j * nrhs + r] = cscale(gj, c);
-  const double2 gn = g[(size_t)(j + 1) * nrhs + r];
-  const double res = sqrt(gn.x * gn.x + gn.y * gn.y);
-  its[r] += 1;
-  kvec[r] = j + 1;
-  hn[r] = hh;
-  if (res <= tol * bnorm[r] || its[r] >= maxit || hh == 0.0 || j + 1 == m || !(res == res)) {
-    iact[r] = 0;
-  } else {
-    atomicAdd(count, 1);
-  }
-}
-
-__global__ void k_gm_trisolve(int m, int nrhs, const double2* __restrict__ H, const double2* __restrict__ g,
-                              const int* __restrict__ kvec, const int* __restrict__ cact, double2* y) {
-  const int r = blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= nrhs) return;
-  const int k = cact[r] ? kvec[r] : 0;
-  for (int i = m - 1; i >= 0; --i) {
-    if (i >= k) { y[(size_t)i * nrhs + r] = make_double2(0, 0); continue; }
-    double2 s = g[(size_t)i * nrhs + r];
-    for (int q = i + 1; q < k; ++q) s = csub(s, cmul(H[((size_t)i * m + q) * nrhs + r], y[(size_t)q * nrhs + r]));
-    const double2 d = H[((size_t)i * m + i) * nrhs + r];
-    const double dn = d.x * d.x + d.y * d.y;
-    y[(size_t)i * nrhs + r] = dn > 0 ? cscale(cmulc(d, s), 1.0 / dn) : make_double2(0, 0);
-  }
-}
-
 // The V-cycle as a CUDA graph: a fixed launch sequence for a given (level, precision, nrhs, mask), captured
 // once on fixed input/output buffers after an eager warm-up pass has allocated every workspace it touches,
 // then replayed between two vector copies.  Not used while the per-kernel timer runs or with K-cycles
@@ -326,8 +261,9 @@ struct GmState {
   typedef typename CT<R>::T C;
   C *V, *Z;
   int *act, *cact, *iact, *kvec, *its, *count;
-  double *bnorm, *beta, *beta2, *hn, *hn2, *cs, *relres;
+  double *bnorm, *beta, *beta2, *hn, *wn2, *cs, *relres;
   double2 *g, *H, *sn, *h1, *h2, *y;
+  KryGm gm;
   void* red;
 };
 
@@ -340,12 +276,12 @@ static GmState<R> gm_state(mgmlmc_hier* h, int l, int nrhs, int m) {
   char* b = (char*)h->work(std::string(tg) + "_V", l, sizeof(C) * n * nrhs * (m + 1));
   s.V = (C*)b;
   s.Z = (C*)h->work(std::string(tg) + "_Z", l, sizeof(C) * n * nrhs * m);
-  size_t ints = (size_t)nrhs * 6 + 8;
+  size_t ints = (size_t)nrhs * 6 + m + 1;  // count: one per step, then one for the start of a cycle
   int* ip = (int*)h->work(std::string(tg) + "_i", l, sizeof(int) * ints);
   s.act = ip; s.cact = ip + nrhs; s.iact = ip + 2 * nrhs; s.kvec = ip + 3 * nrhs; s.its = ip + 4 * nrhs;
   s.count = ip + 6 * nrhs;
   double* dp = (double*)h->work(std::string(tg) + "_d", l, sizeof(double) * (size_t)nrhs * (7 + m));
-  s.bnorm = dp; s.beta = dp + nrhs; s.beta2 = dp + 2 * nrhs; s.hn = dp + 3 * nrhs; s.hn2 = dp + 4 * nrhs;
+  s.bnorm = dp; s.beta = dp + nrhs; s.beta2 = dp + 2 * nrhs; s.hn = dp + 3 * nrhs; s.wn2 = dp + 4 * nrhs;
   s.relres = dp + 5 * nrhs; s.cs = dp + 7 * nrhs;
   double2* cp = (double2*)h->work(std::string(tg) + "_c", l,
                                   sizeof(double2) * (size_t)nrhs * ((m + 1) + (size_t)(m + 1) * m + m + 2 * (m + 1) + m));
@@ -355,7 +291,9 @@ static GmState<R> gm_state(mgmlmc_hier* h, int l, int nrhs, int m) {
   s.h1 = cp; cp += (size_t)(m + 1) * nrhs;
   s.h2 = cp; cp += (size_t)(m + 1) * nrhs;
   s.y = cp;
-  s.red = h->work(std::string(tg) + "_r", l, reduce_work_bytes(n, nrhs, m + 1));
+  s.red = h->work(std::string(tg) + "_r", l, std::max(reduce_work_bytes(n, nrhs, m + 1), kry_work_bytes(nrhs, m)));
+  kry_work_init(h->ctx->stream, s.red, nrhs, m);
+  s.gm = KryGm{nrhs, m, 0, 0.0, s.h1, s.h2, s.H, s.g, s.sn, s.cs, s.hn, s.wn2, s.bnorm, s.iact, s.kvec, s.its, s.count};
   return s;
 }
 
@@ -376,6 +314,10 @@ void fgmres_core(mgmlmc_hier* h, int l, const typename CT<R>::T* b, typename CT<
   const long n = h->lv[l].n;
   MG_CHECK_ARG(m >= 1 && m <= 64, "FGMRES restart length must be 1..64");
   GmState<R> s = gm_state<R>(h, l, nrhs, m);
+  s.gm.tol = tol;
+  s.gm.maxit = maxit;
+  const C* Z = precond ? s.Z : s.V;  // without a preconditioner z_j = v_j
+  int* const started = s.count + m;
   const long vs = n * nrhs;
   const unsigned nb = cdiv(nrhs, 64);
   vnorm2<C>(st, b, n, nrhs, s.beta2, s.red, act_in);
@@ -388,10 +330,10 @@ void fgmres_core(mgmlmc_hier* h, int l, const typename CT<R>::T* b, typename CT<
     else
       op_apply<R>(h, l, x, s.V, b, nrhs, s.act);  // V0 = b - D x
     vnorm2<C>(st, s.V, n, nrhs, s.beta2, s.red, s.act);
-    MG_CUDA(cudaMemsetAsync(s.count, 0, sizeof(int), st));
+    MG_CUDA(cudaMemsetAsync(s.count, 0, sizeof(int) * (m + 1), st));
     MG_LAUNCH(k_gm_cycle, nb, 64, 0, st, s.beta2, s.act, s.cact, s.iact, s.kvec, s.beta, s.g, s.bnorm, s.its,
-              s.relres, tol, maxit, m, nrhs, s.count);
-    const int nstart = read_flag(ctx, s.count);
+              s.relres, tol, maxit, m, nrhs, started);
+    const int nstart = read_flag(ctx, started);
     if (nstart == 0) break;
     g_nact_hint = nstart;
     vscale_inv<C>(st, s.beta, s.V, s.V, n, nrhs, s.cact);
@@ -399,9 +341,8 @@ void fgmres_core(mgmlmc_hier* h, int l, const typename CT<R>::T* b, typename CT<
     for (int j = 0; j < m; ++j) {
       C* Vj = s.V + (size_t)j * vs;
       C* Vj1 = s.V + (size_t)(j + 1) * vs;
-      C* Zj = s.Z + (size_t)j * vs;
-      if (precond)
-      {
+      C* Zj = const_cast<C*>(Z) + (size_t)j * vs;
+      if (precond) {
         vcycle_maybe_graph<R>(h, l, Vj, Zj, nrhs, s.iact);
         if constexpr (sizeof(R) == 4) {
           if (precond == 2 && l == 0 && h->nn) {  // learned correction: z += |t| M(t / |t|), t = v - D z
@@ -422,25 +363,27 @@ void fgmres_core(mgmlmc_hier* h, int l, const typename CT<R>::T* b, typename CT<
             nn_add(st, Zj, cc, n, nrhs, tn);
           }
         }
+      } else if (j >= 2) {
+        // a step is short here, so the host looks at the count of two steps ago; the steps issued meanwhile skip
+        // every right-hand side that has stopped
+        MG_CUDA(cudaEventSynchronize(ctx->flag_event[j & 1]));
+        if (ctx->pinned[j - 2] == 0) break;
       }
-      else
-        vcopy<C>(st, Vj, Zj, n, nrhs);
       op_apply<R>(h, l, Zj, Vj1, nullptr, nrhs, s.iact);
-      vmultidot<C>(st, s.V, vs, j + 1, Vj1, n, nrhs, s.h1, s.red, s.iact);
-      vgs_update_dot<C>(st, s.V, vs, j + 1, s.h1, Vj1, n, nrhs, s.h2, s.red, s.iact);
-      vgs_update_norm<C>(st, s.V, vs, j + 1, s.h2, Vj1, n, nrhs, s.hn2, s.red, s.iact);
-      MG_CUDA(cudaMemsetAsync(s.count, 0, sizeof(int), st));
-      MG_LAUNCH(k_gm_arnoldi, nb, 64, 0, st, j, m, nrhs, s.h1, s.h2, s.hn2, s.hn, s.H, s.cs, s.sn, s.g, s.iact,
-                s.kvec, s.its, s.bnorm, tol, maxit, s.count);
+      kry_step<C>(st, s.V, vs, j + 1, Vj1, n, s.gm, s.red);
       jdone = j + 1;
-      vscale_inv<C>(st, s.hn, Vj1, Vj1, n, nrhs, s.iact);
-      const int nit = read_flag(ctx, s.count);
+      if (!precond) {
+        MG_CUDA(cudaMemcpyAsync(ctx->pinned + j, s.count + j, sizeof(int), cudaMemcpyDeviceToHost, st));
+        MG_CUDA(cudaEventRecord(ctx->flag_event[j & 1], st));
+        continue;
+      }
+      const int nit = read_flag(ctx, s.count + j);
       if (nit == 0) break;
       g_nact_hint = nit;
     }
     g_nact_hint = nstart;
-    MG_LAUNCH(k_gm_trisolve, nb, 64, 0, st, m, nrhs, s.H, s.g, s.kvec, s.cact, s.y);
-    vcombine<C>(st, s.Z, vs, jdone, s.y, x, n, nrhs, s.cact);
+    kry_trisolve(st, s.gm, s.cact, s.y);
+    vcombine<C>(st, Z, vs, jdone, s.y, x, n, nrhs, s.cact);
     g_nact_hint = -1;
   }
   g_nact_hint = -1;

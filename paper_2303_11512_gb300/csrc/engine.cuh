@@ -16,7 +16,8 @@ struct mgmlmc_ctx {
   int device = 0;
   std::string err;
   int64_t launches = 0;
-  int* pinned = nullptr;  // small pinned host buffer for flags
+  int* pinned = nullptr;  // small pinned host buffer for flags (64 ints, then pinned_d)
+  cudaEvent_t flag_event[2] = {nullptr, nullptr};  // behind the two flags last copied to pinned
   double* pinned_d = nullptr;
   mg::KTimer timer;
   std::map<std::string, mg::DBuf> ws;  // workspaces of calls that have no hierarchy (projection)

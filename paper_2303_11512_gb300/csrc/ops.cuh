@@ -115,14 +115,24 @@ void vmultidot(cudaStream_t st, const C* V, long vstride, int k, const C* w, lon
 template <typename C>
 void vgs_update(cudaStream_t st, const C* V, long vstride, int k, const double2* h, C* w, long n, int nrhs,
                 const int* active);
-// the two classical Gram-Schmidt passes, each update fused with the reduction that follows it:
-// w -= sum_i h[i][rhs] V_i, then h2[i][rhs] = V_i^H w   /   w -= sum_i h[i][rhs] V_i, then out[rhs] = ||w||^2
+// Orthogonalisation step of FGMRES (ops_krylov.cu): w against V_0 .. V_{k-1} (classical Gram-Schmidt twice), column
+// k - 1 of the Hessenberg matrix with its Givens update and per-rhs stop, w <- the next basis vector.  Arrays
+// [i][rhs] over nrhs; right-hand sides with iact = 0 are skipped; count[k - 1] (zeroed by the caller) receives the
+// number of those that go on.
+struct KryGm {
+  int nrhs, m, maxit;
+  double tol;
+  double2 *h1, *h2, *H, *g, *sn;
+  double *cs, *hn, *wn2;
+  const double* bnorm;
+  int *iact, *kvec, *its, *count;
+};
+size_t kry_work_bytes(int nrhs, int m);
+void kry_work_init(cudaStream_t st, void* work, int nrhs, int m);  // once before the first step on `work`
 template <typename C>
-void vgs_update_dot(cudaStream_t st, const C* V, long vstride, int k, const double2* h, C* w, long n, int nrhs,
-                    double2* h2, void* work, const int* active);
-template <typename C>
-void vgs_update_norm(cudaStream_t st, const C* V, long vstride, int k, const double2* h, C* w, long n, int nrhs,
-                     double* out, void* work, const int* active);
+void kry_step(cudaStream_t st, const C* V, long vstride, int k, C* w, long n, const KryGm& gm, void* work);
+// y[i][rhs] = (R^{-1} g)_i for the kvec[rhs] x kvec[rhs] triangle R of every rhs with cact != 0, zero elsewhere
+void kry_trisolve(cudaStream_t st, const KryGm& gm, const int* cact, double2* y);
 // x += sum_i y[i][rhs] Z_i
 template <typename C>
 void vcombine(cudaStream_t st, const C* Z, long zstride, int k, const double2* y, C* x, long n, int nrhs,

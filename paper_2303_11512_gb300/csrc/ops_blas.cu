@@ -2,13 +2,18 @@
 // deterministic two-stage reductions used by the Krylov solver (warp-shuffle
 // trees, fixed partition, so repeated runs give identical bits), and the
 // counter-based Rademacher generator.
+#include <algorithm>
+
 #include "ops.cuh"
 
 namespace mg {
 
 namespace {
 constexpr int RT = 256;   // threads per reduction block
-constexpr int RBLK = 64;  // reduction blocks per rhs
+constexpr int RBLK = 64;  // reduction blocks per rhs at most
+// blocks per rhs for vectors of n entries: at least two entries a thread (with 64 blocks for every n a vector of 512
+// entries left 62 of them to reduce zeros: 75 us for 16 dot products of 32 rhs)
+inline int red_blocks(long n) { return (int)std::max<long>(1, std::min<long>(RBLK, n / (2 * RT))); }
 
 template <typename T> __device__ __forceinline__ T warp_sum(T v) {
 #pragma unroll
@@ -48,24 +53,25 @@ __global__ void __launch_bounds__(RT) k_norm2_part(const C* __restrict__ x, long
   __shared__ double sh[32];
   const int rhs = blockIdx.y;
   if (active && !active[rhs]) {
-    if (threadIdx.x == 0) part[(size_t)rhs * RBLK + blockIdx.x] = 0.0;
+    if (threadIdx.x == 0) part[(size_t)rhs * gridDim.x + blockIdx.x] = 0.0;
     return;
   }
   const C* X = x + (size_t)rhs * n;
   R acc = 0;
-  for (long i = blockIdx.x * (long)RT + threadIdx.x; i < n; i += (long)RBLK * RT) {
+  for (long i = blockIdx.x * (long)RT + threadIdx.x; i < n; i += (long)gridDim.x * RT) {
     C v = X[i];
     acc += v.x * v.x + v.y * v.y;
   }
   double r = block_sum((double)acc, sh);
-  if (threadIdx.x == 0) part[(size_t)rhs * RBLK + blockIdx.x] = r;
+  if (threadIdx.x == 0) part[(size_t)rhs * gridDim.x + blockIdx.x] = r;
 }
 
-__global__ void k_finalize_real(const double* __restrict__ part, int nrhs, double* __restrict__ out) {
+__global__ void k_finalize_real(const double* __restrict__ part, int nblk, int nrhs, double* __restrict__ out) {
   const int rhs = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
   const int l = threadIdx.x & 31;
   if (rhs >= nrhs) return;
-  double v = part[(size_t)rhs * RBLK + l] + part[(size_t)rhs * RBLK + l + 32];
+  double v = 0;
+  for (int b = l; b < nblk; b += 32) v += part[(size_t)rhs * nblk + b];
   v = warp_sum(v);
   if (l == 0) out[rhs] = v;
 }
@@ -73,9 +79,9 @@ __global__ void k_finalize_real(const double* __restrict__ part, int nrhs, doubl
 template <typename C>
 void vnorm2(cudaStream_t st, const C* x, long n, int nrhs, double* out, void* work, const int* active) {
   double* part = reinterpret_cast<double*>(work);
-  MG_LAUNCH_W(act_rhs(nrhs) * n * sizeof(C), act_rhs(nrhs) * n * 4.0, k_norm2_part<C>, dim3(RBLK, nrhs), RT, 0, st,
-              x, n, part, active);
-  MG_LAUNCH(k_finalize_real, cdiv(nrhs, 4), 128, 0, st, part, nrhs, out);
+  MG_LAUNCH_W(act_rhs(nrhs) * n * sizeof(C), act_rhs(nrhs) * n * 4.0, k_norm2_part<C>, dim3(red_blocks(n), nrhs), RT,
+              0, st, x, n, part, active);
+  MG_LAUNCH(k_finalize_real, cdiv(nrhs, 4), 128, 0, st, part, red_blocks(n), nrhs, out);
 }
 template void vnorm2<float2>(cudaStream_t, const float2*, long, int, double*, void*, const int*);
 template void vnorm2<double2>(cudaStream_t, const double2*, long, int, double*, void*, const int*);
@@ -129,7 +135,7 @@ __device__ __forceinline__ double block_sum_many(double (&v)[NV], double* sh) {
 
 // part[(i * nrhs + rhs) * RBLK + block] (component c) = t, for dot i, real (c = 0) / imaginary (c = 1)
 __device__ __forceinline__ void store_part(double2* part, int i, int nrhs, int rhs, int c, double t) {
-  reinterpret_cast<double*>(part + ((size_t)i * nrhs + rhs) * RBLK + blockIdx.x)[c] = t;
+  reinterpret_cast<double*>(part + ((size_t)i * nrhs + rhs) * gridDim.x + blockIdx.x)[c] = t;
 }
 
 template <typename C, int MDC>
@@ -149,7 +155,7 @@ __global__ void __launch_bounds__(RT) k_multidot_part(const C* __restrict__ V, l
     for (int q = 0; q < MDC; ++q) { ar[q] = 0; ai[q] = 0; }
     const int cnt = min(MDC, k - i0);
     if (on) {
-      for (long e = blockIdx.x * (long)RT + threadIdx.x; e < n; e += (long)RBLK * RT) {
+      for (long e = blockIdx.x * (long)RT + threadIdx.x; e < n; e += (long)gridDim.x * RT) {
         const C b = W[e];
 #pragma unroll
         for (int q = 0; q < MDC; ++q) {
@@ -169,12 +175,18 @@ __global__ void __launch_bounds__(RT) k_multidot_part(const C* __restrict__ V, l
   }
 }
 
-__global__ void k_finalize_cplx(const double2* __restrict__ part, int count, double2* __restrict__ out) {
+__global__ void k_finalize_cplx(const double2* __restrict__ part, int nblk, int count, double2* __restrict__ out) {
   const int idx = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
   const int l = threadIdx.x & 31;
   if (idx >= count) return;
-  double2 a = part[(size_t)idx * RBLK + l], b = part[(size_t)idx * RBLK + l + 32];
-  double re = warp_sum(a.x + b.x), im = warp_sum(a.y + b.y);
+  double re = 0, im = 0;
+  for (int b = l; b < nblk; b += 32) {
+    const double2 v = part[(size_t)idx * nblk + b];
+    re += v.x;
+    im += v.y;
+  }
+  re = warp_sum(re);
+  im = warp_sum(im);
   if (l == 0) out[idx] = make_double2(re, im);
 }
 
@@ -185,12 +197,12 @@ void vmultidot(cudaStream_t st, const C* V, long vstride, int k, const C* w, lon
   // chunk of dot products per pass: 8 when that covers k (fewer registers, more resident blocks)
   const double bytes = act_rhs(nrhs) * n * sizeof(C) * (k + 1.0), flops = act_rhs(nrhs) * n * 8.0 * k;
   if (k <= 8)
-    MG_LAUNCH_W(bytes, flops, (k_multidot_part<C, 8>), dim3(RBLK, nrhs), RT, 0, st, V, vstride, k, w, n, part,
+    MG_LAUNCH_W(bytes, flops, (k_multidot_part<C, 8>), dim3(red_blocks(n), nrhs), RT, 0, st, V, vstride, k, w, n, part,
                 active);
   else
-    MG_LAUNCH_W(bytes, flops, (k_multidot_part<C, MdChunk<C>::value>), dim3(RBLK, nrhs), RT, 0, st, V, vstride, k,
+    MG_LAUNCH_W(bytes, flops, (k_multidot_part<C, MdChunk<C>::value>), dim3(red_blocks(n), nrhs), RT, 0, st, V, vstride, k,
                 w, n, part, active);
-  MG_LAUNCH(k_finalize_cplx, cdiv((long)k * nrhs, 4), 128, 0, st, part, k * nrhs, h);
+  MG_LAUNCH(k_finalize_cplx, cdiv((long)k * nrhs, 4), 128, 0, st, part, red_blocks(n), k * nrhs, h);
 }
 template void vmultidot<float2>(cudaStream_t, const float2*, long, int, const float2*, long, int, double2*, void*,
                                 const int*);
@@ -251,137 +263,6 @@ template void vgs_update<double2>(cudaStream_t, const double2*, long, int, const
 template void vcombine<float2>(cudaStream_t, const float2*, long, int, const double2*, float2*, long, int, const int*);
 template void vcombine<double2>(cudaStream_t, const double2*, long, int, const double2*, double2*, long, int,
                                 const int*);
-
-// ---- fused classical Gram-Schmidt passes ------------------------------------------------------
-// First-pass update fused with the second pass's dot products: w -= sum_i h_i V_i, then
-// V_i^H w with the updated w; each thread keeps its V_i elements in registers between the two.
-template <typename C, int KM>
-__global__ void __launch_bounds__(RT, sizeof(C) == 8 ? 2 : 1) k_gs_update_dot(const C* __restrict__ V, long vstride, int k,
-                                                      const double2* __restrict__ h, C* __restrict__ w, long n,
-                                                      double2* __restrict__ part, const int* __restrict__ active) {
-  typedef typename Acc<C>::R R;
-  __shared__ C hs[KM];
-  __shared__ double sh[(RT / 32) * 2 * KM];
-  const int rhs = blockIdx.y, nrhs = gridDim.y;
-  const bool on = !(active && !active[rhs]);
-  if ((int)threadIdx.x < k) {
-    const double2 v = h[(size_t)threadIdx.x * nrhs + rhs];
-    hs[threadIdx.x] = cmake((R)v.x, (R)v.y);
-  }
-  __syncthreads();
-  R dr[KM], di[KM];
-#pragma unroll
-  for (int q = 0; q < KM; ++q) { dr[q] = 0; di[q] = 0; }
-  if (on) {
-    C* W = w + (size_t)rhs * n;
-    const C* Vr = V + (size_t)rhs * n;
-    for (long e = blockIdx.x * (long)RT + threadIdx.x; e < n; e += (long)RBLK * RT) {
-      C a[KM];
-      C acc = czero<C>();
-#pragma unroll
-      for (int q = 0; q < KM; ++q) {
-        if (q < k) {
-          a[q] = Vr[(size_t)q * vstride + e];
-          acc = cfma(hs[q], a[q], acc);
-        }
-      }
-      const C x = csub(W[e], acc);
-      W[e] = x;
-#pragma unroll
-      for (int q = 0; q < KM; ++q) {
-        if (q < k) {
-          dr[q] = fma(a[q].x, x.x, fma(a[q].y, x.y, dr[q]));
-          di[q] = fma(a[q].x, x.y, fma(-a[q].y, x.x, di[q]));
-        }
-      }
-    }
-  }
-  double v[2 * KM];
-#pragma unroll
-  for (int q = 0; q < KM; ++q) { v[2 * q] = dr[q]; v[2 * q + 1] = di[q]; }
-  const double t = block_sum_many<2 * KM>(v, sh);
-  if ((int)threadIdx.x < 2 * k) store_part(part, threadIdx.x >> 1, nrhs, rhs, threadIdx.x & 1, t);
-}
-
-// Second-pass update fused with the norm of the result: w -= sum_i h_i V_i, part = ||w||^2.
-template <typename C, int KM>
-__global__ void __launch_bounds__(RT) k_gs_update_norm(const C* __restrict__ V, long vstride, int k,
-                                                       const double2* __restrict__ h, C* __restrict__ w, long n,
-                                                       double* __restrict__ part, const int* __restrict__ active) {
-  typedef typename Acc<C>::R R;
-  __shared__ C hs[KM];
-  __shared__ double sh[32];
-  const int rhs = blockIdx.y, nrhs = gridDim.y;
-  if (active && !active[rhs]) {
-    if (threadIdx.x == 0) part[(size_t)rhs * RBLK + blockIdx.x] = 0.0;
-    return;
-  }
-  if ((int)threadIdx.x < k) {
-    const double2 v = h[(size_t)threadIdx.x * nrhs + rhs];
-    hs[threadIdx.x] = cmake((R)v.x, (R)v.y);
-  }
-  __syncthreads();
-  C* W = w + (size_t)rhs * n;
-  const C* Vr = V + (size_t)rhs * n;
-  R s = 0;
-  for (long e = blockIdx.x * (long)RT + threadIdx.x; e < n; e += (long)RBLK * RT) {
-    C acc = czero<C>();
-#pragma unroll
-    for (int q = 0; q < KM; ++q)
-      if (q < k) acc = cfma(hs[q], Vr[(size_t)q * vstride + e], acc);
-    const C x = csub(W[e], acc);
-    W[e] = x;
-    s += x.x * x.x + x.y * x.y;
-  }
-  const double r = block_sum((double)s, sh);
-  if (threadIdx.x == 0) part[(size_t)rhs * RBLK + blockIdx.x] = r;
-}
-
-template <typename C>
-void vgs_update_dot(cudaStream_t st, const C* V, long vstride, int k, const double2* h, C* w, long n, int nrhs,
-                    double2* h2, void* work, const int* active) {
-  if (k > 16) {
-    vgs_update<C>(st, V, vstride, k, h, w, n, nrhs, active);
-    vmultidot<C>(st, V, vstride, k, w, n, nrhs, h2, work, active);
-    return;
-  }
-  double2* part = reinterpret_cast<double2*>(work);
-  const double bytes = act_rhs(nrhs) * n * sizeof(C) * (k + 2.0), flops = act_rhs(nrhs) * n * 16.0 * k;
-  if (k <= 8)
-    MG_LAUNCH_W(bytes, flops, (k_gs_update_dot<C, 8>), dim3(RBLK, nrhs), RT, 0, st, V, vstride, k, h, w, n, part,
-                active);
-  else
-    MG_LAUNCH_W(bytes, flops, (k_gs_update_dot<C, 16>), dim3(RBLK, nrhs), RT, 0, st, V, vstride, k, h, w, n, part,
-                active);
-  MG_LAUNCH(k_finalize_cplx, cdiv((long)k * nrhs, 4), 128, 0, st, part, k * nrhs, h2);
-}
-
-template <typename C>
-void vgs_update_norm(cudaStream_t st, const C* V, long vstride, int k, const double2* h, C* w, long n, int nrhs,
-                     double* out, void* work, const int* active) {
-  if (k > 16) {
-    vgs_update<C>(st, V, vstride, k, h, w, n, nrhs, active);
-    vnorm2<C>(st, w, n, nrhs, out, work, active);
-    return;
-  }
-  double* part = reinterpret_cast<double*>(work);
-  const double bytes = act_rhs(nrhs) * n * sizeof(C) * (k + 2.0), flops = act_rhs(nrhs) * n * (8.0 * k + 4.0);
-  if (k <= 8)
-    MG_LAUNCH_W(bytes, flops, (k_gs_update_norm<C, 8>), dim3(RBLK, nrhs), RT, 0, st, V, vstride, k, h, w, n, part,
-                active);
-  else
-    MG_LAUNCH_W(bytes, flops, (k_gs_update_norm<C, 16>), dim3(RBLK, nrhs), RT, 0, st, V, vstride, k, h, w, n, part,
-                active);
-  MG_LAUNCH(k_finalize_real, cdiv(nrhs, 4), 128, 0, st, part, nrhs, out);
-}
-template void vgs_update_dot<float2>(cudaStream_t, const float2*, long, int, const double2*, float2*, long, int,
-                                     double2*, void*, const int*);
-template void vgs_update_dot<double2>(cudaStream_t, const double2*, long, int, const double2*, double2*, long, int,
-                                      double2*, void*, const int*);
-template void vgs_update_norm<float2>(cudaStream_t, const float2*, long, int, const double2*, float2*, long, int,
-                                      double*, void*, const int*);
-template void vgs_update_norm<double2>(cudaStream_t, const double2*, long, int, const double2*, double2*, long, int,
-                                       double*, void*, const int*);
 
 // ---- elementwise -------------------------------------------------------------------------------
 template <typename C> void vzero(cudaStream_t st, C* x, long n, int nrhs) {

@@ -148,7 +148,9 @@ void wilson_apply(cudaStream_t st, const typename CT<R>::T* links, R diag, int L
                   typename CT<R>::T* y, const typename CT<R>::T* b, int nrhs, const int* active) {
   if (nrhs <= 0) return;
   const int rpt = sizeof(R) == 4 ? tune_lookup(TUNE_WILSON32, L, nrhs, 0, 1) : 1;
-  dim3 grid(cdiv((long)L * L, 256), cdiv(nrhs, rpt));
+  // blocks of 64 threads where 256 would leave most SMs without one (FP64: two FMAs a clock and SM bound it)
+  const int bt = (long)L * L * cdiv(nrhs, rpt) >= 152L * 256 * 2 ? 256 : 64;
+  dim3 grid(cdiv((long)L * L, bt), cdiv(nrhs, rpt));
   // algorithmic traffic: x read + y written once per site and rhs (+ b), links once per launch
   const double V = (double)L * L, sp = 2.0 * sizeof(typename CT<R>::T), ar = act_rhs(nrhs);
   const double bytes = ar * V * sp * (b ? 3 : 2) + V * sp;
@@ -156,9 +158,9 @@ void wilson_apply(cudaStream_t st, const typename CT<R>::T* links, R diag, int L
 #define MG_WILSON_LAUNCH(RPT_)                                                                                  \
   do {                                                                                                          \
     if (b)                                                                                                      \
-      MG_LAUNCH_W(bytes, flops, (k_wilson<R, true, RPT_>), grid, 256, 0, st, links, diag, L, x, y, b, active, nrhs); \
+      MG_LAUNCH_W(bytes, flops, (k_wilson<R, true, RPT_>), grid, bt, 0, st, links, diag, L, x, y, b, active, nrhs); \
     else                                                                                                        \
-      MG_LAUNCH_W(bytes, flops, (k_wilson<R, false, RPT_>), grid, 256, 0, st, links, diag, L, x, y, b, active, nrhs); \
+      MG_LAUNCH_W(bytes, flops, (k_wilson<R, false, RPT_>), grid, bt, 0, st, links, diag, L, x, y, b, active, nrhs); \
   } while (0)
   if (rpt == 4)
     MG_WILSON_LAUNCH(4);

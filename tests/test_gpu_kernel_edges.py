@@ -71,3 +71,29 @@ def test_fine_smoother_and_cycle_tiles(api, ctx, L, nrhs, prec, tol):
     xd.fill_(float("nan"))  # the cycle starts from zero whatever the output buffer holds
     h.vcycle(0, torch.from_numpy(f).cuda(), xd, getattr(api, prec))
     assert relerr(xd.cpu().numpy(), H.vcycle(0, f.T, 1, 1).T) < 10 * tol
+
+
+@pytest.mark.parametrize("L,nrhs,m", [(16, 1, 1), (16, 5, 30), (32, 33, 40), (64, 3, 16), (80, 2, 24), (128, 2, 20)])
+@pytest.mark.parametrize("prec", ["FP64", "FP32"])
+def test_krylov_step_forms(api, ctx, L, nrhs, m, prec):
+    """GMRES without preconditioner in the one-launch form (up to 16384 entries: 512, 2048, 8192, 12800) and the
+    three-pass form (32768), past 16 basis vectors, at restart lengths 1 and 40: the true residual, computed by the
+    oracle's operator, is what the solver promises (FP32: its own rounding, 6e-8 of a residual amplified by the 6
+    terms of a row, allows 1e-5)."""
+    U = gauge.links(gauge.field(L, 3.0, 0, sweeps=10))
+    m0 = 0.2  # well conditioned: the point is the arithmetic of a step
+    h = api.mg_setup(ctx, torch.from_numpy(U).cuda(), L, m0, ntv=1, setup_sweeps=1, tensor_cores=0, levels=2)
+    try:
+        D = osch.dirac_sparse(U, m0)
+        dt, tol = (np.complex128, 1e-10) if prec == "FP64" else (np.complex64, 1e-5)
+        b = vecs(2 * L * L, nrhs, 4, dt)
+        b[0] *= 1e6  # per-rhs norms and stops
+        bd = torch.from_numpy(b).cuda()
+        xd = torch.empty_like(bd)
+        st = api.fgmres_batched(ctx, h, 0, bd, xd, precond=0, m=m, tol=tol, prec=getattr(api, prec), maxit=4000)
+        x = xd.cpu().numpy().astype(complex)
+        res = np.linalg.norm(b - (D @ x.T).T, axis=1) / np.linalg.norm(b, axis=1)
+        assert st["converged"] and res.max() < 1.5 * tol, res
+        assert st["its"].min() > 0
+    finally:
+        h.close()
