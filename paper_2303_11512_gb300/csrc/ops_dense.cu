@@ -2,6 +2,9 @@
 // Algorithm 2 whose trace is tau_L), the coarsest-level inverse apply, and the
 // Hutch++ pieces of Algorithm 2: the Gram matrix and Cholesky factor of
 // CholeskyQR2 and the projection coefficients Q^H x.
+#include <algorithm>
+#include <type_traits>
+
 #include "ops.cuh"
 
 namespace mg {
@@ -344,38 +347,111 @@ template void invert_large<double2>(cudaStream_t, double2*, int, int*, void*, in
 template void invert_large<float2>(cudaStream_t, float2*, int, int*, void*, int*, int*, long);
 
 // ---- y = A x for the coarsest level (n x n dense, nrhs columns) --------------------------------
-template <typename R>
-__global__ void __launch_bounds__(256) k_dense_apply(const typename CT<R>::T* __restrict__ A, int n,
-                                                     const typename CT<R>::T* __restrict__ x,
-                                                     typename CT<R>::T* __restrict__ y, int nrhs,
-                                                     const int* __restrict__ active) {
-  typedef typename CT<R>::T C;
-  __shared__ C As[16][17];
-  __shared__ C Xs[16][17];
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  const int i = blockIdx.x * 16 + tx;   // row of A
-  const int r = blockIdx.y * 16 + ty;   // rhs
-  C acc = czero<C>();
-  for (int j0 = 0; j0 < n; j0 += 16) {
-    {
-      const int ii = blockIdx.x * 16 + ty, jj = j0 + tx;
-      As[ty][tx] = (ii < n && jj < n) ? A[(size_t)ii * n + jj] : czero<C>();
-      const int rr = blockIdx.y * 16 + ty;
-      Xs[ty][tx] = (rr < nrhs && jj < n) ? x[(size_t)rr * n + jj] : czero<C>();
-    }
-    __syncthreads();
+// Each result is one sum over j in order (a chain of 2 n dependent FMAs: 4 us at n = 1024), so the parallelism is in
+// the results only: blocks of 64 threads with RI rows x NR right-hand sides each, tiles of A and x staged ST chunks of
+// 32 columns deep by cp.async (L2 answers in about 1 us).  In FP32 the bytes that shared memory returns come next,
+// hence 2 x 2 (32 bytes for 16 FMAs).  FP64: each quarter of an SM has its own share of the two FMAs a clock, so the
+// results are spread over as many warps as there are, one a thread.  n = 1024 with 8, 32, 64 rhs: FP32 32, 33, 43 ->
+// 23, 30, 33 us, FP64 275, 275, 523 -> 151, 270, 537 us (tiles of 16 x 16 results and a barrier every 16 columns before).
+template <typename C>
+__device__ __forceinline__ void cp_async_elem(C* dst, const C* src) {
+  const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+  if constexpr (sizeof(C) == 16)
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
+  else
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d), "l"(src) : "memory");
+}
+
+template <typename C, int RI, int NR>
+struct DenseTile {
+  static constexpr int KC = 32, ST = sizeof(C) == 8 ? 8 : 4, TI = 8 * RI, TR = 8 * NR;
+  static constexpr int AP = TI + 16 / (int)sizeof(C), XP = TR + 16 / (int)sizeof(C);  // padded, rows 16-byte aligned
+  C As[ST][KC][AP];  // [column][row]
+  C Xs[ST][KC][XP];  // [column][rhs]
+};
+
+template <typename C, int RI, int NR>
+__global__ void __launch_bounds__(64) k_dense_apply(const C* __restrict__ A, int n, const C* __restrict__ x,
+                                                    C* __restrict__ y, int nrhs, const int* __restrict__ active) {
+  typedef DenseTile<C, RI, NR> DT;
+  constexpr int KC = DT::KC, ST = DT::ST, TI = DT::TI, TR = DT::TR;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  DT& t = *reinterpret_cast<DT*>(smem_raw);
+  const int tid = threadIdx.x, i0 = blockIdx.x * TI, r0 = blockIdx.y * TR;
+  const int ti = tid & 7, tr = tid >> 3;
+  auto fetch = [&](int c) {  // chunk c into stage c % ST: a warp reads 32 consecutive columns of a row
+    const int s = c % ST, j = c * KC + (tid & 31);
+    if (j < n) {
 #pragma unroll
-    for (int q = 0; q < 16; ++q) acc = cfma(As[tx][q], Xs[ty][q], acc);
-    __syncthreads();
+      for (int q = tid >> 5; q < TI; q += 2)
+        if (i0 + q < n) cp_async_elem(&t.As[s][tid & 31][q], A + (size_t)(i0 + q) * n + j);
+#pragma unroll
+      for (int q = tid >> 5; q < TR; q += 2)
+        if (r0 + q < nrhs) cp_async_elem(&t.Xs[s][tid & 31][q], x + (size_t)(r0 + q) * n + j);
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  C acc[RI][NR];
+#pragma unroll
+  for (int a = 0; a < RI; ++a)
+#pragma unroll
+    for (int b = 0; b < NR; ++b) acc[a][b] = czero<C>();
+  const int nch = (n + KC - 1) / KC;
+  for (int c = 0; c < ST - 1; ++c) fetch(c);  // chunks past the end fetch nothing
+  for (int c = 0; c < nch; ++c) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(ST - 2) : "memory");
+    __syncthreads();  // chunk c has landed and chunk c - 1 is consumed
+    fetch(c + ST - 1);
+    const int s = c % ST, cols = min(KC, n - c * KC);
+    auto column = [&](int j) {
+      C m[RI], v[NR];
+#pragma unroll
+      for (int a = 0; a < RI; ++a) m[a] = t.As[s][j][ti * RI + a];
+#pragma unroll
+      for (int b = 0; b < NR; ++b) v[b] = t.Xs[s][j][tr * NR + b];
+#pragma unroll
+      for (int a = 0; a < RI; ++a)
+#pragma unroll
+        for (int b = 0; b < NR; ++b) acc[a][b] = cfma(m[a], v[b], acc[a][b]);
+    };
+    if (cols == KC) {
+#pragma unroll 8
+      for (int j = 0; j < KC; ++j) column(j);
+    } else {
+      for (int j = 0; j < cols; ++j) column(j);
+    }
   }
-  if (i < n && r < nrhs && !(active && !active[r])) y[(size_t)r * n + i] = acc;
+#pragma unroll
+  for (int b = 0; b < NR; ++b) {
+    const int r = r0 + tr * NR + b;
+    if (r >= nrhs || (active && !active[r])) continue;
+#pragma unroll
+    for (int a = 0; a < RI; ++a)
+      if (i0 + ti * RI + a < n) y[(size_t)r * n + i0 + ti * RI + a] = acc[a][b];
+  }
 }
 
 template <typename R>
 void dense_apply(cudaStream_t st, const typename CT<R>::T* A, int n, const typename CT<R>::T* x,
                  typename CT<R>::T* y, int nrhs, const int* active) {
-  dim3 grid(cdiv(n, 16), cdiv(nrhs, 16));
-  MG_LAUNCH(k_dense_apply<R>, grid, 256, 0, st, A, n, x, y, nrhs, active);
+  typedef typename CT<R>::T C;
+  if (nrhs <= 0) return;
+  const double bytes = ((double)n * n + 2.0 * act_rhs(nrhs) * n) * sizeof(C), flops = 8.0 * n * (double)n * act_rhs(nrhs);
+  auto go = [&](auto ri, auto nr) {
+    constexpr int RI = decltype(ri)::value, NR = decltype(nr)::value;
+    constexpr int sm = (int)sizeof(DenseTile<C, RI, NR>);
+    ensure_max_smem((const void*)k_dense_apply<C, RI, NR>, sm);
+    MG_LAUNCH_W(bytes, flops, (k_dense_apply<C, RI, NR>), dim3(cdiv(n, 8 * RI), cdiv(nrhs, 8 * NR)), 64, sm, st, A, n,
+                x, y, nrhs, active);
+  };
+  typedef std::integral_constant<int, 1> I1;
+  typedef std::integral_constant<int, 2> I2;
+  if constexpr (sizeof(R) == 8)
+    go(I1(), I1());
+  else if (nrhs <= 8)
+    go(I2(), I1());
+  else
+    go(I2(), I2());
 }
 template void dense_apply<float>(cudaStream_t, const float2*, int, const float2*, float2*, int, const int*);
 template void dense_apply<double>(cudaStream_t, const double2*, int, const double2*, double2*, int, const int*);

@@ -97,3 +97,16 @@ def test_krylov_step_forms(api, ctx, L, nrhs, m, prec):
         assert st["its"].min() > 0
     finally:
         h.close()
+
+
+@pytest.mark.parametrize("prec,tol", [("FP64", 1e-12), ("FP32", 1e-5)])
+@pytest.mark.parametrize("nrhs", [1, 8, 9, 17, 65])
+def test_coarsest_apply_tiles(api, ctx, nrhs, prec, tol):
+    """The coarsest level's dense inverse at the remainders of its 8 and 16 rhs tiles (sums of 128 products; the
+    inverse's condition, below 100, is in the tolerance)."""
+    h, H = hierarchy(api, ctx, 16)
+    top = h.levels - 1
+    b = vecs(H.n[top], nrhs, 6, np.complex128 if prec == "FP64" else np.complex64)
+    xd = torch.empty(b.shape, dtype=torch.from_numpy(b).dtype, device="cuda")
+    h.vcycle(top, torch.from_numpy(b).cuda(), xd, getattr(api, prec))
+    assert relerr(xd.cpu().numpy(), H.vcycle(top, b.T).T) < tol
