@@ -416,9 +416,12 @@ void nn_forward(NNet* net, const float2* r, float2* y, int nrhs, bool tape, cuda
 double nn_backward(NNet* net, const float2* r, const float2* e, int nrhs, cudaStream_t st, int* pinned) {
   const int L = net->L, V = L * L;
   const long n = 2L * V;  // complex per rhs of the input/output fields
-  DBuf y(sizeof(float2) * n * nrhs, st), g(sizeof(float2) * n * nrhs, st);
+  DBuf &y = net->b_y, &g = net->b_g, &nrm = net->b_n, &red = net->b_red;  // kept between steps
+  y.ensure(sizeof(float2) * n * nrhs, st);
+  g.ensure(sizeof(float2) * n * nrhs, st);
+  nrm.ensure(sizeof(double) * 2 * nrhs, st);
+  red.ensure(reduce_work_bytes(n, nrhs, 1), st);
   nn_forward(net, r, y.as<float2>(), nrhs, true, st);
-  DBuf nrm(sizeof(double) * 2 * nrhs, st), red(reduce_work_bytes(n, nrhs, 1), st);
   vnorm2<float2>(st, e, n, nrhs, nrm.as<double>(), red.p, nullptr);
   MG_LAUNCH(k_nn_diff, dim3(cdiv(n, 256), nrhs), 256, 0, st, y.as<float2>(), e, g.as<float2>(), n);
   vnorm2<float2>(st, g.as<float2>(), n, nrhs, nrm.as<double>() + nrhs, red.p, nullptr);

@@ -19,6 +19,9 @@ struct NNet {
   std::vector<DBuf> acts, zs; // training tape (FP32 layer inputs, hidden pre-activations)
   std::vector<DBuf> acts16;   // tensor-core layers: BF16 layer inputs (the tape, or two ping-pong buffers)
   std::vector<DBuf> wimg;     // tensor-core weight images per layer: forward, conjugate-transposed
+  // training workspaces: output, its gradient, norms and their partial sums; tensor-core backward: BF16 g_z, layer
+  // gradient, bias and weight partials
+  DBuf b_y, b_g, b_n, b_red, b_gz, b_ga, b_bpart, b_wpart;
   DBuf err;                   // device int: set by a tensor-core kernel whose bounded wait expired
   int dim(int l) const;
   size_t w_offset(int l) const;
@@ -39,7 +42,8 @@ void nn_check(NNet* net, cudaStream_t st);
 
 // tensor-core layers (nn_tc.cu): lattice sides that are multiples of 16 (whole 128-site tiles per rhs)
 bool nn_tc_supported(int L);
-void nn_tc_weights(NNet* net, cudaStream_t st);
+// weight images of the current parameters, the conjugate-transposed ones of the backward pass if asked for
+void nn_tc_weights(NNet* net, bool backward, cudaStream_t st);
 // y = M(r / rscale[rhs]) (rscale null: 1); with a tape the BF16 layer inputs and FP32 pre-activations are kept
 void nn_tc_forward(NNet* net, const float2* r, const double* rscale, float2* y, int nrhs, bool tape, int* err,
                    cudaStream_t st);

@@ -362,6 +362,18 @@ __host__ __device__ constexpr uint32_t nw_cols(int ci) {
   return nw_nb(ci) <= 32 ? 32u : nw_nb(ci) <= 64 ? 64u : nw_nb(ci) <= 128 ? 128u : 256u;
 }
 
+// NW consecutive words (16-, 8- or 4-byte load; the address is aligned to it)
+template <int NW>
+__device__ __forceinline__ void nw_load(const uint32_t* __restrict__ p, uint32_t* v) {
+  if constexpr (NW == 4) {
+    const uint4 q = __ldg(reinterpret_cast<const uint4*>(p));
+    v[0] = q.x; v[1] = q.y; v[2] = q.z; v[3] = q.w;
+  } else {
+    const uint2 q = __ldg(reinterpret_cast<const uint2*>(p));
+    v[0] = q.x; v[1] = q.y;
+  }
+}
+
 // part[cta][2 CO][9 CI]: this CTA's sums over its chunks of Re / Im (g_z conj(u_d)) for (k, d, c)
 template <int CI, int CO>
 __global__ void __launch_bounds__(NW_THREADS, 1)
@@ -418,24 +430,35 @@ __global__ void __launch_bounds__(NW_THREADS, 1)
       const long R0 = (long)(blockIdx.x + (long)i * gridDim.x) * NW_X;
       const long rr = R0 / V;
       const int s0 = (int)(R0 - rr * V);
+      // The lanes of a warp take consecutive sites of one row group, so their 4-byte words fall into 32 distinct
+      // banks (with the taps of a site in neighbouring lanes nine of them met in one bank); a site's channels come
+      // as 16-byte loads.
       // A: g_z rows (Re: (g_re, g_im), Im: (g_im, -g_re) on the site's K pair)
-      for (int u = tid; u < NW_X * CO; u += NW_CONV_WARPS * 32) {
-        const int xl = u / CO, k = u - xl * CO;
-        const uint32_t v = __ldg(gz16 + (size_t)(R0 + xl) * CO + k);
+      constexpr int AW = CO < 4 ? CO : 4, BW = CI < 4 ? CI : 4;  // 4-byte words per load
+      for (int u = tid; u < NW_X * (CO / AW); u += NW_CONV_WARPS * 32) {
+        const int xl = u % NW_X, k0 = (u / NW_X) * AW;
+        uint32_t v[AW];
+        nw_load<AW>(gz16 + (size_t)(R0 + xl) * CO + k0, v);
         uint32_t* A = reinterpret_cast<uint32_t*>(sA(s, xl >> 5));
-        A[word(k, xl)] = v;
-        A[word(CO + k, xl)] = (v >> 16) | (((v & 0xFFFFu) ^ 0x8000u) << 16);
+#pragma unroll
+        for (int q = 0; q < AW; ++q) {
+          A[word(k0 + q, xl)] = v[q];
+          A[word(CO + k0 + q, xl)] = (v[q] >> 16) | (((v[q] & 0xFFFFu) ^ 0x8000u) << 16);
+        }
       }
       // B: transported inputs u_d(x)_c = T_d(x) a(x + d)_c, rows d * CI + c
       for (int u = tid; u < NW_X * NM_TAPS; u += NW_CONV_WARPS * 32) {
-        const int xl = u / NM_TAPS, e = u - xl * NM_TAPS;
+        const int xl = u % NW_X, e = u / NW_X;
         const int site = s0 + xl, t = site / L, x = site - t * L;
         const float2 te = __ldg(T + (size_t)site * NM_TAPS + e);
         const uint32_t* ar = a16 + ((size_t)rr * V + nm_nbr(t, x, e, L)) * CI;
         uint32_t* B = reinterpret_cast<uint32_t*>(sB(s, xl >> 5));
+        uint32_t w[CI];
+#pragma unroll
+        for (int c = 0; c < CI; c += BW) nw_load<BW>(ar + c, w + c);
 #pragma unroll
         for (int c = 0; c < CI; ++c) {
-          const float2 av = bf16x2_to_f2(__ldg(ar + c));
+          const float2 av = bf16x2_to_f2(w[c]);
           B[word(e * CI + c, xl)] = bf16x2_rn(te.x * av.x - te.y * av.y, te.x * av.y + te.y * av.x);
         }
       }
@@ -492,25 +515,44 @@ __global__ void __launch_bounds__(NW_THREADS, 1)
   }
 }
 
-// grad[2 ((d CO + k) CI + c) + {0, 1}] = sums over the CTAs (fixed order) of the Re / Im partials
-__global__ void k_nn_wgrad_reduce(const float* __restrict__ part, int nblk, int ci, int co, float* __restrict__ grad) {
-  const int w = blockIdx.x * blockDim.x + threadIdx.x;  // (d, k, c)
-  if (w >= 9 * co * ci) return;
-  const int d = w / (co * ci), k = (w / ci) % co, c = w % ci;
-  const size_t stride = (size_t)2 * co * 9 * ci;
-  const size_t ore = (size_t)k * 9 * ci + d * ci + c, oim = (size_t)(co + k) * 9 * ci + d * ci + c;
+// grad[2 ((d CO + k) CI + c) + {0, 1}] = sums over the CTAs of the Re / Im partials: 32 weights by 8 slices of the
+// partials per block (fixed order)
+__global__ void __launch_bounds__(256) k_nn_wgrad_reduce(const float* __restrict__ part, int nblk, int ci, int co,
+                                                         float* __restrict__ grad) {
+  __shared__ double sh[2][8][33];
+  const int x = threadIdx.x & 31, y = threadIdx.x >> 5;
+  const int w = blockIdx.x * 32 + x;  // (d, k, c)
   double re = 0, im = 0;
-  for (int b = 0; b < nblk; ++b) {
-    re += part[b * stride + ore];
-    im += part[b * stride + oim];
+  if (w < 9 * co * ci) {
+    const int d = w / (co * ci), k = (w / ci) % co, c = w % ci;
+    const size_t stride = (size_t)2 * co * 9 * ci;
+    const size_t ore = (size_t)k * 9 * ci + d * ci + c, oim = (size_t)(co + k) * 9 * ci + d * ci + c;
+    for (int b = y; b < nblk; b += 8) {
+      re += part[b * stride + ore];
+      im += part[b * stride + oim];
+    }
   }
-  grad[2 * w] = (float)re;
-  grad[2 * w + 1] = (float)im;
+  sh[0][y][x] = re;
+  sh[1][y][x] = im;
+  __syncthreads();
+  if (y < 2 && w < 9 * co * ci) {
+    double t = 0;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) t += sh[y][q][x];
+    grad[2 * w + y] = (float)t;
+  }
 }
 
-// weight image of one layer: forward B_d = W_d (rows = outputs co), or backward B_e = conj(W_(8-e))^T (rows =
-// inputs ci); rows [0, NC) Re, [NC, 2 NC) Im, K element j = 2 c + part; BF16 in the 64-byte swizzle
-__global__ void k_nn_wimg(const float* __restrict__ p, int ci, int co, int bwd, __nv_bfloat16* __restrict__ img) {
+// weight images: forward B_d = W_d (rows = outputs co), or backward B_e = conj(W_(8-e))^T (rows = inputs ci); rows
+// [0, NC) Re, [NC, 2 NC) Im, K element j = 2 c + part; BF16 in the 64-byte swizzle.  All images of a net in one
+// launch (blockIdx.y).
+struct WimgTable {
+  struct { const float* p; __nv_bfloat16* img; int ci, co, bwd; } e[16];
+};
+__global__ void k_nn_wimg(WimgTable tab) {
+  const float* __restrict__ p = tab.e[blockIdx.y].p;
+  const int ci = tab.e[blockIdx.y].ci, co = tab.e[blockIdx.y].co, bwd = tab.e[blockIdx.y].bwd;
+  __nv_bfloat16* __restrict__ img = tab.e[blockIdx.y].img;
   const int nout = bwd ? ci : co, nin = bwd ? co : ci;
   const int NC = nout < 8 ? 8 : nout, N = 2 * NC;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;  // (e, n, j)
@@ -542,53 +584,74 @@ __global__ void k_nn_to_bf16(const float2* __restrict__ x, long n, const double*
   }
 }
 
-// activation backward: g (w.r.t. the activation output, FP32) and the pre-activation z -> g_z as BF16 pairs;
-// bias partial sums per block
+// activation backward: g (w.r.t. the activation output, FP32) and the pre-activation z -> g_z as BF16 pairs; bias
+// partial sums per block of 128 rows.  Bound by memory (20 bytes per entry): a thread takes two channels of a row as
+// 16-byte loads, CO / 2 neighbouring threads a row, every thread the same channels of its rows.
 template <int CO>
-__global__ void __launch_bounds__(128) k_nn_act_bwd16(const float2* __restrict__ z, const float* __restrict__ b,
+__global__ void __launch_bounds__(256) k_nn_act_bwd16(const float2* __restrict__ z, const float* __restrict__ b,
                                                       const float2* __restrict__ g, long rows,
                                                       uint32_t* __restrict__ gz, float* __restrict__ bpart) {
-  __shared__ float red[4][CO];
-  const long i = blockIdx.x * (long)blockDim.x + threadIdx.x;
-  float rb[CO];
+  constexpr int TPR = CO / 2, RPB = 256 / TPR;  // threads per row, rows at a time
+  __shared__ float red[8][CO];
+  const int kp = threadIdx.x % TPR;
+  const float bk[2] = {b[2 * kp], b[2 * kp + 1]};
+  float rb[2] = {0.f, 0.f};
 #pragma unroll
-  for (int k = 0; k < CO; ++k) rb[k] = 0.f;
-  if (i < rows) {
+  for (int q = 0; q < 128 / RPB; ++q) {
+    const long i = blockIdx.x * 128L + q * RPB + threadIdx.x / TPR;
+    if (i < rows) {
+      const float4 z4 = *reinterpret_cast<const float4*>(z + i * CO + 2 * kp);
+      const float4 g4 = *reinterpret_cast<const float4*>(g + i * CO + 2 * kp);
+      uint32_t o16[2];
 #pragma unroll
-    for (int k = 0; k < CO; ++k) {
-      const float2 zz = z[i * CO + k];
-      const float2 gg = g[i * CO + k];
-      const float mg = sqrtf(zz.x * zz.x + zz.y * zz.y);
-      float2 o = make_float2(0.f, 0.f);
-      if (mg > 0.f && mg + b[k] > 0.f) {
-        const float2 ph = make_float2(zz.x / mg, zz.y / mg);
-        const float rad = ph.x * gg.x + ph.y * gg.y;
-        const float sc = (mg + b[k]) / mg;
-        o = make_float2(rad * ph.x + sc * (gg.x - rad * ph.x), rad * ph.y + sc * (gg.y - rad * ph.y));
-        rb[k] = rad;
+      for (int c = 0; c < 2; ++c) {
+        const float2 zz = c ? make_float2(z4.z, z4.w) : make_float2(z4.x, z4.y);
+        const float2 gg = c ? make_float2(g4.z, g4.w) : make_float2(g4.x, g4.y);
+        const float mg = sqrtf(zz.x * zz.x + zz.y * zz.y);
+        float2 o = make_float2(0.f, 0.f);
+        if (mg > 0.f && mg + bk[c] > 0.f) {
+          const float2 ph = make_float2(zz.x / mg, zz.y / mg);
+          const float rad = ph.x * gg.x + ph.y * gg.y;
+          const float sc = (mg + bk[c]) / mg;
+          o = make_float2(rad * ph.x + sc * (gg.x - rad * ph.x), rad * ph.y + sc * (gg.y - rad * ph.y));
+          rb[c] += rad;
+        }
+        o16[c] = bf16x2_rn(o.x, o.y);
       }
-      gz[i * CO + k] = bf16x2_rn(o.x, o.y);
+      *reinterpret_cast<uint2*>(gz + i * CO + 2 * kp) = make_uint2(o16[0], o16[1]);
     }
   }
   const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
 #pragma unroll
-  for (int k = 0; k < CO; ++k) {
-    float v = rb[k];
-    for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffff, v, o);
-    if (l == 0) red[w][k] = v;
+  for (int c = 0; c < 2; ++c) {
+    float v = rb[c];
+#pragma unroll
+    for (int o = 16; o >= TPR; o >>= 1) v += __shfl_xor_sync(0xffffffff, v, o);  // lanes of the same channels
+    if (l < TPR) red[w][2 * l + c] = v;
   }
   __syncthreads();
-  if (threadIdx.x < CO)
-    bpart[(size_t)blockIdx.x * CO + threadIdx.x] =
-        red[0][threadIdx.x] + red[1][threadIdx.x] + red[2][threadIdx.x] + red[3][threadIdx.x];
+  if (threadIdx.x < CO) {
+    float v = 0.f;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) v += red[q][threadIdx.x];
+    bpart[(size_t)blockIdx.x * CO + threadIdx.x] = v;
+  }
 }
 
-__global__ void k_nn_reduce_bias(const float* __restrict__ part, int nblk, int count, float* __restrict__ grad) {
-  const int w = blockIdx.x * blockDim.x + threadIdx.x;
-  if (w >= count) return;
+// bias gradient: one block per channel, the partials summed in a fixed order
+__global__ void __launch_bounds__(256) k_nn_reduce_bias(const float* __restrict__ part, int nblk, int count,
+                                                        float* __restrict__ grad) {
+  __shared__ double sh[256];
   double s = 0;
-  for (int b = 0; b < nblk; ++b) s += part[(size_t)b * count + w];
-  grad[w] = (float)s;
+  for (int b = threadIdx.x; b < nblk; b += 256) s += part[(size_t)b * count + blockIdx.x];
+  sh[threadIdx.x] = s;
+  __syncthreads();
+#pragma unroll
+  for (int o = 128; o; o >>= 1) {
+    if (threadIdx.x < o) sh[threadIdx.x] += sh[threadIdx.x + o];
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) grad[blockIdx.x] = (float)sh[0];
 }
 
 template <typename F>
@@ -678,26 +741,28 @@ size_t nn_tc_wimg_bytes(int co) { return (size_t)nm_wbytes(co); }
 
 bool nn_tc_supported(int L) { return L >= 16 && L % 16 == 0; }
 
-void nn_tc_weights(NNet* net, cudaStream_t st) {
+void nn_tc_weights(NNet* net, bool backward, cudaStream_t st) {
   net->wimg.resize(2 * net->layers);
+  WimgTable tab;
+  int cnt = 0, most = 0;
   for (int l = 0; l < net->layers; ++l) {
     const int ci = net->dim(l), co = net->dim(l + 1);
-    for (int bwd = 0; bwd < 2; ++bwd) {
+    for (int bwd = 0; bwd <= (backward ? 1 : 0); ++bwd) {
       const int nout = bwd ? ci : co;
       DBuf& img = net->wimg[2 * l + bwd];
       img.ensure(nn_tc_wimg_bytes(nout), st);
-      const int cnt = NM_TAPS * nm_n(nout) * 32;
-      MG_LAUNCH(k_nn_wimg, cdiv(cnt, 256), 256, 0, st, net->params.as<float>() + net->w_offset(l), ci, co, bwd,
-                img.as<__nv_bfloat16>());
+      tab.e[cnt++] = {net->params.as<float>() + net->w_offset(l), img.as<__nv_bfloat16>(), ci, co, bwd};
+      most = std::max(most, NM_TAPS * nm_n(nout) * 32);
     }
   }
+  MG_LAUNCH(k_nn_wimg, dim3(cdiv(most, 256), cnt), 256, 0, st, tab);
 }
 
 void nn_tc_forward(NNet* net, const float2* r, const double* rscale, float2* y, int nrhs, bool tape, int* err,
                    cudaStream_t st) {
   const int L = net->L, V = L * L;
   const long n = 2L * V;
-  nn_tc_weights(net, st);
+  nn_tc_weights(net, tape, st);
   const int nl = net->layers;
   net->acts16.resize(nl);
   if (tape) net->zs.resize(nl);
@@ -731,7 +796,9 @@ void nn_tc_backward(NNet* net, float2* g, int nrhs, int* err, cudaStream_t st) {
   const int L = net->L, V = L * L;
   const long rows = (long)nrhs * V;
   const int nl = net->layers;
-  DBuf gz16(sizeof(uint32_t) * rows * 16, st), ga(sizeof(float2) * rows * 16, st);
+  DBuf &gz16 = net->b_gz, &ga = net->b_ga, &bpart = net->b_bpart, &part = net->b_wpart;  // kept between steps
+  gz16.ensure(sizeof(uint32_t) * rows * net->channels, st);
+  ga.ensure(sizeof(float2) * rows * net->channels, st);
   MG_LAUNCH(k_nn_to_bf16, dim3((unsigned)std::min<long>(cdiv(2L * V, 256), 1024), nrhs), 256, 0, st, g, 2L * V,
             nullptr, gz16.as<uint32_t>());
   const int nsm = nsm_count();
@@ -740,21 +807,21 @@ void nn_tc_backward(NNet* net, float2* g, int nrhs, int* err, cudaStream_t st) {
     const size_t woff = net->w_offset(l);
     if (l < nl - 1) {  // activation backward: ga (w.r.t. this layer's output) -> gz16, bias gradient
       const int nb = (int)cdiv(rows, 128);
-      DBuf bpart(sizeof(float) * nb * co, st);
+      bpart.ensure(sizeof(float) * nb * co, st);
       const float* b = net->params.as<float>() + woff + 2 * 9 * co * ci;
       switch (co) {
-        case 4: MG_LAUNCH((k_nn_act_bwd16<4>), nb, 128, 0, st, net->zs[l].as<float2>(), b, ga.as<float2>(), rows, gz16.as<uint32_t>(), bpart.as<float>()); break;
-        case 8: MG_LAUNCH((k_nn_act_bwd16<8>), nb, 128, 0, st, net->zs[l].as<float2>(), b, ga.as<float2>(), rows, gz16.as<uint32_t>(), bpart.as<float>()); break;
-        case 16: MG_LAUNCH((k_nn_act_bwd16<16>), nb, 128, 0, st, net->zs[l].as<float2>(), b, ga.as<float2>(), rows, gz16.as<uint32_t>(), bpart.as<float>()); break;
+        case 4: MG_LAUNCH((k_nn_act_bwd16<4>), nb, 256, 0, st, net->zs[l].as<float2>(), b, ga.as<float2>(), rows, gz16.as<uint32_t>(), bpart.as<float>()); break;
+        case 8: MG_LAUNCH((k_nn_act_bwd16<8>), nb, 256, 0, st, net->zs[l].as<float2>(), b, ga.as<float2>(), rows, gz16.as<uint32_t>(), bpart.as<float>()); break;
+        case 16: MG_LAUNCH((k_nn_act_bwd16<16>), nb, 256, 0, st, net->zs[l].as<float2>(), b, ga.as<float2>(), rows, gz16.as<uint32_t>(), bpart.as<float>()); break;
         default: throw Error(MGMLMC_ERR_INVALID_ARG, "unsupported hidden channel count");
       }
-      MG_LAUNCH(k_nn_reduce_bias, cdiv(co, 64), 64, 0, st, bpart.as<float>(), nb, co,
+      MG_LAUNCH(k_nn_reduce_bias, co, 256, 0, st, bpart.as<float>(), nb, co,
                 net->grad.as<float>() + woff + 2 * 9 * co * ci);
     }
     // weight gradient
     const int nchunks = (int)(rows / NW_X);
     const int grid = std::max(1, std::min(nchunks, nsm));
-    DBuf part(sizeof(float) * (size_t)grid * 2 * co * 9 * ci, st);
+    part.ensure(sizeof(float) * (size_t)grid * 2 * co * 9 * ci, st);
     with_dims_tc(ci, co, [&](auto CI, auto CO) {
       auto* k = &k_nn_wgrad<CI.value, CO.value>;
       const int sm = nw_smem(CI.value);
@@ -763,7 +830,7 @@ void nn_tc_backward(NNet* net, float2* g, int nrhs, int* err, cudaStream_t st) {
                   net->acts16[l].as<uint32_t>(), gz16.as<uint32_t>(), net->T.as<float2>(), L, nchunks,
                   part.as<float>(), err);
     });
-    MG_LAUNCH(k_nn_wgrad_reduce, cdiv(9 * co * ci, 128), 128, 0, st, part.as<float>(), grid, ci, co,
+    MG_LAUNCH(k_nn_wgrad_reduce, cdiv(9 * co * ci, 32), 256, 0, st, part.as<float>(), grid, ci, co,
               net->grad.as<float>() + woff);
     // input gradient (the gathered mixing with the conjugate-transposed weights), FP32
     if (l > 0) mix_launch(st, net, co, ci, false, gz16.p, net->wimg[2 * l + 1].p, nullptr, ga.as<float2>(), nullptr, nrhs, err);
