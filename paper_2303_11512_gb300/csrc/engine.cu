@@ -50,6 +50,12 @@ void op_apply(mgmlmc_hier* h, int l, const typename CT<R>::T* x, typename CT<R>:
     coarse_apply<R>(st, st_of<R>(L), L.side, L.dof, x, y, b, nrhs, active);
 }
 
+// the SAP sweeps of level l run on the tensor cores
+template <typename R>
+static bool tc_smoother(const mgmlmc_hier* h, int l) {
+  return sizeof(R) == 4 && h->use_tc(l) && h->lv[l].sap_bs == 2 && h->lv[l].tcInv[0].p;
+}
+
 template <typename R>
 void sap_sweep(mgmlmc_hier* h, int l, const typename CT<R>::T* f, typename CT<R>::T* x, int nrhs,
                const int* active, void* x16, bool zero) {
@@ -57,7 +63,7 @@ void sap_sweep(mgmlmc_hier* h, int l, const typename CT<R>::T* f, typename CT<R>
   cudaStream_t st = h->ctx->stream;
   if (sizeof(R) == 8 && !L.sap64_ok) throw Error(MGMLMC_ERR_INVALID_ARG, "FP64 SAP inverse not built at this level");
   if constexpr (sizeof(R) == 4) {
-    if (h->use_tc(l) && L.sap_bs == 2 && L.tcInv[0].p) {
+    if (tc_smoother<R>(h, l)) {
       float2* res = (float2*)h->work("tc_res", l, sizeof(float2) * L.n * nrhs);
       if (!x16 && tc_block_selected(L.tc_bf, L.side, nrhs)) {  // the block stencil reads a 16-bit copy of x
         x16 = h->work("sap_x16", l, sizeof(uint32_t) * L.n * nrhs);
@@ -74,7 +80,8 @@ void sap_sweep(mgmlmc_hier* h, int l, const typename CT<R>::T* f, typename CT<R>
       sap_half_fine<R>(st, links_of<R>(L), (R)L.diag, L.side, L.sap_bs, sapinv_of<R>(L), f, x, color, nrhs, active,
                        sizeof(R) == 4 && L.sapinv32_t, !zero ? SAP_X : color == 0 ? SAP_ZERO : SAP_OTHER);
     else
-      sap_half_coarse<R>(st, st_of<R>(L), L.side, L.dof, L.sap_bs, sapinv_of<R>(L), f, x, color, nrhs, active);
+      sap_half_coarse<R>(st, st_of<R>(L), L.side, L.dof, L.sap_bs, sapinv_of<R>(L), f, x, color, nrhs, active,
+                         zero && color == 0);
   }
 }
 
@@ -111,15 +118,15 @@ void vcycle(mgmlmc_hier* h, int l, const typename CT<R>::T* r, typename CT<R>::T
     if (h->use_tc(l) && tc_block_selected(L.tc_bf, L.side, nrhs))
       e16 = h->work("vc_e16", l, sizeof(uint32_t) * L.n * nrhs);
   }
-  // the fine smoother starts from zero without reading e; its two colours then write every site
-  const bool lazy_zero = l == 0 && L.sap_bs == 4 && h->prm.pre_smooth > 0;
+  // the CUDA-core smoothers start from zero without reading e; their two colours then write every site
+  const bool lazy_zero = h->prm.pre_smooth > 0 && (l == 0 ? L.sap_bs == 4 : !tc_smoother<R>(h, l));
   if (!lazy_zero) vzero<C>(st, e, L.n, nrhs);
   if (e16) MG_CUDA(cudaMemsetAsync(e16, 0, sizeof(uint32_t) * L.n * nrhs, st));
   for (int s = 0; s < h->prm.pre_smooth; ++s) sap_sweep<R>(h, l, r, e, nrhs, active, e16, lazy_zero && s == 0);
   bool done = false;
   if constexpr (sizeof(R) == 4) {
     if (h->use_tc(l)) {  // res = r - D e on the tensor cores (preconditioner accuracy)
-      if (h->prm.pre_smooth > 0 && L.sap_bs == 2 && L.tcInv[0].p)  // zero on the blocks the sweep solved last
+      if (h->prm.pre_smooth > 0 && tc_smoother<R>(h, l))  // zero on the blocks the sweep solved last
         tc_residual_after_sap(st, L.tcW.p, L.tc_bf, L.side, e, e16, res, r, nrhs, active, h->tc_err.as<int>());
       else
         tc_stencil_apply(st, L.tcW.p, L.tc_bf, L.side, e, e16, res, r, nrhs, active, h->tc_err.as<int>());

@@ -135,7 +135,8 @@ void build_hierarchy(mgmlmc_ctx* ctx, mgmlmc_hier* h, const double2* U);
 
 // One SAP sweep (colour 0 then 1) for D_l x = f.  x16: the planar 16-bit copy of x that the tensor-core sweep
 // keeps up to date where the 2x2-block stencil is selected (tc_block_selected); nullptr makes the sweep derive
-// one from x first.  zero (level 0 with 4 x 4 blocks only): x counts as zero, its old values are not read.
+// one from x first.  zero: x counts as zero, its old values are not read
+// (level 0 with 4 x 4 blocks and the CUDA-core sweeps of coarse levels).
 template <typename R>
 void sap_sweep(mgmlmc_hier* h, int l, const typename CT<R>::T* f, typename CT<R>::T* x, int nrhs, const int* active,
                void* x16 = nullptr, bool zero = false);

@@ -42,7 +42,7 @@ void blocks_to_fp32_transposed(cudaStream_t st, const double2* in, int nb, int b
 template <typename R>
 void sap_half_coarse(cudaStream_t st, const typename CT<R>::T* stencil, int Ls, int d, int bs,
                      const typename CT<R>::T* inv, const typename CT<R>::T* f, typename CT<R>::T* x,
-                     int color, int nrhs, const int* active);
+                     int color, int nrhs, const int* active, bool zero = false);  // zero: x counts as zero, it is not read
 
 // ---------------------------------------------------------------- transfer
 // P layout: [aggregate][chirality 2][bsz = agg*agg*d/2][ntv]

@@ -144,85 +144,146 @@ void coarse_block_matrices(cudaStream_t stm, const double2* st, int Ls, int d, i
   MG_LAUNCH(k_coarse_blocks, nb, 256, 0, stm, st, Ls, d, bs, out);
 }
 
-template <typename R>
-__global__ void __launch_bounds__(256) k_sap_coarse(const typename CT<R>::T* __restrict__ st, int Ls, int d, int bs,
-                                                    const typename CT<R>::T* __restrict__ inv,
-                                                    const typename CT<R>::T* __restrict__ f,
-                                                    typename CT<R>::T* __restrict__ x, int color, int nrhs,
-                                                    const int* __restrict__ active) {
+// SAP half sweep.  The blocks of one colour do not couple, so with E the hops that leave the block
+// x_B + D_BB^{-1} (f - D x)_B = D_BB^{-1} (f - E x)_B: the hops inside the block and the old x_B drop out (of the 5
+// stencil blocks of a site in a 2 x 2 block 2 remain).  One CTA per block and tile of G right-hand sides; a thread
+// owns one row of the block (lanes: consecutive rows) and 4 right-hand sides.
+// FP64 is bound by its units (two FMAs a clock and SM, a share in each quarter): the rows of the inverse and the
+// stencil come straight from global memory (32 lines per load, which costs an eighth of the FMAs they feed) and the
+// CTA stays small, so that lattices with few blocks fill the chip (one 150 KB CTA of 4 rhs per SM before: 0.70 TF).
+// FP32 stages both transposed in shared memory.
+constexpr int SC_T = 128, SC_R = 4;
+struct SapCoarseShape {
+  int bs, d, bd, ng, G, GP, nslot;
+  __host__ __device__ SapCoarseShape(int bs_, int d_) : bs(bs_), d(d_) {
+    bd = bs * bs * d;
+    ng = SC_T / bd;
+    G = ng * SC_R;
+    GP = G + 1;
+    nslot = 4 * bs;
+  }
+  __host__ __device__ int complexes(bool stage) const {
+    return bd * GP + nslot * d * GP + (stage ? bd * bd + nslot * d * d : 0);
+  }
+};
+
+template <typename R, int BS, int DT>  // BS, DT: block side and dof at compile time (0: runtime)
+__global__ void __launch_bounds__(SC_T) k_sap_coarse(const typename CT<R>::T* __restrict__ st, int Ls, int d_, int bs_,
+                                                     const typename CT<R>::T* __restrict__ inv,
+                                                     const typename CT<R>::T* __restrict__ f,
+                                                     typename CT<R>::T* __restrict__ x, int color, int nrhs, bool zero,
+                                                     const int* __restrict__ active) {
   typedef typename CT<R>::T C;
+  constexpr bool STAGE = sizeof(R) == 4;
+  const SapCoarseShape sh(BS ? BS : bs_, DT ? DT : d_);
+  const int bs = sh.bs, d = sh.d, bd = sh.bd, G = sh.G, GP = sh.GP, dd = d * d;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int ns = bs * bs, bd = ns * d, dd = d * d;
-  const int G = max(1, (int)blockDim.x / bd);
-  C* sinv = reinterpret_cast<C*>(smem_raw);     // [bd][bd]
-  C* sst = sinv + bd * bd;                      // [j][dir][k'][k] transposed stencil of block sites
-  C* sres = sst + ns * 5 * dd;                  // [g][bd]
+  C* sres = reinterpret_cast<C*>(smem_raw);      // [row][rhs]
+  C* sx = sres + bd * GP;                        // [slot][k][rhs]: x on the sites around the block
+  C* sinv = sx + sh.nslot * d * GP;              // [column][row] (FP32)
+  C* sst = sinv + bd * bd;                       // [slot][k][row of the site] (FP32)
+  const int tid = threadIdx.x;
   const int nbx = Ls / bs, half = nbx / 2;
-  const int kb = blockIdx.x;
-  const int BT = kb / half;
-  const int BX = 2 * (kb % half) + ((BT + color) & 1);
-  const int blk = BT * nbx + BX;
-  const C* I = inv + (size_t)blk * bd * bd;
-  // transposed, sinv[j * bd + i] = inv[i][j]: threads of a warp differ in i
-  for (int e = threadIdx.x; e < bd * bd; e += blockDim.x) sinv[(e % bd) * bd + e / bd] = I[e];
-  for (int e = threadIdx.x; e < ns * 5 * dd; e += blockDim.x) {
-    const int j = e / (5 * dd), r = e % (5 * dd), dir = r / dd, q = r % dd, i = q / d, k = q % d;
-    const int s = (BT * bs + j / bs) * Ls + BX * bs + j % bs;
-    sst[(j * 5 + dir) * dd + k * d + i] = st[((size_t)s * 5 + dir) * dd + q];
-  }
+  const int BT = blockIdx.x / half;
+  const int BX = 2 * (blockIdx.x - BT * half) + ((BT + color) & 1);
+  const int t0 = BT * bs, x0 = BX * bs, r0 = blockIdx.y * G;
   const size_t n = (size_t)Ls * Ls * d;
-  for (int r0 = 0; r0 < nrhs; r0 += G) {
-    __syncthreads();
-    for (int q = threadIdx.x; q < G * bd; q += blockDim.x) {
-      const int g = q / bd, i = q % bd, j = i / d, k = i % d;
-      const int rhs = r0 + g;
-      if (rhs < nrhs && !(active && !active[rhs])) {
-        const int s = (BT * bs + j / bs) * Ls + BX * bs + j % bs;
-        const C* X = x + rhs * n;
-        C acc = __ldg(f + rhs * n + (size_t)s * d + k);
-        for (int dir = 0; dir < 5; ++dir) {
-          const C* xv = X + (size_t)nbr_site(s, dir, Ls) * d;
-          const C* a = sst + (j * 5 + dir) * dd + k;
-          for (int kk = 0; kk < d; ++kk) acc = csub(acc, cmul(a[kk * d], xv[kk]));
-        }
-        sres[g * bd + i] = acc;
-      }
-    }
-    __syncthreads();
-    for (int q = threadIdx.x; q < G * bd; q += blockDim.x) {
-      const int g = q / bd, i = q % bd, j = i / d, k = i % d;
-      const int rhs = r0 + g;
-      if (rhs < nrhs && !(active && !active[rhs])) {
-        C acc = czero<C>();
-        for (int jj = 0; jj < bd; ++jj) acc = cfma(sinv[jj * bd + i], sres[g * bd + jj], acc);
-        const int s = (BT * bs + j / bs) * Ls + BX * bs + j % bs;
-        C* px = x + rhs * n + (size_t)s * d + k;
-        *px = cadd(*px, acc);
-      }
+  const C* I = inv + (size_t)(BT * nbx + BX) * bd * bd;
+  // slot: the -x, +x neighbours by row, then the -t, +t neighbours by column; the block's site and direction of each
+  auto slot_site = [&](int s) { const int e = s / bs, i = s - e * bs; return e < 2 ? i * bs + (e ? bs - 1 : 0) : (e == 3 ? (bs - 1) * bs : 0) + i; };
+  auto slot_dir = [&](int s) { const int e = s / bs; return e == 0 ? 2 : e == 1 ? 1 : e == 2 ? 4 : 3; };
+  auto site_of = [&](int j) { return (t0 + j / bs) * Ls + x0 + j % bs; };
+  if (!zero) {
+    for (int q = tid; q < sh.nslot * G * d; q += SC_T) {
+      const int k = q % d, g = (q / d) % G, s = q / (d * G), rhs = r0 + g;
+      if (rhs < nrhs && !(active && !active[rhs]))
+        sx[(s * d + k) * GP + g] = x[rhs * n + (size_t)nbr_site(site_of(slot_site(s)), slot_dir(s), Ls) * d + k];
     }
   }
+  if (STAGE) {
+    for (int e = tid; e < bd * bd; e += SC_T) sinv[(e % bd) * bd + e / bd] = I[e];
+    if (!zero)
+      for (int e = tid; e < sh.nslot * dd; e += SC_T) {
+        const int s = e / dd, r = e - s * dd;
+        sst[s * dd + (r % d) * d + r / d] = st[((size_t)site_of(slot_site(s)) * 5 + slot_dir(s)) * dd + r];
+      }
+  }
+  const int row = tid % bd, grp = tid / bd, j = row / d, i = row - j * d;
+  const bool mine = grp < sh.ng;
+  const int site = site_of(j);
+  C acc[SC_R];
+  bool on[SC_R];
+#pragma unroll
+  for (int b = 0; b < SC_R; ++b) {
+    const int rhs = r0 + grp * SC_R + b;
+    on[b] = mine && rhs < nrhs && !(active && !active[rhs]);
+    acc[b] = on[b] ? f[rhs * n + (size_t)site * d + i] : czero<C>();
+  }
+  __syncthreads();
+  if (mine) {
+    if (!zero) {
+      const int jt = j / bs, jx = j % bs;
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        if (!(e == 0 ? jx == 0 : e == 1 ? jx == bs - 1 : e == 2 ? jt == 0 : jt == bs - 1)) continue;
+        const int s = e * bs + (e < 2 ? jt : jx);
+        const C* w = STAGE ? sst + s * dd + i : st + ((size_t)site * 5 + slot_dir(s)) * dd + (size_t)i * d;
+        const C* xv = sx + s * d * GP + grp * SC_R;
+#pragma unroll 8
+        for (int k = 0; k < d; ++k) {
+          const C m = cneg(STAGE ? w[k * d] : w[k]);
+#pragma unroll
+          for (int b = 0; b < SC_R; ++b) acc[b] = cfma(m, xv[k * GP + b], acc[b]);
+        }
+      }
+    }
+#pragma unroll
+    for (int b = 0; b < SC_R; ++b) sres[row * GP + grp * SC_R + b] = acc[b];
+  }
+  __syncthreads();
+  if (!mine) return;
+#pragma unroll
+  for (int b = 0; b < SC_R; ++b) acc[b] = czero<C>();
+  const C* rv = sres + grp * SC_R;
+#pragma unroll 8
+  for (int c = 0; c < bd; ++c) {
+    const C m = STAGE ? sinv[c * bd + row] : __ldg(I + (size_t)row * bd + c);
+#pragma unroll
+    for (int b = 0; b < SC_R; ++b) acc[b] = cfma(m, rv[c * GP + b], acc[b]);
+  }
+#pragma unroll
+  for (int b = 0; b < SC_R; ++b)
+    if (on[b]) x[(size_t)(r0 + grp * SC_R + b) * n + (size_t)site * d + i] = acc[b];
 }
 
 template <typename R>
 void sap_half_coarse(cudaStream_t stm, const typename CT<R>::T* st, int Ls, int d, int bs,
                      const typename CT<R>::T* inv, const typename CT<R>::T* f, typename CT<R>::T* x, int color,
-                     int nrhs, const int* active) {
+                     int nrhs, const int* active, bool zero) {
   typedef typename CT<R>::T C;
-  const int ns = bs * bs, bd = ns * d;
-  const int G = std::max(1, 256 / bd);
-  size_t sm = sizeof(C) * ((size_t)bd * bd + (size_t)ns * 5 * d * d + (size_t)G * bd);
-  MG_CHECK_ARG(sm <= 220 * 1024, "coarse SAP block too large for shared memory");
-  ensure_max_smem((const void*)k_sap_coarse<R>, 220 * 1024);
+  if (nrhs <= 0) return;
+  const SapCoarseShape sh(bs, d);
+  MG_CHECK_ARG(sh.bd <= 64, "coarse SAP blocks have at most 64 unknowns");
+  const size_t sm = sizeof(C) * (size_t)sh.complexes(sizeof(R) == 4);
   const int nb = (Ls / bs) * (Ls / bs) / 2;
-  const double cs = sizeof(C), ar = act_rhs(nrhs);
-  const double bytes = nb * (ar * 3.0 * bd * cs + ((double)bd * bd + ns * 5.0 * d * d) * cs);
-  const double flops = nb * ar * (8.0 * bd * 5.0 * d + 8.0 * bd * bd);
-  MG_LAUNCH_W(bytes, flops, k_sap_coarse<R>, nb, 256, sm, stm, st, Ls, d, bs, inv, f, x, color, nrhs, active);
+  const double cs = sizeof(C), ar = act_rhs(nrhs), ext = zero ? 0.0 : sh.nslot * (double)d * d;
+  const double bytes = nb * (ar * (zero ? 2.0 : 3.0) * sh.bd * cs + ((double)sh.bd * sh.bd + ext) * cs);
+  const double flops = nb * ar * 8.0 * (ext + (double)sh.bd * sh.bd);
+  const dim3 grid(nb, cdiv(nrhs, sh.G));
+  if (bs == 2 && d == 16) {
+    ensure_max_smem((const void*)k_sap_coarse<R, 2, 16>, 120 * 1024);
+    MG_LAUNCH_W(bytes, flops, (k_sap_coarse<R, 2, 16>), grid, SC_T, sm, stm, st, Ls, d, bs, inv, f, x, color, nrhs,
+                zero, active);
+  } else {
+    ensure_max_smem((const void*)k_sap_coarse<R, 0, 0>, 120 * 1024);
+    MG_LAUNCH_W(bytes, flops, (k_sap_coarse<R, 0, 0>), grid, SC_T, sm, stm, st, Ls, d, bs, inv, f, x, color, nrhs,
+                zero, active);
+  }
 }
 template void sap_half_coarse<float>(cudaStream_t, const float2*, int, int, int, const float2*, const float2*,
-                                     float2*, int, int, const int*);
+                                     float2*, int, int, const int*, bool);
 template void sap_half_coarse<double>(cudaStream_t, const double2*, int, int, int, const double2*,
-                                      const double2*, double2*, int, int, const int*);
+                                      const double2*, double2*, int, int, const int*, bool);
 
 // ---- restriction / prolongation ---------------------------------------------------
 // Aggregate (T, X) of agg x agg sites; block of chirality c has rows

@@ -110,3 +110,17 @@ def test_coarsest_apply_tiles(api, ctx, nrhs, prec, tol):
     xd = torch.empty(b.shape, dtype=torch.from_numpy(b).dtype, device="cuda")
     h.vcycle(top, torch.from_numpy(b).cuda(), xd, getattr(api, prec))
     assert relerr(xd.cpu().numpy(), H.vcycle(top, b.T).T) < tol
+
+
+@pytest.mark.parametrize("prec,tol", [("FP64", 1e-12), ("FP32", 2e-5)])
+@pytest.mark.parametrize("ntv,nrhs", [(4, 1), (4, 17), (8, 8), (8, 9), (1, 33)])
+def test_coarse_smoother_tiles(api, ctx, ntv, nrhs, prec, tol):
+    """SAP sweeps on level 1 on the CUDA cores (2 x 2 blocks of 2, 8 and 16 dof per site), remainders of the rhs tile
+    (tolerances as for the fine smoother: block condition about 10)."""
+    h, H = hierarchy(api, ctx, 64, ntv=ntv)
+    dt = np.complex128 if prec == "FP64" else np.complex64
+    f, x = vecs(H.n[1], nrhs, 1, dt), vecs(H.n[1], nrhs, 2, dt)
+    ref = H.sap(1).sweep(f.T.astype(complex), x.T.astype(complex)).T
+    xd = torch.from_numpy(x).cuda()
+    h.smooth(1, torch.from_numpy(f).cuda(), xd, getattr(api, prec), 1)
+    assert relerr(xd.cpu().numpy(), ref) < tol
