@@ -244,11 +244,14 @@ int mg_tc_status(mgmlmc_ctx* ctx, mgmlmc_hier* h);
 /* In-place inverse of one dense n x n matrix on the device (the coarsest-level
  * direct solve of Section 3.1: tau_L of Algorithm 2 is the trace of D_L^{-1}):
  * Gauss-Jordan elimination with partial pivoting (largest |A_ik|, ties to the
- * smallest row) in one cooperative kernel whose CTAs meet at a grid barrier per
- * column.  A: device, row-major, complex128 (prec MGMLMC_FP64) or complex64
- * (MGMLMC_FP32), 1 <= n <= 8192 (the pivot row is staged in shared memory).
- * barrier_polls: poll limit of every barrier wait (0 = the default, about a
- * second); negative = self-test of the bounded wait: the barrier then waits for
+ * smallest row), by block columns: a cluster eliminates 8 columns, the grid
+ * applies them.  A: device, row-major, complex128 (prec MGMLMC_FP64) or complex64
+ * (MGMLMC_FP32), 1 <= n <= 8192.
+ * barrier_polls: 0 = as above (no software barrier).  Otherwise one cooperative
+ * kernel whose CTAs meet at a grid barrier per column, with the same pivots:
+ * positive = poll limit of every barrier wait (a wait that expires returns
+ * MGMLMC_ERR_TIMEOUT);
+ * negative = self-test of the bounded wait: the barrier then waits for
  * one arrival more than the grid has, so every wait runs out after
  * -barrier_polls polls and the call returns MGMLMC_ERR_TIMEOUT with A left
  * partly eliminated (the kernel stops at the first expired wait; the device

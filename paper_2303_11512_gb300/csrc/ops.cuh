@@ -67,11 +67,12 @@ void dense_from_stencil(cudaStream_t st, const double2* stencil, int Ls, int d, 
 // batched in-place Gauss-Jordan inverse with partial pivoting (one CTA per matrix, bd <= 64), C = double2 / float2
 template <typename C>
 void invert_small_batched(cudaStream_t st, C* A, int nmat, int bd, int* fail);
-// in-place inverse of one n x n matrix (large n), one cooperative kernel; work: invert_large_work_bytes(n);
-// fail set on a zero pivot, timeout on an expired grid barrier; C = double2 / float2
+// in-place inverse of one n x n matrix (large n); work: invert_large_work_bytes(n); fail set on a zero pivot;
+// C = double2 / float2
 size_t invert_large_work_bytes(int n);
-// polls: poll limit of each grid-barrier wait (0 = default, about a second; < 0 = bounded-wait self-test:
-// the barrier expects one arrival more than the grid has, so every wait runs out after -polls polls)
+// polls: 0 = by block columns (n > 32); otherwise one cooperative kernel with a grid barrier per column, > 0: poll
+// limit of each wait (timeout set when one expires), < 0: bounded-wait self-test (the barrier expects one arrival more
+// than the grid has, so every wait runs out after -polls polls)
 template <typename C>
 void invert_large(cudaStream_t st, C* A, int n, int* piv, void* work, int* fail, int* timeout, long polls = 0);
 template <typename R>

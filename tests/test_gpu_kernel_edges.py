@@ -124,3 +124,24 @@ def test_coarse_smoother_tiles(api, ctx, ntv, nrhs, prec, tol):
     xd = torch.from_numpy(x).cuda()
     h.smooth(1, torch.from_numpy(f).cuda(), xd, getattr(api, prec), 1)
     assert relerr(xd.cpu().numpy(), ref) < tol
+
+
+@pytest.mark.parametrize("n", [33, 40, 250, 257, 600])
+@pytest.mark.parametrize("prec,eps", [("FP64", 1.1e-16), ("FP32", 6e-8)])
+def test_dense_inverse_block_columns(api, ctx, n, prec, eps):
+    """Remainders of the 8-column blocks, of the cluster's row shares and of the 32 x 32 update tiles, with a zero
+    leading entry so that rows are swapped from the first column on: A times the inverse is the identity to n
+    roundings amplified by the condition number."""
+    rs = np.random.default_rng(n)
+    A = (rs.standard_normal((n, n)) + 1j * rs.standard_normal((n, n))).astype(
+        np.complex128 if prec == "FP64" else np.complex64)
+    A[0, 0] = 0
+    B = torch.from_numpy(A).cuda()
+    api.mg_dense_inverse(ctx, B, getattr(api, prec))
+    A = A.astype(complex)
+    err = np.abs(B.cpu().numpy() @ A - np.eye(n)).max()
+    assert err < n * eps * np.linalg.cond(A)
+    S = torch.zeros((n, n), dtype=B.dtype, device="cuda")
+    S[0, 1] = S[1, 0] = 1  # singular from the third column on
+    with pytest.raises(Exception):
+        api.mg_dense_inverse(ctx, S, getattr(api, prec))
