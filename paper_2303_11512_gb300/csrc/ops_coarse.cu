@@ -190,7 +190,10 @@ __global__ void __launch_bounds__(SC_T) k_sap_coarse(const typename CT<R>::T* __
   const size_t n = (size_t)Ls * Ls * d;
   const C* I = inv + (size_t)(BT * nbx + BX) * bd * bd;
   // slot: the -x, +x neighbours by row, then the -t, +t neighbours by column; the block's site and direction of each
-  auto slot_site = [&](int s) { const int e = s / bs, i = s - e * bs; return e < 2 ? i * bs + (e ? bs - 1 : 0) : (e == 3 ? (bs - 1) * bs : 0) + i; };
+  auto slot_site = [&](int s) {
+    const int e = s / bs, i = s - e * bs;
+    return e < 2 ? i * bs + (e ? bs - 1 : 0) : (e == 3 ? (bs - 1) * bs : 0) + i;
+  };
   auto slot_dir = [&](int s) { const int e = s / bs; return e == 0 ? 2 : e == 1 ? 1 : e == 2 ? 4 : 3; };
   auto site_of = [&](int j) { return (t0 + j / bs) * Ls + x0 + j % bs; };
   if (!zero) {
@@ -542,8 +545,64 @@ __global__ void k_orthonormalise(double2* __restrict__ P, int nblocks, int bsz, 
   }
 }
 
+// The same for NTV columns with the block in registers: LPB lanes hold four rows each (LPB = bsz / 4: 4 on the fine
+// level, 32 above), so a warp works on 32 / LPB blocks and a dot product takes 16 FMAs and log2(LPB) shuffles of all
+// of them (with one block per warp the FP64 additions of the shuffles were the work: 3.1 ms of the set-up at L = 512).
+template <int NTV, int LPB>
+__global__ void __launch_bounds__(128) k_orthonormalise_reg(double2* __restrict__ P, int nblocks, int* fail) {
+  constexpr int BSZ = 4 * LPB;
+  const int t = blockIdx.x * 128 + threadIdx.x, blk = t / LPB, l = t % LPB;
+  const bool on = blk < nblocks;
+  double2* B = P + (size_t)(on ? blk : 0) * BSZ * NTV;
+  double2 v[NTV][4];  // rows l, l + LPB, ..
+#pragma unroll
+  for (int r = 0; r < 4; ++r)
+#pragma unroll
+    for (int m = 0; m < NTV; ++m) v[m][r] = B[(l + r * LPB) * NTV + m];
+  auto sum = [](double s) {
+#pragma unroll
+    for (int o = LPB / 2; o; o >>= 1) s += __shfl_xor_sync(0xffffffff, s, o);
+    return s;
+  };
+  bool bad = false;
+#pragma unroll
+  for (int m = 0; m < NTV; ++m) {
+#pragma unroll
+    for (int pass = 0; pass < 2; ++pass)
+#pragma unroll
+      for (int i = 0; i < m; ++i) {
+        double2 a = make_double2(0, 0);
+#pragma unroll
+        for (int r = 0; r < 4; ++r) a = cfmac(v[i][r], v[m][r], a);
+        a.x = -sum(a.x);
+        a.y = -sum(a.y);
+#pragma unroll
+        for (int r = 0; r < 4; ++r) v[m][r] = cfma(v[i][r], a, v[m][r]);
+      }
+    double nr = 0;
+#pragma unroll
+    for (int r = 0; r < 4; ++r) nr = fma(v[m][r].x, v[m][r].x, fma(v[m][r].y, v[m][r].y, nr));
+    nr = sum(nr);
+    bad |= !(nr > 0.0);
+    const double inv = 1.0 / sqrt(nr);
+#pragma unroll
+    for (int r = 0; r < 4; ++r) v[m][r] = cscale(v[m][r], inv);
+  }
+  if (!on) return;
+  if (bad && l == 0) atomicExch(fail, 1);
+#pragma unroll
+  for (int r = 0; r < 4; ++r)
+#pragma unroll
+    for (int m = 0; m < NTV; ++m) B[(l + r * LPB) * NTV + m] = v[m][r];
+}
+
 void orthonormalise_blocks(cudaStream_t stm, double2* P, int nblocks, int bsz, int ntv, int* fail) {
-  MG_LAUNCH(k_orthonormalise, cdiv(nblocks, 4), 128, 0, stm, P, nblocks, bsz, ntv, fail);
+  if (ntv == 8 && bsz == 16)
+    MG_LAUNCH((k_orthonormalise_reg<8, 4>), cdiv(nblocks * 4L, 128), 128, 0, stm, P, nblocks, fail);
+  else if (ntv == 8 && bsz == 128)
+    MG_LAUNCH((k_orthonormalise_reg<8, 32>), cdiv(nblocks * 32L, 128), 128, 0, stm, P, nblocks, fail);
+  else
+    MG_LAUNCH(k_orthonormalise, cdiv(nblocks, 4), 128, 0, stm, P, nblocks, bsz, ntv, fail);
 }
 
 // ---- Galerkin coarse operator ------------------------------------------------------
@@ -551,7 +610,9 @@ void orthonormalise_blocks(cudaStream_t stm, double2* P, int nblocks, int bsz, i
 // site s of aggregate B and stencil direction f, with s' the f-neighbour of s,
 //   D_{l+1}[B, f or self] += P(s)^H D_l(s, f) P(s'),
 // where P(s) (d x dc) is block diagonal in chirality and s' lies in B itself or in the aggregate
-// adjacent to B in direction f (a fine hop crosses only the aggregate face it points to).
+// adjacent to B in direction f (a fine hop crosses only the aggregate face it points to).  The products
+// D_l(s, f) P(s') of the directions that stay in B are summed before P(s)^H multiplies them, so a site of a 4 x 4
+// aggregate takes two products with P^H on average instead of five (FP64 is bound by its two FMAs a clock and SM).
 __device__ __forceinline__ void wilson_hop(const double2* __restrict__ lk, double diag, int L, int s, int f,
                                            double2* M) {
   double2 w;
@@ -590,7 +651,7 @@ __global__ void __launch_bounds__(GAL_T) k_galerkin(const double2* __restrict__ 
   const int hd = d / 2, na = agg * agg, bsz = na * hd, dc = 2 * ntv, Lc = Ls / agg;
   const int dd = d * d, ddc = d * dc, dcc = dc * dc;
   double2* sA = reinterpret_cast<double2*>(smem_raw);  // [f][r][k]   D_l(s, f)
-  double2* sT = sA + 5 * dd;                            // [f][r][j]   D_l(s, f) P(s'_f)
+  double2* sT = sA + 5 * dd;                            // [c][r][j]   D_l(s, f) P(s'_f): c = 0 sum inside B, else f = c
   __shared__ int s_nb[5], s_js[5];                      // aggregate and local site of s'_f
   const int B = blockIdx.x, BT = B / Lc, BX = B % Lc;
   const size_t pblk = (size_t)2 * bsz * ntv;
@@ -621,13 +682,37 @@ __global__ void __launch_bounds__(GAL_T) k_galerkin(const double2* __restrict__ 
       for (int e = threadIdx.x; e < 5 * dd; e += GAL_T) sA[e] = __ldg(As + e);
     }
     __syncthreads();
-    for (int e = threadIdx.x; e < 5 * ddc; e += GAL_T) {
-      const int f = e / ddc, rem = e % ddc, r = rem / dc, j = rem % dc, cj = j / ntv, m = j % ntv;
-      const double2* p = P + (size_t)s_nb[f] * pblk + ((size_t)cj * bsz + s_js[f] * hd) * ntv + m;
-      const double2* a = sA + f * dd + r * d + cj * hd;
-      double2 t = make_double2(0, 0);
-      for (int k = 0; k < hd; ++k) t = cfma(a[k], __ldg(p + (size_t)k * ntv), t);
-      sT[e] = t;
+    if (WILSON) {  // few products per site: the five directions in parallel, then the sum
+      for (int e5 = threadIdx.x; e5 < 5 * ddc; e5 += GAL_T) {
+        const int f = e5 / ddc, e = e5 - f * ddc, r = e / dc, j = e % dc, cj = j / ntv, m = j % ntv;
+        const double2* p = P + (size_t)s_nb[f] * pblk + ((size_t)cj * bsz + s_js[f]) * ntv + m;
+        sT[e5] = cmul(sA[f * dd + r * d + cj], __ldg(p));
+      }
+      __syncthreads();
+      for (int e = threadIdx.x; e < ddc; e += GAL_T) {
+        double2 self = sT[e];
+#pragma unroll
+        for (int f = 1; f < 5; ++f)
+          if (inside[f]) self = cadd(self, sT[f * ddc + e]);
+        sT[e] = self;
+      }
+    } else {
+      for (int e = threadIdx.x; e < ddc; e += GAL_T) {
+        const int r = e / dc, j = e % dc, cj = j / ntv, m = j % ntv;
+        double2 self = make_double2(0, 0);
+#pragma unroll
+        for (int f = 0; f < 5; ++f) {
+          const double2* p = P + (size_t)s_nb[f] * pblk + ((size_t)cj * bsz + s_js[f] * hd) * ntv + m;
+          const double2* a = sA + f * dd + r * d + cj * hd;
+          double2 t = inside[f] ? self : make_double2(0, 0);
+          for (int k = 0; k < hd; ++k) t = cfma(a[k], __ldg(p + (size_t)k * ntv), t);
+          if (inside[f])
+            self = t;
+          else
+            sT[f * ddc + e] = t;
+        }
+        sT[e] = self;
+      }
     }
     __syncthreads();
 #pragma unroll
@@ -637,14 +722,10 @@ __global__ void __launch_bounds__(GAL_T) k_galerkin(const double2* __restrict__ 
         const int i = e / dc, j = e % dc, ci = i / ntv, mi = i % ntv;
         const double2* p = PB + ((size_t)ci * bsz + js * hd) * ntv + mi;
 #pragma unroll
-        for (int f = 0; f < 5; ++f) {
-          const double2* t = sT + f * ddc + (ci * hd) * dc + j;
-          double2 v = make_double2(0, 0);
-          for (int k = 0; k < hd; ++k) v = cfmac(__ldg(p + (size_t)k * ntv), t[k * dc], v);
-          if (inside[f])
-            acc[0][q] = cadd(acc[0][q], v);
-          else
-            acc[f][q] = cadd(acc[f][q], v);
+        for (int c = 0; c < 5; ++c) {
+          if (c && inside[c]) continue;
+          const double2* t = sT + c * ddc + (ci * hd) * dc + j;
+          for (int k = 0; k < hd; ++k) acc[c][q] = cfmac(__ldg(p + (size_t)k * ntv), t[k * dc], acc[c][q]);
         }
       }
     }
@@ -658,6 +739,62 @@ __global__ void __launch_bounds__(GAL_T) k_galerkin(const double2* __restrict__ 
   }
 }
 
+// The fine level with 4 x 4 aggregates and dc = 16 (one dof per chirality and site, 256 entries of a block): all 16
+// sites of the aggregate at once, one thread per (site, spin, column) of D P and then one per entry of the blocks.  A
+// site by site pass has 32 such products for 256 threads.  sT[site][c][spin][j]: c = 0 the hops that stay in B, 1 the
+// x hop and 2 the t hop that leave it (a site has at most one of each).
+__global__ void __launch_bounds__(256) k_galerkin_fine4(const double2* __restrict__ lk, double diag, int Ls,
+                                                        const double2* __restrict__ P, double2* __restrict__ out) {
+  constexpr int NTV = 8, DC = 16, BSZ = 16;
+  __shared__ double2 sT[16][3][2][DC];
+  const int Lc = Ls / 4, B = blockIdx.x, BT = B / Lc, BX = B % Lc, tid = threadIdx.x;
+  constexpr size_t PB = (size_t)2 * BSZ * NTV;
+  const int nb[5] = {B, BT * Lc + (BX + 1 == Lc ? 0 : BX + 1), BT * Lc + (BX == 0 ? Lc - 1 : BX - 1),
+                     (BT + 1 == Lc ? 0 : BT + 1) * Lc + BX, (BT == 0 ? Lc - 1 : BT - 1) * Lc + BX};
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+    const int e = tid + q * 256, js = e >> 5, r = (e >> 4) & 1, j = e & 15, cj = j >> 3, m = j & 7;
+    const int jt = js >> 2, jx = js & 3, s = (4 * BT + jt) * Ls + 4 * BX + jx;
+    double2 self = make_double2(0, 0), ox = self, ot = self;
+#pragma unroll
+    for (int f = 0; f < 5; ++f) {
+      double2 M[4];
+      wilson_hop(lk, diag, Ls, s, f, M);
+      const int js2 = f == 0 ? js : f == 1 ? (jx == 3 ? js - 3 : js + 1) : f == 2 ? (jx == 0 ? js + 3 : js - 1)
+                    : f == 3 ? (js + 4) & 15 : (js + 12) & 15;
+      const bool in = f == 0 || (f == 1 ? jx < 3 : f == 2 ? jx > 0 : f == 3 ? jt < 3 : jt > 0);
+      const double2 p = __ldg(P + (size_t)(in ? B : nb[f]) * PB + (cj * BSZ + js2) * NTV + m);
+      const double2 a = r ? (cj ? M[3] : M[2]) : (cj ? M[1] : M[0]);
+      if (in)
+        self = cfma(a, p, self);
+      else if (f <= 2)
+        ox = cfma(a, p, ox);
+      else
+        ot = cfma(a, p, ot);
+    }
+    sT[js][0][r][j] = self;
+    sT[js][1][r][j] = ox;
+    sT[js][2][r][j] = ot;
+  }
+  __syncthreads();
+  const int i = tid >> 4, j = tid & 15, ci = i >> 3, mi = i & 7;
+  const double2* p = P + (size_t)B * PB + ci * BSZ * NTV + mi;
+  double2 acc[5];
+#pragma unroll
+  for (int c = 0; c < 5; ++c) acc[c] = make_double2(0, 0);
+#pragma unroll
+  for (int js = 0; js < 16; ++js) {
+    const double2 pc = __ldg(p + js * NTV);
+    acc[0] = cfmac(pc, sT[js][0][ci][j], acc[0]);
+    if ((js & 3) == 3) acc[1] = cfmac(pc, sT[js][1][ci][j], acc[1]);
+    if ((js & 3) == 0) acc[2] = cfmac(pc, sT[js][1][ci][j], acc[2]);
+    if ((js >> 2) == 3) acc[3] = cfmac(pc, sT[js][2][ci][j], acc[3]);
+    if ((js >> 2) == 0) acc[4] = cfmac(pc, sT[js][2][ci][j], acc[4]);
+  }
+#pragma unroll
+  for (int c = 0; c < 5; ++c) out[((size_t)B * 5 + c) * 256 + tid] = acc[c];
+}
+
 void galerkin(cudaStream_t stm, const double2* A, bool wilson, double diag, int Ls, int d, int agg, int ntv,
               const double2* P, double2* out) {
   const int dc = 2 * ntv, Lc = Ls / agg;
@@ -665,10 +802,12 @@ void galerkin(cudaStream_t stm, const double2* A, bool wilson, double diag, int 
   const size_t sm = sizeof(double2) * 5 * ((size_t)d * d + (size_t)d * dc);
   MG_CHECK_ARG(sm <= 200 * 1024, "Galerkin blocks too large for shared memory");
   const double na = agg * agg, hd = d / 2;
-  const double flops = (double)Lc * Lc * na * 5.0 * 8.0 * hd * ((double)d * dc + (double)dc * dc);
+  const double flops = (double)Lc * Lc * 8.0 * hd * (na * 5.0 * d * dc + (na + 4.0 * agg) * (double)dc * dc);
   const double bytes = (double)Lc * Lc * (na * (wilson ? 32.0 : 5.0 * d * d * 16.0) + 5.0 * dc * dc * 16.0 +
                                           2.0 * na * hd * ntv * 16.0);
-  if (wilson) {
+  if (wilson && agg == 4 && ntv == 8) {
+    MG_LAUNCH_W(bytes, flops, k_galerkin_fine4, Lc * Lc, 256, 0, stm, A, diag, Ls, P, out);
+  } else if (wilson) {
     ensure_max_smem((const void*)k_galerkin<true>, 200 * 1024);
     MG_LAUNCH_W(bytes, flops, k_galerkin<true>, Lc * Lc, GAL_T, sm, stm, A, diag, Ls, d, agg, ntv, P, out);
   } else {

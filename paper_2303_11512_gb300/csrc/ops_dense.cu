@@ -84,12 +84,12 @@ __global__ void __launch_bounds__(256) k_invert_small(C* __restrict__ Ag, int bd
     if (t < bd) {
       if (p != k) A[p * bd + t] = tk;
       A[k * bd + t] = (t == k) ? a : cmul(tp, a);
-      sf[t] = (t == k) ? czero<C>() : (t == p ? akk : ck);
+      sf[t] = (t == k) ? czero<C>() : cneg(t == p ? akk : ck);  // minus the multiplier
     }
     __syncthreads();
     for (int e = threadIdx.x; e < bd * bd; e += 256) {
       const int i = e / bd, j = e - i * bd;
-      if (i != k) A[e] = csub(j == k ? czero<C>() : A[e], cmul(sf[i], A[k * bd + j]));
+      if (i != k) A[e] = cfma(sf[i], A[k * bd + j], j == k ? czero<C>() : A[e]);
     }
     __syncthreads();
   }
@@ -391,7 +391,7 @@ __global__ void __cluster_dims__(GJ_CS, 1, 1) __launch_bounds__(GJ_PT)
         src = i == p ? krow[c] : row[c];
       }
       __syncwarp();
-      if (rr < nrow) row[c] = i == k ? r : c == q ? cneg(cmul(f, r)) : csub(src, cmul(f, r));
+      if (rr < nrow) row[c] = i == k ? r : cfma(cneg(f), r, c == q ? czero<C>() : src);
       __syncwarp();
     }
     __syncthreads();
