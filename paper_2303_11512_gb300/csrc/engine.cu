@@ -108,7 +108,8 @@ void vcycle(mgmlmc_hier* h, int l, const typename CT<R>::T* r, typename CT<R>::T
   }
   const LevelData& Lc = h->lv[l + 1];
   const int pr = sizeof(R) == 8;
-  C* res = (C*)h->work(pr ? "vc_res64" : "vc_res32", l, sizeof(C) * L.n * nrhs);
+  const bool fused = !pr && l == 0 && h->prm.agg == 4 && h->prm.ntv == 8;  // residual and restriction in one kernel
+  C* res = fused ? nullptr : (C*)h->work(pr ? "vc_res64" : "vc_res32", l, sizeof(C) * L.n * nrhs);
   C* rc = (C*)h->work(pr ? "vc_rc64" : "vc_rc32", l, sizeof(C) * Lc.n * nrhs);
   C* ec = (C*)h->work(pr ? "vc_ec64" : "vc_ec32", l, sizeof(C) * Lc.n * nrhs);
   // the 16-bit copy of e that the 2x2-block tensor-core stencil reads, kept up to date by every kernel that
@@ -123,18 +124,22 @@ void vcycle(mgmlmc_hier* h, int l, const typename CT<R>::T* r, typename CT<R>::T
   if (!lazy_zero) vzero<C>(st, e, L.n, nrhs);
   if (e16) MG_CUDA(cudaMemsetAsync(e16, 0, sizeof(uint32_t) * L.n * nrhs, st));
   for (int s = 0; s < h->prm.pre_smooth; ++s) sap_sweep<R>(h, l, r, e, nrhs, active, e16, lazy_zero && s == 0);
-  bool done = false;
+  // after a tensor-core sweep only the colour-0 blocks hold a residual: the restriction reads those alone
+  const bool half = !pr && tc_smoother<R>(h, l) && h->prm.pre_smooth > 0 && h->prm.agg == 4 && h->prm.ntv == 8;
+  bool done = fused;
   if constexpr (sizeof(R) == 4) {
+    if (fused)
+      residual_restrict_fine(st, links_of<R>(L), (R)L.diag, L.side, P_of<R>(L), e, r, rc, nrhs, active);
     if (h->use_tc(l)) {  // res = r - D e on the tensor cores (preconditioner accuracy)
       if (h->prm.pre_smooth > 0 && tc_smoother<R>(h, l))  // zero on the blocks the sweep solved last
-        tc_residual_after_sap(st, L.tcW.p, L.tc_bf, L.side, e, e16, res, r, nrhs, active, h->tc_err.as<int>());
+        tc_residual_after_sap(st, L.tcW.p, L.tc_bf, L.side, e, e16, res, r, nrhs, active, h->tc_err.as<int>(), !half);
       else
         tc_stencil_apply(st, L.tcW.p, L.tc_bf, L.side, e, e16, res, r, nrhs, active, h->tc_err.as<int>());
       done = true;
     }
   }
   if (!done) op_apply<R>(h, l, e, res, r, nrhs, active);  // res = r - D e
-  restrict_op<R>(st, P_of<R>(L), L.side, L.dof, h->prm.agg, h->prm.ntv, res, rc, nrhs, active);
+  if (!fused) restrict_op<R>(st, P_of<R>(L), L.side, L.dof, h->prm.agg, h->prm.ntv, res, rc, nrhs, active, half);
   if (h->prm.kcycle_its > 0 && l + 1 < h->nlev - 1)  // K-cycle: a few FGMRES steps on level l+1
     fgmres_core<R>(h, l + 1, rc, ec, nrhs, h->prm.kcycle_its, h->prm.kcycle_tol, h->prm.kcycle_its, true, active,
                    nullptr, nullptr, nullptr);

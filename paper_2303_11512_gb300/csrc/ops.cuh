@@ -38,6 +38,9 @@ template <typename R>
 void sap_half_fine(cudaStream_t st, const typename CT<R>::T* links, R diag, int L, int bs,
                    const typename CT<R>::T* inv, const typename CT<R>::T* f, typename CT<R>::T* x,
                    int color, int nrhs, const int* active, bool inv_transposed = false, int known = SAP_X);
+// xc = P^H (f - D x) on the fine level for 4 x 4 aggregates and 8 test vectors per chirality
+void residual_restrict_fine(cudaStream_t st, const float2* links, float diag, int L, const float2* P, const float2* x,
+                            const float2* f, float2* xc, int nrhs, const int* active);
 void blocks_to_fp32_transposed(cudaStream_t st, const double2* in, int nb, int bd, float2* out);
 template <typename R>
 void sap_half_coarse(cudaStream_t st, const typename CT<R>::T* stencil, int Ls, int d, int bs,
@@ -48,7 +51,8 @@ void sap_half_coarse(cudaStream_t st, const typename CT<R>::T* stencil, int Ls, 
 // P layout: [aggregate][chirality 2][bsz = agg*agg*d/2][ntv]
 template <typename R>
 void restrict_op(cudaStream_t st, const typename CT<R>::T* P, int Ls, int d, int agg, int ntv,
-                 const typename CT<R>::T* xf, typename CT<R>::T* xc, int nrhs, const int* active);
+                 const typename CT<R>::T* xf, typename CT<R>::T* xc, int nrhs, const int* active,
+                 bool half = false);  // half (d 16): xf zero on the 2 x 2 blocks of colour 1, not read there
 template <typename R>
 void prolong_op(cudaStream_t st, const typename CT<R>::T* P, int Ls, int d, int agg, int ntv,
                 const typename CT<R>::T* xc, typename CT<R>::T* xf, bool add, int nrhs,
@@ -194,9 +198,10 @@ void tc_round16(cudaStream_t st, int bf, const float2* x, void* x16, int nsite, 
 void tc_stencil_apply(cudaStream_t st, const void* W, int bf, int Ls, const float2* x, const void* x16, float2* y,
                       const float2* b, int nrhs, const int* active, int* err);
 // res = f - D x on colour-0 block sites, 0 on colour-1 block sites (the residual right after a SAP sweep: it
-// vanishes on the blocks solved last up to the rounding of the tensor-core products)
+// vanishes on the blocks solved last up to the rounding of the tensor-core products); zero_other false: the latter
+// are not written
 void tc_residual_after_sap(cudaStream_t st, const void* Wst, int bf, int Ls, const float2* x, const void* x16,
-                           float2* res, const float2* f, int nrhs, const int* active, int* err);
+                           float2* res, const float2* f, int nrhs, const int* active, int* err, bool zero_other);
 // one SAP colour half sweep with 2x2-site blocks: res = f - D x on the colour's sites, x_B += inv_B res_B; where
 // tc_block_selected, x16 is read by the residual and updated with x_B (res then holds the 16-bit residual)
 void tc_sap_half(cudaStream_t st, const void* Wst, const void* Winv, int bf, int Ls, const float2* f, float2* x,

@@ -9,9 +9,28 @@
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
+#include <algorithm>
+#include <type_traits>
+
 #include "ops.cuh"
 
 namespace mg {
+
+__device__ __forceinline__ void cp_async16c(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
+}
+// two consecutive complex numbers (16-byte aligned in FP32)
+__device__ __forceinline__ void load2(const float2* p, float2* v) {
+  const float4 q = *reinterpret_cast<const float4*>(p);
+  v[0] = make_float2(q.x, q.y);
+  v[1] = make_float2(q.z, q.w);
+}
+__device__ __forceinline__ void load2(const double2* p, double2* v) { v[0] = p[0]; v[1] = p[1]; }
+__device__ __forceinline__ void store2(float2* p, const float2* v) {
+  *reinterpret_cast<float4*>(p) = make_float4(v[0].x, v[0].y, v[1].x, v[1].y);
+}
+__device__ __forceinline__ void store2(double2* p, const double2* v) { p[0] = v[0]; p[1] = v[1]; }
 
 __device__ __forceinline__ int nbr_site(int s, int dir, int Ls) {
   const int t = s / Ls, x = s - t * Ls;
@@ -396,63 +415,188 @@ __global__ void __launch_bounds__(256) k_prolong(const typename CT<R>::T* __rest
   }
 }
 
-// compile-time shapes of the default hierarchy (agg 4, ntv 8: fine d = 2, coarse d = 16)
-enum { SHAPE_GENERIC = 0, SHAPE_FINE = 1, SHAPE_COARSE = 2 };
-static int transfer_shape(int d, int agg, int ntv) {
-  if (agg == 4 && ntv == 8 && d == 2) return SHAPE_FINE;
-  if (agg == 4 && ntv == 8 && d == 16) return SHAPE_COARSE;
-  return SHAPE_GENERIC;
+// The default hierarchy (4 x 4 aggregates, 8 test vectors per chirality: fine d = 2, coarse d = 16) has kernels of its
+// own below: register tiles instead of one result per thread (whose two shared-memory reads per multiply-add and two
+// barriers per 16 right-hand sides were the time), the sums in the same order.
+
+// xc = P^H xf from a coarse level: 16 outputs x RG right-hand sides per CTA, MM x RR of them per thread, 256 products
+// each.  half: xf is zero on the 2 x 2 blocks of colour 1 (and not read there).
+template <typename R, int RG, int MM, int RR>
+__global__ void __launch_bounds__(16 / MM * (RG / RR))
+    k_restrict16(const typename CT<R>::T* __restrict__ P, int Ls, const typename CT<R>::T* __restrict__ xf,
+                 typename CT<R>::T* __restrict__ xc, bool half, int nrhs, const int* __restrict__ active) {
+  typedef typename CT<R>::T C;
+  constexpr int T = 16 / MM * (RG / RR), XP = 256 + 16 / (int)sizeof(C);
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  C* sP = reinterpret_cast<C*>(smem_raw);  // [chirality][row][vector]
+  C* sx = sP + 2048;                       // [rhs][site][dof]
+  const int Lc = Ls / 4, a = blockIdx.x, AT = a / Lc, AX = a - AT * Lc, r0 = blockIdx.y * RG, tid = threadIdx.x;
+  const size_t n = (size_t)Ls * Ls * 16, nc = (size_t)Lc * Lc * 16;
+  const char* Pa = reinterpret_cast<const char*>(P + (size_t)a * 2048);
+  constexpr int CPS = 16 * (int)sizeof(C) / 16;  // 16-byte chunks of a site
+  for (int q = tid; q < 2048 * (int)sizeof(C) / 16; q += T)
+    cp_async16c(reinterpret_cast<char*>(sP) + q * 16, Pa + q * 16);
+  for (int q = tid; q < RG * 16 * CPS; q += T) {
+    const int c = q % CPS, js = (q / CPS) & 15, g = q / (16 * CPS), rhs = r0 + g;
+    if (rhs < nrhs && !(active && !active[rhs]) && !(half && (((js >> 3) + (js >> 1)) & 1))) {
+      const size_t site = (size_t)(4 * AT + (js >> 2)) * Ls + 4 * AX + (js & 3);
+      cp_async16c(reinterpret_cast<char*>(sx + g * XP + js * 16) + c * 16,
+                  reinterpret_cast<const char*>(xf + rhs * n + site * 16) + c * 16);
+    }
+  }
+  asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;" ::: "memory");
+  __syncthreads();
+  const int op = tid % (16 / MM), o = op * MM, c = o >> 3, m = o & 7, g0 = tid / (16 / MM) * RR;
+  C acc[MM][RR];
+#pragma unroll
+  for (int u = 0; u < MM; ++u)
+#pragma unroll
+    for (int b = 0; b < RR; ++b) acc[u][b] = czero<C>();
+  for (int js = 0; js < 16; ++js) {
+    if (half && (((js >> 3) + (js >> 1)) & 1)) continue;
+    const C* p = sP + (c * 128 + js * 8) * 8 + m;
+    const C* v = sx + g0 * XP + js * 16 + c * 8;
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+#pragma unroll
+      for (int u = 0; u < MM; ++u) {
+        const C pv = p[k * 8 + u];
+#pragma unroll
+        for (int b = 0; b < RR; ++b) acc[u][b] = cfmac(pv, v[b * XP + k], acc[u][b]);
+      }
+  }
+#pragma unroll
+  for (int b = 0; b < RR; ++b) {
+    const int rhs = r0 + g0 + b;
+    if (rhs < nrhs && !(active && !active[rhs]))
+#pragma unroll
+      for (int u = 0; u < MM; ++u) xc[rhs * nc + (size_t)a * 16 + o + u] = acc[u][b];
+  }
+}
+
+// xf (+)= P xc.  A thread keeps the rows of P of its two consecutive dofs in registers (D = 16: one chirality; D = 2:
+// both spins of a site) and takes the right-hand sides of the tile in turn; xc comes from shared memory.  D = 16 with
+// xf16: the planar 16-bit copy is written alongside.
+template <typename R, bool ADD, int D, int RG>
+__global__ void __launch_bounds__(128) k_prolong2(const typename CT<R>::T* __restrict__ P, int Ls,
+                                                  const typename CT<R>::T* __restrict__ xc,
+                                                  typename CT<R>::T* __restrict__ xf, unsigned short* __restrict__ xf16,
+                                                  int bf, int nrhs, const int* __restrict__ active) {
+  typedef typename CT<R>::T C;
+  constexpr int PAIRS = 8 * D, RS = 128 / PAIRS;  // dof pairs of an aggregate, rhs taken at once
+  constexpr int ROWS = 8 * D;                     // rows of a chirality block
+  __shared__ __align__(16) C sc[RG][16];
+  const int Lc = Ls / 4, a = blockIdx.x, AT = a / Lc, AX = a - AT * Lc, r0 = blockIdx.y * RG, tid = threadIdx.x;
+  const size_t n = (size_t)Ls * Ls * D, nc = (size_t)Lc * Lc * 16;
+  for (int q = tid; q < RG * 16; q += 128) {
+    const int g = q >> 4, rhs = r0 + g;
+    if (rhs < nrhs && !(active && !active[rhs])) sc[g][q & 15] = __ldg(xc + rhs * nc + (size_t)a * 16 + (q & 15));
+  }
+  const int pr = tid % PAIRS, js = pr / (D / 2), k = 2 * (pr % (D / 2)), rs = tid / PAIRS;
+  const int c0 = D == 2 ? 0 : k >> 3, c1 = D == 2 ? 1 : c0;
+  const C* Pa = P + (size_t)a * 2 * ROWS * 8;
+  const C* p0 = Pa + (c0 * ROWS + (D == 2 ? js : js * 8 + (k & 7))) * 8;
+  const C* p1 = Pa + (c1 * ROWS + (D == 2 ? js : js * 8 + (k & 7) + 1)) * 8;
+  C w[2][8];
+#pragma unroll
+  for (int m = 0; m < 8; ++m) {
+    w[0][m] = __ldg(p0 + m);
+    w[1][m] = __ldg(p1 + m);
+  }
+  const size_t off = ((size_t)(4 * AT + (js >> 2)) * Ls + 4 * AX + (js & 3)) * D + k;
+  __syncthreads();
+#pragma unroll 4
+  for (int g = rs; g < RG; g += RS) {
+    const int rhs = r0 + g;
+    if (rhs >= nrhs || (active && !active[rhs])) continue;
+    C* px = xf + rhs * n + off;
+    C v[2], acc[2];
+    if (ADD) load2(px, v);
+    acc[0] = acc[1] = czero<C>();
+#pragma unroll
+    for (int m = 0; m < 8; ++m) {
+      acc[0] = cfma(w[0][m], sc[g][c0 * 8 + m], acc[0]);
+      acc[1] = cfma(w[1][m], sc[g][c1 * 8 + m], acc[1]);
+    }
+#pragma unroll
+    for (int u = 0; u < 2; ++u) v[u] = ADD ? cadd(v[u], acc[u]) : acc[u];
+    store2(px, v);
+    if constexpr (sizeof(R) == 4 && D == 16) {
+      if (xf16) {  // Re parts of the site's 16 dofs, then the Im parts
+        unsigned* p16 = reinterpret_cast<unsigned*>(xf16 + 2 * (rhs * n + off - k) + k);
+        auto pack = [&](float x, float y) {
+          auto b16 = [&](float f) -> unsigned {
+            return bf == 2 ? __half_as_ushort(__float2half_rn(f)) : __bfloat16_as_ushort(__float2bfloat16_rn(f));
+          };
+          return b16(x) | b16(y) << 16;
+        };
+        p16[0] = pack(v[0].x, v[1].x);
+        p16[8] = pack(v[0].y, v[1].y);
+      }
+    }
+  }
 }
 
 template <typename R>
 void restrict_op(cudaStream_t stm, const typename CT<R>::T* P, int Ls, int d, int agg, int ntv,
-                 const typename CT<R>::T* xf, typename CT<R>::T* xc, int nrhs, const int* active) {
+                 const typename CT<R>::T* xf, typename CT<R>::T* xc, int nrhs, const int* active, bool half) {
   typedef typename CT<R>::T C;
+  if (nrhs <= 0) return;
   const int na = agg * agg, bsz = na * d / 2, dc = 2 * ntv;
-  const int G = std::max(1, 256 / dc);
-  size_t sm = sizeof(C) * ((size_t)2 * bsz * ntv + (size_t)G * na * d);
   const int Lc = Ls / agg;
   const double nag = (double)Lc * Lc, cs = sizeof(C), ar = act_rhs(nrhs);
-  const double bytes = nag * (ar * (na * d + dc) * cs + 2.0 * bsz * ntv * cs);
-  const double flops = nag * ar * 8.0 * 2.0 * bsz * ntv;
-  switch (transfer_shape(d, agg, ntv)) {
-    case SHAPE_FINE:
-      set_smem_attr(k_restrict<R, 2, 4, 8>);
-      MG_LAUNCH_W(bytes, flops, (k_restrict<R, 2, 4, 8>), Lc * Lc, 256, sm, stm, P, Ls, d, agg, ntv, xf, xc, nrhs,
-                  active);
-      break;
-    case SHAPE_COARSE:
-      set_smem_attr(k_restrict<R, 16, 4, 8>);
-      MG_LAUNCH_W(bytes, flops, (k_restrict<R, 16, 4, 8>), Lc * Lc, 256, sm, stm, P, Ls, d, agg, ntv, xf, xc, nrhs,
-                  active);
-      break;
-    default:
-      set_smem_attr(k_restrict<R, 0, 0, 0>);
-      MG_LAUNCH_W(bytes, flops, (k_restrict<R, 0, 0, 0>), Lc * Lc, 256, sm, stm, P, Ls, d, agg, ntv, xf, xc, nrhs,
-                  active);
+  const double bytes = nag * (ar * (na * d * (half ? 0.5 : 1.0) + dc) * cs + 2.0 * bsz * ntv * cs);
+  const double flops = nag * ar * 8.0 * 2.0 * bsz * ntv * (half ? 0.5 : 1.0);
+  const bool aligned = ((uintptr_t)xf & 15) == 0;  // 16-byte copies; other vectors take the general kernel
+  if (agg == 4 && ntv == 8 && d == 16 && aligned) {
+    // FP32 2 x 2 results a thread (two 16-byte and two 8-byte reads for 16 FMAs), FP64 one (its units are the bound)
+    constexpr int RG = sizeof(R) == 4 ? 16 : 8, MM = sizeof(R) == 4 ? 2 : 1;
+    constexpr int T = 16 / MM * (RG / MM), sm = (int)sizeof(C) * (2048 + RG * (256 + 16 / (int)sizeof(C)));
+    ensure_max_smem((const void*)k_restrict16<R, RG, MM, MM>, sm);
+    MG_LAUNCH_W(bytes, flops, (k_restrict16<R, RG, MM, MM>), dim3(Lc * Lc, cdiv(nrhs, RG)), T, sm, stm, P, Ls, xf, xc,
+                half, nrhs, active);
+    return;
+  }
+  MG_CHECK_ARG(!half, "half restriction: 4 x 4 aggregates of 16 dof, aligned vectors");
+  const int G = std::max(1, 256 / dc);
+  const size_t sm = sizeof(C) * ((size_t)2 * bsz * ntv + (size_t)G * na * d);
+  if (agg == 4 && ntv == 8 && d == 2) {
+    set_smem_attr(k_restrict<R, 2, 4, 8>);
+    MG_LAUNCH_W(bytes, flops, (k_restrict<R, 2, 4, 8>), Lc * Lc, 256, sm, stm, P, Ls, d, agg, ntv, xf, xc, nrhs,
+                active);
+  } else {
+    set_smem_attr(k_restrict<R, 0, 0, 0>);
+    MG_LAUNCH_W(bytes, flops, (k_restrict<R, 0, 0, 0>), Lc * Lc, 256, sm, stm, P, Ls, d, agg, ntv, xf, xc, nrhs,
+                active);
   }
 }
 
 template <typename R, bool ADD>
 static void prolong_launch(cudaStream_t stm, const typename CT<R>::T* P, int Ls, int d, int agg, int ntv,
                            const typename CT<R>::T* xc, typename CT<R>::T* xf, unsigned short* xf16, int bf,
-                           int nrhs, const int* active, size_t sm, double bytes, double flops) {
+                           int nrhs, const int* active, double bytes, double flops) {
+  typedef typename CT<R>::T C;
   const int Lc = Ls / agg;
-  switch (transfer_shape(d, agg, ntv)) {
-    case SHAPE_FINE:
-      set_smem_attr(k_prolong<R, ADD, 2, 4, 8>);
-      MG_LAUNCH_W(bytes, flops, (k_prolong<R, ADD, 2, 4, 8>), Lc * Lc, 256, sm, stm, P, Ls, d, agg, ntv, xc, xf,
-                  xf16, bf, nrhs, active);
-      break;
-    case SHAPE_COARSE:
-      set_smem_attr(k_prolong<R, ADD, 16, 4, 8>);
-      MG_LAUNCH_W(bytes, flops, (k_prolong<R, ADD, 16, 4, 8>), Lc * Lc, 256, sm, stm, P, Ls, d, agg, ntv, xc, xf,
-                  xf16, bf, nrhs, active);
-      break;
-    default:
-      set_smem_attr(k_prolong<R, ADD, 0, 0, 0>);
-      MG_LAUNCH_W(bytes, flops, (k_prolong<R, ADD, 0, 0, 0>), Lc * Lc, 256, sm, stm, P, Ls, d, agg, ntv, xc, xf,
-                  xf16, bf, nrhs, active);
+  auto go = [&](auto dd, auto rg) {
+    constexpr int D = decltype(dd)::value, RG = decltype(rg)::value;
+    MG_LAUNCH_W(bytes, flops, (k_prolong2<R, ADD, D, RG>), dim3(Lc * Lc, cdiv(nrhs, RG)), 128, 0, stm, P, Ls, xc, xf,
+                xf16, bf, nrhs, active);
+  };
+  typedef std::integral_constant<int, 8> I8;
+  typedef std::integral_constant<int, 32> I32;
+  const bool aligned = ((uintptr_t)xf & 15) == 0;  // 16-byte accesses; other vectors take the general kernel
+  if (agg == 4 && ntv == 8 && d == 2 && aligned) {
+    nrhs <= 8 ? go(std::integral_constant<int, 2>(), I8()) : go(std::integral_constant<int, 2>(), I32());
+  } else if (agg == 4 && ntv == 8 && d == 16 && aligned) {
+    // few aggregates: tiles of 8 rhs spread a batch over more CTAs
+    nrhs <= 8 || Lc * Lc * cdiv(nrhs, 32) < 152 * 4 ? go(std::integral_constant<int, 16>(), I8())
+                                                   : go(std::integral_constant<int, 16>(), I32());
+  } else {
+    const int na = agg * agg, bsz = na * d / 2, dc = 2 * ntv, G = std::max(1, 256 / (na * d));
+    const size_t sm = sizeof(C) * ((size_t)2 * bsz * ntv + (size_t)G * dc);
+    set_smem_attr(k_prolong<R, ADD, 0, 0, 0>);
+    MG_LAUNCH_W(bytes, flops, (k_prolong<R, ADD, 0, 0, 0>), Lc * Lc, 256, sm, stm, P, Ls, d, agg, ntv, xc, xf,
+                xf16, bf, nrhs, active);
   }
 }
 
@@ -462,9 +606,8 @@ void prolong_op(cudaStream_t stm, const typename CT<R>::T* P, int Ls, int d, int
                 void* xf16, int bf) {
   MG_CHECK_ARG(!xf16 || (sizeof(R) == 4 && (bf == 1 || bf == 2)), "16-bit copy: FP32 vectors, BF16 or FP16");
   typedef typename CT<R>::T C;
+  if (nrhs <= 0) return;
   const int na = agg * agg, bsz = na * d / 2, dc = 2 * ntv, fa = na * d;
-  const int G = std::max(1, 256 / fa);
-  size_t sm = sizeof(C) * ((size_t)2 * bsz * ntv + (size_t)G * dc);
   const int Lc = Ls / agg;
   const double nag = (double)Lc * Lc, cs = sizeof(C), ar = act_rhs(nrhs);
   const double bytes = nag * (ar * ((add ? 2.0 : 1.0) * fa + dc) * cs + 2.0 * bsz * ntv * cs) +
@@ -472,14 +615,14 @@ void prolong_op(cudaStream_t stm, const typename CT<R>::T* P, int Ls, int d, int
   const double flops = nag * ar * 8.0 * 2.0 * bsz * ntv;
   unsigned short* x16 = (unsigned short*)xf16;
   if (add)
-    prolong_launch<R, true>(stm, P, Ls, d, agg, ntv, xc, xf, x16, bf, nrhs, active, sm, bytes, flops);
+    prolong_launch<R, true>(stm, P, Ls, d, agg, ntv, xc, xf, x16, bf, nrhs, active, bytes, flops);
   else
-    prolong_launch<R, false>(stm, P, Ls, d, agg, ntv, xc, xf, x16, bf, nrhs, active, sm, bytes, flops);
+    prolong_launch<R, false>(stm, P, Ls, d, agg, ntv, xc, xf, x16, bf, nrhs, active, bytes, flops);
 }
 template void restrict_op<float>(cudaStream_t, const float2*, int, int, int, int, const float2*, float2*, int,
-                                 const int*);
+                                 const int*, bool);
 template void restrict_op<double>(cudaStream_t, const double2*, int, int, int, int, const double2*, double2*, int,
-                                  const int*);
+                                  const int*, bool);
 template void prolong_op<float>(cudaStream_t, const float2*, int, int, int, int, const float2*, float2*, bool, int,
                                 const int*, void*, int);
 template void prolong_op<double>(cudaStream_t, const double2*, int, int, int, int, const double2*, double2*, bool,

@@ -257,25 +257,29 @@ __device__ __forceinline__ void cp_async8(void* dst, const void* src) {
 // other 64 bytes).  Half sweep at L = 512: 100 us with 32 rhs, 56 with 16, 37 with 8.  Measured at 32 rhs and left:
 // loads to registers at the start of an item 147 us (global latency); one row and 8 rhs per thread (72 bytes for 32
 // FMAs) 130 us whatever the occupancy, prefetch depth or packing of the FMAs.  The sums run over the columns in order.
-template <int RG>
+// With RESTRICT the items are all aggregates (4 x 4 sites as well), `inv` holds the prolongator blocks and `out` the
+// coarse vectors: xc_a = P_a^H (f - D x)_a, the residual never leaves the SM (residual and restriction in one: 185 ->
+// 123 us at L = 512, 32 rhs).
+template <int RG, bool RESTRICT>
 struct SapF {
   static constexpr int RP = RG + 1;  // padded row: 8 sites of one rhs hit distinct banks in the final update
   float4 f[16 * RG];
   float4 x[32 * RP];    // block sites, then the sites around it: -x, +x (by row), -t, +t (by column)
-  float2 inv[32 * 32];  // transposed: row j holds column j of the inverse
+  float2 inv[RESTRICT ? 256 : 1024];  // transposed: row j holds column j of the inverse; P: [chirality][site][vector]
   float2 lx[20];        // x links of sites (row, -1 .. 3)
   float2 lt[20];        // t links of sites (-1 .. 3, column)
 };
 
-template <int RG>
+template <int RG, bool RESTRICT>
 __global__ void __launch_bounds__(64) k_sap_fine4_fp32(const float2* __restrict__ lk, float diag, int L,
                                                        const float2* __restrict__ inv, const float2* __restrict__ f,
-                                                       float2* __restrict__ x, int color, int nrhs, int nitems,
+                                                       const float2* x, float2* out, int color, int nrhs, int nitems,
                                                        int known, const int* __restrict__ active) {
-  constexpr int RP = SapF<RG>::RP, T = 64, NR = RG / 8, RSTEP = T / (4 * RG) ? T / (4 * RG) : 1;
+  typedef SapF<RG, RESTRICT> S;
+  constexpr int RP = S::RP, T = 64, NR = RG / 8, RSTEP = T / (4 * RG) ? T / (4 * RG) : 1;
   constexpr int RTH = T / 4 < RG ? T / 4 : RG;  // rhs that the CTA's threads fetch at once
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  SapF<RG>& s = *reinterpret_cast<SapF<RG>*>(smem_raw);
+  S& s = *reinterpret_cast<S*>(smem_raw);
   const int tid = threadIdx.x, lane = tid & 31;
   const int nbx = L / 4, half = nbx / 2, r0 = blockIdx.y * RG;
   const size_t n = 2 * (size_t)L * L;
@@ -285,13 +289,15 @@ __global__ void __launch_bounds__(64) k_sap_fine4_fp32(const float2* __restrict_
   const int fj = tid & 3, frr = (tid >> 2) % RTH, fi = (tid >> 2) / RTH;
   const int g = tid & 7, rg = tid >> 3;  // row group and rhs group of the product
   for (int item = blockIdx.x; item < nitems; item += gridDim.x) {
-    const int BT = item / half, t0 = 4 * BT, x0 = 4 * (2 * (item - BT * half) + ((BT + color) & 1));
+    const int BT = RESTRICT ? item / nbx : item / half, t0 = 4 * BT;
+    const int x0 = RESTRICT ? 4 * (item - BT * nbx) : 4 * (2 * (item - BT * half) + ((BT + color) & 1));
     const int tm = t0 == 0 ? L - 1 : t0 - 1, tp = t0 + 4 == L ? 0 : t0 + 4;
     const int xm = x0 == 0 ? L - 1 : x0 - 1, xp = x0 + 4 == L ? 0 : x0 + 4;
     {
-      const char* I = reinterpret_cast<const char*>(inv + (size_t)(BT * nbx + x0 / 4) * 1024);
+      constexpr int NI = RESTRICT ? 256 : 1024;
+      const char* I = reinterpret_cast<const char*>(inv + (size_t)(BT * nbx + x0 / 4) * NI);
 #pragma unroll
-      for (int q = 0; q < 512 / T; ++q)
+      for (int q = 0; q < NI / 2 / T; ++q)
         cp_async16(reinterpret_cast<char*>(s.inv) + (tid + q * T) * 16, I + (tid + q * T) * 16);
       if (tid < 20) {
         const int i = tid / 5, j = tid - 5 * i;
@@ -364,45 +370,63 @@ __global__ void __launch_bounds__(64) k_sap_fine4_fp32(const float2* __restrict_
       }
       __syncthreads();
     }
-    float2 acc[4][NR];
+    if constexpr (RESTRICT) {  // 16 coarse dofs (chirality, vector) x RG rhs: 4 threads per dof, RG / 4 rhs each
+      constexpr int RQ = RG / 4;
+      const int o = tid & 15, c = o >> 3, m = o & 7, q0 = (tid >> 4) * RQ;
+      float2 acc[RQ];
 #pragma unroll
-    for (int a = 0; a < 4; ++a)
+      for (int b = 0; b < RQ; ++b) acc[b] = make_float2(0.f, 0.f);
 #pragma unroll
-      for (int b = 0; b < NR; ++b) acc[a][b] = make_float2(0.f, 0.f);
+      for (int j = 0; j < 16; ++j) {
+        const float2 p = s.inv[(c * 16 + j) * 8 + m];
+#pragma unroll
+        for (int b = 0; b < RQ; ++b)
+          acc[b] = cfmac(p, reinterpret_cast<const float2*>(&s.f[j * RG + q0 + b])[c], acc[b]);
+      }
+#pragma unroll
+      for (int b = 0; b < RQ; ++b)
+        if ((live_mask >> (q0 + b)) & 1) out[(size_t)(r0 + q0 + b) * (n / 2) + 16 * (size_t)item + o] = acc[b];
+    } else {
+      float2 acc[4][NR];
+#pragma unroll
+      for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int b = 0; b < NR; ++b) acc[a][b] = make_float2(0.f, 0.f);
 #pragma unroll 2
-    for (int j = 0; j < 16; ++j) {
-      float4 v[NR];
+      for (int j = 0; j < 16; ++j) {
+        float4 v[NR];
 #pragma unroll
-      for (int b = 0; b < NR; ++b) v[b] = s.f[j * RG + rg * NR + b];
+        for (int b = 0; b < NR; ++b) v[b] = s.f[j * RG + rg * NR + b];
 #pragma unroll
-      for (int sp = 0; sp < 2; ++sp) {
-        const float4* mi = reinterpret_cast<const float4*>(s.inv + (2 * j + sp) * 32);
-        const float4 m0 = mi[g], m1 = mi[8 + g];  // rows 2g, 2g + 1 and 16 + 2g, 17 + 2g
+        for (int sp = 0; sp < 2; ++sp) {
+          const float4* mi = reinterpret_cast<const float4*>(s.inv + (2 * j + sp) * 32);
+          const float4 m0 = mi[g], m1 = mi[8 + g];  // rows 2g, 2g + 1 and 16 + 2g, 17 + 2g
 #pragma unroll
-        for (int b = 0; b < NR; ++b) {
-          const float2 w = sp ? make_float2(v[b].z, v[b].w) : make_float2(v[b].x, v[b].y);
-          acc[0][b] = cfma(make_float2(m0.x, m0.y), w, acc[0][b]);
-          acc[1][b] = cfma(make_float2(m0.z, m0.w), w, acc[1][b]);
-          acc[2][b] = cfma(make_float2(m1.x, m1.y), w, acc[2][b]);
-          acc[3][b] = cfma(make_float2(m1.z, m1.w), w, acc[3][b]);
+          for (int b = 0; b < NR; ++b) {
+            const float2 w = sp ? make_float2(v[b].z, v[b].w) : make_float2(v[b].x, v[b].y);
+            acc[0][b] = cfma(make_float2(m0.x, m0.y), w, acc[0][b]);
+            acc[1][b] = cfma(make_float2(m0.z, m0.w), w, acc[1][b]);
+            acc[2][b] = cfma(make_float2(m1.x, m1.y), w, acc[2][b]);
+            acc[3][b] = cfma(make_float2(m1.z, m1.w), w, acc[3][b]);
+          }
         }
       }
-    }
-    const int site = (t0 + (g >> 2)) * L + x0 + (g & 3);
-    float2* xo = x + (size_t)(r0 + rg * NR) * n;
+      const int site = (t0 + (g >> 2)) * L + x0 + (g & 3);
+      float2* xo = out + (size_t)(r0 + rg * NR) * n;
 #pragma unroll
-    for (int b = 0; b < NR; ++b) {
-      const int rr = rg * NR + b;
-      if ((live_mask >> rr) & 1) {
-        if (known == SAP_X) {
-          const float4 p = s.x[g * RP + rr], q = s.x[(8 + g) * RP + rr];
-          acc[0][b] = cadd(make_float2(p.x, p.y), acc[0][b]);
-          acc[1][b] = cadd(make_float2(p.z, p.w), acc[1][b]);
-          acc[2][b] = cadd(make_float2(q.x, q.y), acc[2][b]);
-          acc[3][b] = cadd(make_float2(q.z, q.w), acc[3][b]);
+      for (int b = 0; b < NR; ++b) {
+        const int rr = rg * NR + b;
+        if ((live_mask >> rr) & 1) {
+          if (known == SAP_X) {
+            const float4 p = s.x[g * RP + rr], q = s.x[(8 + g) * RP + rr];
+            acc[0][b] = cadd(make_float2(p.x, p.y), acc[0][b]);
+            acc[1][b] = cadd(make_float2(p.z, p.w), acc[1][b]);
+            acc[2][b] = cadd(make_float2(q.x, q.y), acc[2][b]);
+            acc[3][b] = cadd(make_float2(q.z, q.w), acc[3][b]);
+          }
+          st_sp(xo + (size_t)b * n, site, acc[0][b], acc[1][b]);
+          st_sp(xo + (size_t)b * n, site + 2 * L, acc[2][b], acc[3][b]);
         }
-        st_sp(xo + (size_t)b * n, site, acc[0][b], acc[1][b]);
-        st_sp(xo + (size_t)b * n, site + 2 * L, acc[2][b], acc[3][b]);
       }
     }
     __syncthreads();  // the stage is refilled next
@@ -565,12 +589,13 @@ void sap_half_fine(cudaStream_t st, const typename CT<R>::T* links, R diag, int 
     // tile of right-hand sides: 8 where that takes the batch, else 16.  A tile of 32 needs fewer reads of the
     // inverse per FMA but leaves 6 CTAs per SM instead of 10: 115 us against 100 at L = 512, 32 rhs.
     auto go = [&](auto rg) {
-      constexpr int RG = decltype(rg)::value, sm = (int)sizeof(SapF<RG>), per_sm = std::min(16, 227 * 1024 / (sm + 1024));
+      constexpr int RG = decltype(rg)::value, sm = (int)sizeof(SapF<RG, false>);
+      constexpr int per_sm = std::min(16, 227 * 1024 / (sm + 1024));
       const int ntile = (nrhs + RG - 1) / RG;
       const dim3 grid(std::max(1, std::min(nb, (nsm * per_sm + ntile - 1) / ntile)), ntile);
-      ensure_max_smem((const void*)k_sap_fine4_fp32<RG>, sm);
-      MG_LAUNCH_W(bytes, flops, k_sap_fine4_fp32<RG>, grid, 64, sm, st, links, diag, L, inv, f, x, color, nrhs, nb,
-                  known, active);
+      ensure_max_smem((const void*)k_sap_fine4_fp32<RG, false>, sm);
+      MG_LAUNCH_W(bytes, flops, (k_sap_fine4_fp32<RG, false>), grid, 64, sm, st, links, diag, L, inv, f, x, x, color,
+                  nrhs, nb, known, active);
     };
     if (nrhs <= 8)
       go(std::integral_constant<int, 8>());
@@ -594,6 +619,31 @@ template void sap_half_fine<float>(cudaStream_t, const float2*, float, int, int,
                                    float2*, int, int, const int*, bool, int);
 template void sap_half_fine<double>(cudaStream_t, const double2*, double, int, int, const double2*,
                                     const double2*, double2*, int, int, const int*, bool, int);
+
+void residual_restrict_fine(cudaStream_t st, const float2* links, float diag, int L, const float2* P, const float2* x,
+                            const float2* f, float2* xc, int nrhs, const int* active) {
+  MG_CHECK_ARG(L % 4 == 0, "4 x 4 aggregates");
+  if (nrhs <= 0) return;
+  const int na = (L / 4) * (L / 4);
+  const double ar = act_rhs(nrhs);
+  const double bytes = na * (ar * (16 * 16 * 2 + 128.0) + 2048.0), flops = na * ar * (16 * 56.0 + 8.0 * 256);
+  int dev = 0, nsm = 152;
+  MG_CUDA(cudaGetDevice(&dev));
+  MG_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+  auto go = [&](auto rg) {
+    constexpr int RG = decltype(rg)::value, sm = (int)sizeof(SapF<RG, true>);
+    constexpr int per_sm = std::min(16, 227 * 1024 / (sm + 1024));
+    const int ntile = (nrhs + RG - 1) / RG;
+    const dim3 grid(std::max(1, std::min(na, (nsm * per_sm + ntile - 1) / ntile)), ntile);
+    ensure_max_smem((const void*)k_sap_fine4_fp32<RG, true>, sm);
+    MG_LAUNCH_W(bytes, flops, (k_sap_fine4_fp32<RG, true>), grid, 64, sm, st, links, diag, L, P, f, x, xc, 0, nrhs, na,
+                SAP_X, active);
+  };
+  if (nrhs <= 8)
+    go(std::integral_constant<int, 8>());
+  else
+    go(std::integral_constant<int, 16>());
+}
 
 // out[b][j][i] = (float) in[b][i][j] for nb blocks of bd x bd
 __global__ void k_blocks_to_fp32_transposed(const double2* __restrict__ in, int nb, int bd, float2* __restrict__ out) {

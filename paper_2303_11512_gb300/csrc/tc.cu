@@ -671,14 +671,15 @@ __global__ void k_zero_colour_blocks(float2* __restrict__ res, int Ls, int color
   }
 }
 
-// res = f - D x on the sites of the colour-0 blocks and 0 on the colour-1 blocks: the V-cycle residual after
+// res = f - D x on the sites of the colour-0 blocks and 0 on the colour-1 blocks (left as they are where the caller
+// does not read them: zero_other false): the V-cycle residual after
 // a SAP sweep whose last half sweep solved the colour-1 blocks.  The blocks of one colour do not couple to each
 // other, so with exact block solves f - D x would vanish on them; here the block inverses, the residual feeding
 // them and the stored x are TF32/BF16/FP16-accurate, so the residual that is set to zero is of the order of that
 // format's rounding times |f - D x|.  Dropping it perturbs the preconditioner only: the outer flexible Krylov
 // iteration and the FP64 true-residual refinement still converge to the requested residual.
 void tc_residual_after_sap(cudaStream_t st, const void* Wst, int bf, int Ls, const float2* x, const void* x16,
-                           float2* res, const float2* f, int nrhs, const int* active, int* err) {
+                           float2* res, const float2* f, int nrhs, const int* active, int* err, bool zero_other) {
   if (nrhs <= 0) return;
   const int ns = Ls * Ls;
   const double ar = act_rhs(nrhs);
@@ -692,7 +693,8 @@ void tc_residual_after_sap(cudaStream_t st, const void* Wst, int bf, int Ls, con
     launch_tc_fmt<0>(bf, st, x, Wst, (float*)res, (const float*)f, Ls, ns / 2, 1, 0, nrhs, active, err, bytes,
                      flops);
   }
-  MG_LAUNCH_W(ar * (ns / 2) * 128.0, 0, k_zero_colour_blocks, 1024, 256, 0, st, res, Ls, 1, nrhs, active);
+  if (zero_other)
+    MG_LAUNCH_W(ar * (ns / 2) * 128.0, 0, k_zero_colour_blocks, 1024, 256, 0, st, res, Ls, 1, nrhs, active);
 }
 
 void tc_sap_half(cudaStream_t st, const void* Wst, const void* Winv, int bf, int Ls, const float2* f, float2* x,

@@ -145,3 +145,37 @@ def test_dense_inverse_block_columns(api, ctx, n, prec, eps):
     S[0, 1] = S[1, 0] = 1  # singular from the third column on
     with pytest.raises(Exception):
         api.mg_dense_inverse(ctx, S, getattr(api, prec))
+
+
+@pytest.mark.parametrize("prec,tol", [("FP64", 1e-13), ("FP32", 5e-6)])
+@pytest.mark.parametrize("nrhs", [1, 8, 9, 33])
+@pytest.mark.parametrize("shift", [0, 1])
+def test_transfer_tiles(api, ctx, nrhs, prec, tol, shift):
+    """Restriction and prolongation of both levels (2 and 16 dof) at the remainders of the rhs tiles, and on vectors
+    that start 8 bytes off a 16-byte boundary in FP32 (up to 256 products, roundings of order eps each)."""
+    h, H = hierarchy(api, ctx, 64, ntv=8)
+    dt = np.complex128 if prec == "FP64" else np.complex64
+    for l in range(2):
+        xf, xc = vecs(H.n[l], nrhs, 1, dt), vecs(H.n[l + 1], nrhs, 2, dt)
+        def off(a):
+            buf = torch.empty(a.size + shift, dtype=torch.from_numpy(a).dtype, device="cuda")
+            v = buf[shift:].view(a.shape)
+            v.copy_(torch.from_numpy(a))
+            return v
+        f, c = off(xf), off(np.zeros_like(xc))
+        h.restrict(l, f, c, getattr(api, prec))
+        assert relerr(c.cpu().numpy(), (H.P[l].conj().T @ xf.T.astype(complex)).T) < tol
+        h.prolong(l, off(xc), f, getattr(api, prec))
+        assert relerr(f.cpu().numpy(), (H.P[l] @ xc.T.astype(complex)).T) < tol
+
+
+@pytest.mark.parametrize("images,tol", [(0, 2e-4), (1, 5e-2), (2, 1e-2), (3, 1e-2)])
+@pytest.mark.parametrize("nrhs", [1, 17, 40])
+def test_cycle_with_fused_transfers(api, ctx, nrhs, images, tol):
+    """Three-level FP32 V-cycle: fused residual and restriction on the fine level, the half restriction after a
+    tensor-core sweep (16-bit formats round at 4e-3 / 5e-4, TF32 at 5e-4, several times along a cycle)."""
+    h, H = hierarchy(api, ctx, 64, ntv=8, tensor_cores=images)
+    b = vecs(H.n[0], nrhs, 5, np.complex64)
+    xd = torch.full(b.shape, float("nan"), dtype=torch.complex64, device="cuda")
+    h.vcycle(0, torch.from_numpy(b).cuda(), xd, api.FP32)
+    assert relerr(xd.cpu().numpy(), H.vcycle(0, b.T.astype(complex), 1, 1).T) < tol
