@@ -134,15 +134,24 @@ int schwinger_apply(mgmlmc_ctx* ctx, const double* U, int L, double m0, const vo
     check_prec(prec);
     if (nrhs == 0) return;
     cudaStream_t st = ctx->stream;
-    DBuf l64(sizeof(double2) * 2 * L * L, st);
-    DBuf l32(prec == MGMLMC_FP32 ? sizeof(float2) * 2 * L * L : 0, st);
-    prepare_links(st, (const double2*)U, L, l64.as<double2>(), prec == MGMLMC_FP32 ? l32.as<float2>() : nullptr);
+    const double diag = m0 + 2.0;
+    // Up to 64 K sites x rhs the operator reads U itself (twice the link bytes and 8 FP64 multiplications a site, but
+    // one launch and no workspace: 10 us a call before, of which the operator 4); longer batches prepare the links
+    // once per call, in a workspace of the context.
+    if ((int64_t)L * L * nrhs <= 65536) {
+      if (prec == MGMLMC_FP32)
+        wilson_apply_raw<float>(st, (const double2*)U, (float)diag, L, (const float2*)x, (float2*)y, nrhs);
+      else
+        wilson_apply_raw<double>(st, (const double2*)U, diag, L, (const double2*)x, (double2*)y, nrhs);
+      return;
+    }
+    double2* l64 = (double2*)ctx->work("sa_links64", sizeof(double2) * 2 * L * L);
+    float2* l32 = prec == MGMLMC_FP32 ? (float2*)ctx->work("sa_links32", sizeof(float2) * 2 * L * L) : nullptr;
+    prepare_links(st, (const double2*)U, L, l64, l32);
     if (prec == MGMLMC_FP32)
-      wilson_apply<float>(st, l32.as<float2>(), (float)(m0 + 2.0), L, (const float2*)x, (float2*)y, nullptr, nrhs,
-                          nullptr);
+      wilson_apply<float>(st, l32, (float)diag, L, (const float2*)x, (float2*)y, nullptr, nrhs, nullptr);
     else
-      wilson_apply<double>(st, l64.as<double2>(), m0 + 2.0, L, (const double2*)x, (double2*)y, nullptr, nrhs,
-                           nullptr);
+      wilson_apply<double>(st, l64, diag, L, (const double2*)x, (double2*)y, nullptr, nrhs, nullptr);
   });
 }
 

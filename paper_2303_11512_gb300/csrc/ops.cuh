@@ -19,6 +19,10 @@ template <typename R>
 void wilson_apply(cudaStream_t st, const typename CT<R>::T* links, R diag, int L,
                   const typename CT<R>::T* x, typename CT<R>::T* y, const typename CT<R>::T* b,
                   int nrhs, const int* active);
+// y = D x straight from U (no prepared links), for small batches
+template <typename R>
+void wilson_apply_raw(cudaStream_t st, const double2* U, R diag, int L, const typename CT<R>::T* x,
+                      typename CT<R>::T* y, int nrhs);
 // dense diagonal blocks D_BB (bs x bs sites, 2 dof) of the fine operator: out[block][bd][bd]
 void fine_block_matrices(cudaStream_t st, const double2* l64, double diag, int L, int bs, double2* out);
 

@@ -67,9 +67,31 @@ __device__ __forceinline__ void st_sp(double2* p, long s, double2 a, double2 b) 
   p[2 * s + 1] = b;
 }
 
-// (D x)(s) for one site of one rhs (X points at that rhs).
+// Links of a site's hops: prepared ones (k_prepare_links), or straight from U (same values: a factor of +-1/2 before the
+// rounding to R), which saves a launch and a workspace where a call is a few microseconds.
 template <typename R>
-__device__ __forceinline__ void wilson_site(const typename CT<R>::T* __restrict__ lk, R diag, int L,
+struct PreparedLinks {
+  const typename CT<R>::T* __restrict__ lk;
+  __device__ __forceinline__ typename CT<R>::T x(int s) const { return __ldg(lk + 2 * s); }
+  __device__ __forceinline__ typename CT<R>::T t(int s, bool) const { return __ldg(lk + 2 * s + 1); }
+};
+template <typename R>
+struct RawLinks {
+  const double2* __restrict__ U;
+  __device__ __forceinline__ typename CT<R>::T x(int s) const {
+    const double2 u = __ldg(U + 2 * s);
+    return cmake((R)(-0.5 * u.x), (R)(-0.5 * u.y));
+  }
+  __device__ __forceinline__ typename CT<R>::T t(int s, bool last_slice) const {
+    const double2 u = __ldg(U + 2 * s + 1);
+    const double f = last_slice ? 0.5 : -0.5;
+    return cmake((R)(f * u.x), (R)(f * u.y));
+  }
+};
+
+// (D x)(s) for one site of one rhs (X points at that rhs).
+template <typename R, typename LK>
+__device__ __forceinline__ void wilson_site(const LK& lk, R diag, int L,
                                             const typename CT<R>::T* __restrict__ X, int s,
                                             typename CT<R>::T& o0, typename CT<R>::T& o1) {
   typedef typename CT<R>::T C;
@@ -85,91 +107,188 @@ __device__ __forceinline__ void wilson_site(const typename CT<R>::T* __restrict_
   o1 = cscale(a1, diag);
   {  // +x : (1 - sigma_1) W_0(s) x(s+x)
     ld_sp(X, sxp, a0, a1);
-    C u = cmul(__ldg(lk + 2 * s), csub(a0, a1));
+    C u = cmul(lk.x(s), csub(a0, a1));
     o0 = cadd(o0, u);
     o1 = csub(o1, u);
   }
   {  // -x : (1 + sigma_1) conj(W_0(s-x)) x(s-x)
     ld_sp(X, sxm, a0, a1);
-    C u = cmulc(__ldg(lk + 2 * sxm), cadd(a0, a1));
+    C u = cmulc(lk.x(sxm), cadd(a0, a1));
     o0 = cadd(o0, u);
     o1 = cadd(o1, u);
   }
   {  // +t : (1 - sigma_2) W_1(s) x(s+t)
     ld_sp(X, stp, a0, a1);
-    C u = cmul(__ldg(lk + 2 * s + 1), cadd(a0, cmuli(a1)));
+    C u = cmul(lk.t(s, t == L - 1), cadd(a0, cmuli(a1)));
     o0 = cadd(o0, u);
     o1 = cadd(o1, cmulmi(u));
   }
   {  // -t : (1 + sigma_2) conj(W_1(s-t)) x(s-t)
     ld_sp(X, stm, a0, a1);
-    C u = cmulc(__ldg(lk + 2 * stm + 1), cadd(a0, cmulmi(a1)));
+    C u = cmulc(lk.t(stm, t == 0), cadd(a0, cmulmi(a1)));
     o0 = cadd(o0, u);
     o1 = cadd(o1, cmuli(u));
   }
 }
 
-// One thread per site and RPT right-hand sides (blockIdx.y * RPT + j): the RPT sites' neighbour loads are
-// independent, so each thread keeps RPT times as many loads in flight (the tuner picks RPT per batch size).
-template <typename R, bool RES, int RPT>
-__global__ void __launch_bounds__(256) k_wilson(const typename CT<R>::T* __restrict__ lk, R diag, int L,
-                                                const typename CT<R>::T* __restrict__ x,
+// One thread per site and rhs.
+template <typename R, bool RES, typename LK>
+__global__ void __launch_bounds__(256) k_wilson(LK lk, R diag, int L, const typename CT<R>::T* __restrict__ x,
                                                 typename CT<R>::T* __restrict__ y,
                                                 const typename CT<R>::T* __restrict__ b,
-                                                const int* __restrict__ active, int nrhs) {
+                                                const int* __restrict__ active) {
   typedef typename CT<R>::T C;
-  const int V = L * L;
-  const int s = blockIdx.x * blockDim.x + threadIdx.x;
-  if (s >= V) return;
-  C o0[RPT], o1[RPT];
+  const int V = L * L, s = blockIdx.x * blockDim.x + threadIdx.x, rhs = blockIdx.y;
+  if (s >= V || (active && !active[rhs])) return;
+  const size_t off = (size_t)rhs * 2 * V;
+  C o0, o1;
+  wilson_site<R>(lk, diag, L, x + off, s, o0, o1);
+  if (RES) {
+    C b0, b1;
+    ld_sp(b + off, s, b0, b1);
+    o0 = csub(b0, o0);
+    o1 = csub(b1, o1);
+  }
+  st_sp(y + off, s, o0, o1);
+}
+
+// FP32, long batches: a thread walks WT time slices of its column, for RPT right-hand sides (blockIdx.y * RPT + j),
+// with the spinors of the last, this and the next slice in registers, so that a spinor comes from L2 (1 + 2 / WT)
+// times instead of three times and a link 1 / RPT times; its x neighbours are L1 hits of the same row.  One thread
+// per site and rhs moved 80 bytes of L2 traffic per site and rhs for 32 of DRAM (5.0 TB/s at L = 512, 256 rhs).
+constexpr int WT = 8;
+template <bool RES, int RPT>
+__global__ void __launch_bounds__(128) k_wilson_walk(const float2* __restrict__ lk, float diag, int L, int xblocks,
+                                                     const float2* __restrict__ x, float2* __restrict__ y,
+                                                     const float2* __restrict__ b, const int* __restrict__ active,
+                                                     int nrhs) {
+  const int V = L * L, tb = blockIdx.x / xblocks, xx = (blockIdx.x - tb * xblocks) * 128 + threadIdx.x;
+  const int t0 = tb * WT, t1 = min(t0 + WT, L);
+  if (xx >= L) return;
+  const float4* X[RPT];
   bool on[RPT];
+  float4 prev[RPT], cur[RPT];
+  const int xr = xx == L - 1 ? 0 : xx + 1, xl = xx == 0 ? L - 1 : xx - 1, tp0 = t0 == 0 ? L - 1 : t0 - 1;
 #pragma unroll
   for (int j = 0; j < RPT; ++j) {
     const int rhs = blockIdx.y * RPT + j;
     on[j] = rhs < nrhs && !(active && !active[rhs]);
-    if (on[j]) wilson_site<R>(lk, diag, L, x + (size_t)rhs * 2 * V, s, o0[j], o1[j]);
-  }
-#pragma unroll
-  for (int j = 0; j < RPT; ++j) {
-    if (!on[j]) continue;
-    const size_t off = (size_t)(blockIdx.y * RPT + j) * 2 * V;
-    if (RES) {
-      C b0, b1;
-      ld_sp(b + off, s, b0, b1);
-      o0[j] = csub(b0, o0[j]);
-      o1[j] = csub(b1, o1[j]);
+    X[j] = reinterpret_cast<const float4*>(x + (size_t)(on[j] ? rhs : 0) * 2 * V);
+    if (on[j]) {
+      prev[j] = __ldg(X[j] + (size_t)tp0 * L + xx);
+      cur[j] = __ldg(X[j] + (size_t)t0 * L + xx);
     }
-    st_sp(y + off, s, o0[j], o1[j]);
   }
+  float2 wt_prev = __ldg(lk + 2 * (tp0 * L + xx) + 1);
+#pragma unroll 2
+  for (int t = t0; t < t1; ++t) {
+    const int row = t * L, s = row + xx, next = (t == L - 1 ? 0 : row + L) + xx;
+    const float4 w = __ldg(reinterpret_cast<const float4*>(lk) + s);  // both links of the site
+    const float2 wx = make_float2(w.x, w.y), wt = make_float2(w.z, w.w), wl = __ldg(lk + 2 * (row + xl));
+#pragma unroll
+    for (int j = 0; j < RPT; ++j) {
+      if (!on[j]) continue;
+      const float4 nx = __ldg(X[j] + next), rt = __ldg(X[j] + row + xr), lf = __ldg(X[j] + row + xl);
+      float2 o0 = cscale(make_float2(cur[j].x, cur[j].y), diag), o1 = cscale(make_float2(cur[j].z, cur[j].w), diag);
+      float2 a0, a1;
+      a0 = make_float2(rt.x, rt.y); a1 = make_float2(rt.z, rt.w);
+      {
+        const float2 u = cmul(wx, csub(a0, a1));
+        o0 = cadd(o0, u);
+        o1 = csub(o1, u);
+      }
+      a0 = make_float2(lf.x, lf.y); a1 = make_float2(lf.z, lf.w);
+      {
+        const float2 u = cmulc(wl, cadd(a0, a1));
+        o0 = cadd(o0, u);
+        o1 = cadd(o1, u);
+      }
+      a0 = make_float2(nx.x, nx.y); a1 = make_float2(nx.z, nx.w);
+      {
+        const float2 u = cmul(wt, cadd(a0, cmuli(a1)));
+        o0 = cadd(o0, u);
+        o1 = cadd(o1, cmulmi(u));
+      }
+      a0 = make_float2(prev[j].x, prev[j].y); a1 = make_float2(prev[j].z, prev[j].w);
+      {
+        const float2 u = cmulc(wt_prev, cadd(a0, cmulmi(a1)));
+        o0 = cadd(o0, u);
+        o1 = cadd(o1, cmuli(u));
+      }
+      const size_t off = (size_t)(blockIdx.y * RPT + j) * 2 * V;
+      if (RES) {
+        float2 b0, b1;
+        ld_sp(b + off, s, b0, b1);
+        o0 = csub(b0, o0);
+        o1 = csub(b1, o1);
+      }
+      st_sp(y + off, s, o0, o1);
+      prev[j] = cur[j];
+      cur[j] = nx;
+    }
+    wt_prev = wt;
+  }
+}
+
+template <typename R, typename LK>
+static void wilson_sites(cudaStream_t st, LK lk, R diag, int L, const typename CT<R>::T* x, typename CT<R>::T* y,
+                         const typename CT<R>::T* b, int nrhs, const int* active, double bytes, double flops) {
+  // blocks of 64 threads where 256 would leave most SMs without one (FP64: two FMAs a clock and SM bound it)
+  const int bt = (long)L * L * nrhs >= 152L * 256 * 2 ? 256 : 64;
+  const dim3 grid(cdiv((long)L * L, bt), nrhs);
+  if (b)
+    MG_LAUNCH_W(bytes, flops, (k_wilson<R, true, LK>), grid, bt, 0, st, lk, diag, L, x, y, b, active);
+  else
+    MG_LAUNCH_W(bytes, flops, (k_wilson<R, false, LK>), grid, bt, 0, st, lk, diag, L, x, y, b, active);
 }
 
 template <typename R>
 void wilson_apply(cudaStream_t st, const typename CT<R>::T* links, R diag, int L, const typename CT<R>::T* x,
                   typename CT<R>::T* y, const typename CT<R>::T* b, int nrhs, const int* active) {
   if (nrhs <= 0) return;
-  const int rpt = sizeof(R) == 4 ? tune_lookup(TUNE_WILSON32, L, nrhs, 0, 1) : 1;
-  // blocks of 64 threads where 256 would leave most SMs without one (FP64: two FMAs a clock and SM bound it)
-  const int bt = (long)L * L * cdiv(nrhs, rpt) >= 152L * 256 * 2 ? 256 : 64;
-  dim3 grid(cdiv((long)L * L, bt), cdiv(nrhs, rpt));
   // algorithmic traffic: x read + y written once per site and rhs (+ b), links once per launch
   const double V = (double)L * L, sp = 2.0 * sizeof(typename CT<R>::T), ar = act_rhs(nrhs);
   const double bytes = ar * V * sp * (b ? 3 : 2) + V * sp;
   const double flops = ar * V * (b ? 56.0 : 52.0);
-#define MG_WILSON_LAUNCH(RPT_)                                                                                  \
-  do {                                                                                                          \
-    if (b)                                                                                                      \
-      MG_LAUNCH_W(bytes, flops, (k_wilson<R, true, RPT_>), grid, bt, 0, st, links, diag, L, x, y, b, active, nrhs); \
-    else                                                                                                        \
-      MG_LAUNCH_W(bytes, flops, (k_wilson<R, false, RPT_>), grid, bt, 0, st, links, diag, L, x, y, b, active, nrhs); \
+  if constexpr (sizeof(R) == 4) {
+    // the walking form needs L * L / WT threads per rhs to fill the chip; at L = 512 with 256 rhs it takes 375 us (86 %
+    // of the copy bandwidth) with one rhs per thread, 392 with two, 477 with four, 413 with 16 slices and one rhs, and
+    // one thread per site 418 us
+    const int rpt = tune_lookup(TUNE_WILSON32, L, nrhs, 0, 1);
+    if (V * nrhs / (WT * rpt) >= 152.0 * 1024) {
+      const int xb = cdiv(L, 128);
+      const dim3 grid(xb * cdiv(L, WT), cdiv(nrhs, rpt));
+#define MG_WILSON_LAUNCH(RPT_)                                                                                        \
+  do {                                                                                                                \
+    if (b)                                                                                                            \
+      MG_LAUNCH_W(bytes, flops, (k_wilson_walk<true, RPT_>), grid, 128, 0, st, links, diag, L, xb, x, y, b, active,   \
+                  nrhs);                                                                                              \
+    else                                                                                                              \
+      MG_LAUNCH_W(bytes, flops, (k_wilson_walk<false, RPT_>), grid, 128, 0, st, links, diag, L, xb, x, y, b, active,  \
+                  nrhs);                                                                                              \
   } while (0)
-  if (rpt == 4)
-    MG_WILSON_LAUNCH(4);
-  else if (rpt == 2)
-    MG_WILSON_LAUNCH(2);
-  else
-    MG_WILSON_LAUNCH(1);
+      if (rpt == 4)
+        MG_WILSON_LAUNCH(4);
+      else if (rpt == 2)
+        MG_WILSON_LAUNCH(2);
+      else
+        MG_WILSON_LAUNCH(1);
 #undef MG_WILSON_LAUNCH
+      return;
+    }
+  }
+  wilson_sites<R>(st, PreparedLinks<R>{links}, diag, L, x, y, b, nrhs, active, bytes, flops);
 }
+
+template <typename R>
+void wilson_apply_raw(cudaStream_t st, const double2* U, R diag, int L, const typename CT<R>::T* x,
+                      typename CT<R>::T* y, int nrhs) {
+  const double V = (double)L * L, sp = 2.0 * sizeof(typename CT<R>::T);
+  wilson_sites<R>(st, RawLinks<R>{U}, diag, L, x, y, (const typename CT<R>::T*)nullptr, nrhs, nullptr,
+                  nrhs * V * sp * 2 + V * 32.0, nrhs * V * 52.0);
+}
+template void wilson_apply_raw<float>(cudaStream_t, const double2*, float, int, const float2*, float2*, int);
+template void wilson_apply_raw<double>(cudaStream_t, const double2*, double, int, const double2*, double2*, int);
 template void wilson_apply<float>(cudaStream_t, const float2*, float, int, const float2*, float2*, const float2*,
                                   int, const int*);
 template void wilson_apply<double>(cudaStream_t, const double2*, double, int, const double2*, double2*,
@@ -543,7 +662,7 @@ __global__ void __launch_bounds__(256) k_sap_fine2(const typename CT<R>::T* __re
       if (rhs < nrhs && !(active && !active[rhs])) {
         const int s = (BT * 2 + j / 2) * L + BX * 2 + (j % 2);
         C o0, o1, f0, f1;
-        wilson_site<R>(lk, diag, L, x + rhs * n, s, o0, o1);
+        wilson_site<R>(PreparedLinks<R>{lk}, diag, L, x + rhs * n, s, o0, o1);
         ld_sp(f + rhs * n, s, f0, f1);
         sres[g * BD + 2 * j] = csub(f0, o0);
         sres[g * BD + 2 * j + 1] = csub(f1, o1);

@@ -179,3 +179,18 @@ def test_cycle_with_fused_transfers(api, ctx, nrhs, images, tol):
     xd = torch.full(b.shape, float("nan"), dtype=torch.complex64, device="cuda")
     h.vcycle(0, torch.from_numpy(b).cuda(), xd, api.FP32)
     assert relerr(xd.cpu().numpy(), H.vcycle(0, b.T.astype(complex), 1, 1).T) < tol
+
+
+@pytest.mark.parametrize("L,nrhs", [(4, 1), (6, 7), (130, 80), (142, 61), (512, 5), (512, 6)])
+@pytest.mark.parametrize("prec,tol", [("FP64", 1e-14), ("FP32", 2e-6)])
+def test_stencil_forms(api, ctx, L, nrhs, prec, tol):
+    """Fine operator straight from U (up to 64 K sites x rhs), from prepared links, and walking along t with lattice
+    sides that are no multiple of its 128 columns or 8 slices (nine terms, a few roundings each)."""
+    rs = np.random.default_rng(L)
+    U = np.exp(1j * rs.uniform(-3, 3, (L, L, 2)))
+    dt = np.complex128 if prec == "FP64" else np.complex64
+    x = vecs(2 * L * L, nrhs, 3, dt)
+    y = torch.full(x.shape, float("nan"), dtype=torch.from_numpy(x).dtype, device="cuda")
+    api.schwinger_apply(ctx, torch.from_numpy(U).cuda(), L, 0.1, torch.from_numpy(x).cuda(), y, getattr(api, prec))
+    ref = (osch.dirac_sparse(U, 0.1) @ x.T.astype(complex)).T
+    assert relerr(y.cpu().numpy(), ref) < tol
