@@ -104,6 +104,51 @@ inline double act_rhs(int nrhs) { return (g_nact_hint >= 0 && g_nact_hint < nrhs
 #define MG_LAUNCH(kernel, grid, block, smem, stream, ...) \
   MG_LAUNCH_W(0, 0, kernel, grid, block, smem, stream, __VA_ARGS__)
 
+// Programmatic dependent launch: a kernel that begins with pdl_begin() may be launched with MG_LAUNCH_P, and the GPU
+// then places its blocks while the last blocks of the kernel before it still run.  pdl_begin() waits until that
+// kernel has completed and its writes are visible, so nothing may be read or written before it (and what an earlier
+// kernel wrote is not read through __restrict__ const pointers or __ldg, whose loads need not stay behind it); it
+// also lets the next kernel be placed.  Used by the kernels of a V-cycle, where a launch below PDL_BYTES takes 5 to
+// 12 us of which this hides about 2 (V(1,1) at L = 128 with 5 right-hand sides: 157 -> 129 us).  Larger launches lose
+// by it (V(2,2) at L = 512 with 32: 1.82 -> 1.93 ms with every launch), and in a graph there is nothing left to hide.
+__device__ __forceinline__ void pdl_begin() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+constexpr double PDL_BYTES = 8e6;
+extern thread_local bool g_capturing;  // launches go into a graph
+template <typename... Par, typename... Arg>
+inline void launch_pdl(bool early, void (*kernel)(Par...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
+                       Arg&&... arg) {
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cfg.attrs = &at;
+  cfg.numAttrs = early ? 1 : 0;
+  MG_CUDA(cudaLaunchKernelEx(&cfg, kernel, static_cast<Par>(arg)...));
+}
+#define MG_LAUNCH_P(bytes, flops, kernel, grid, block, smem, stream, ...)          \
+  do {                                                                             \
+    ::mg::KTimer* t_ = ::mg::g_timer;                                              \
+    cudaEvent_t a_ = nullptr, b_ = nullptr;                                        \
+    if (t_ && t_->want(#kernel)) {                                                 \
+      a_ = t_->get();                                                              \
+      b_ = t_->get();                                                              \
+      MG_CUDA(cudaEventRecord(a_, (stream)));                                      \
+    }                                                                              \
+    ::mg::launch_pdl((bytes) < PDL_BYTES && !::mg::g_capturing, kernel, (grid), (block), (smem), (stream), __VA_ARGS__);      \
+    if (a_) {                                                                      \
+      MG_CUDA(cudaEventRecord(b_, (stream)));                                      \
+      t_->recs.push_back({#kernel, __PRETTY_FUNCTION__, (double)(bytes), (double)(flops), a_, b_}); \
+    }                                                                              \
+    if (::mg::g_launch_counter) ++*::mg::g_launch_counter;                         \
+  } while (0)
+
 // ---------------------------------------------------------------- complex
 template <typename R> struct CT;
 template <> struct CT<float> { typedef float2 T; };

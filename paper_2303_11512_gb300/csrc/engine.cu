@@ -14,6 +14,7 @@ namespace mg {
 thread_local int64_t* g_launch_counter = nullptr;
 thread_local KTimer* g_timer = nullptr;
 thread_local int g_nact_hint = -1;
+thread_local bool g_capturing = false;
 
 // ---------------------------------------------------------------- helpers
 template <typename R> static inline const typename CT<R>::T* links_of(const LevelData& L) {
@@ -232,20 +233,20 @@ static void vcycle_maybe_graph(mgmlmc_hier* h, int l, const typename CT<R>::T* i
     if (!h->capture_stream) MG_CUDA(cudaStreamCreateWithFlags(&h->capture_stream, cudaStreamNonBlocking));
     cudaStream_t cs = h->capture_stream;
     MG_CUDA(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
-    h->capturing = true;
+    h->capturing = g_capturing = true;
     h->ctx->stream = cs;  // the V-cycle's launches go to the capturing stream
     try {
       vcycle<R>(h, l, gin, gout, nrhs, active);
     } catch (...) {
       h->ctx->stream = st;
-      h->capturing = false;
+      h->capturing = g_capturing = false;
       cudaStreamEndCapture(cs, &graph);
       if (graph) cudaGraphDestroy(graph);
       cudaGetLastError();
       throw;
     }
     h->ctx->stream = st;
-    h->capturing = false;
+    h->capturing = g_capturing = false;
     MG_CUDA(cudaStreamEndCapture(cs, &graph));
     const int64_t captured = g_launch_counter ? *g_launch_counter - before : 0;
     if (g_launch_counter) *g_launch_counter = before;  // capturing issued nothing

@@ -423,8 +423,9 @@ __global__ void __launch_bounds__(256) k_prolong(const typename CT<R>::T* __rest
 // each.  half: xf is zero on the 2 x 2 blocks of colour 1 (and not read there).
 template <typename R, int RG, int MM, int RR>
 __global__ void __launch_bounds__(16 / MM * (RG / RR))
-    k_restrict16(const typename CT<R>::T* __restrict__ P, int Ls, const typename CT<R>::T* __restrict__ xf,
-                 typename CT<R>::T* __restrict__ xc, bool half, int nrhs, const int* __restrict__ active) {
+    k_restrict16(const typename CT<R>::T* __restrict__ P, int Ls, const typename CT<R>::T* xf,
+                 typename CT<R>::T* __restrict__ xc, bool half, int nrhs, const int* active) {
+  pdl_begin();
   typedef typename CT<R>::T C;
   constexpr int T = 16 / MM * (RG / RR), XP = 256 + 16 / (int)sizeof(C);
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -479,9 +480,10 @@ __global__ void __launch_bounds__(16 / MM * (RG / RR))
 // xf16: the planar 16-bit copy is written alongside.
 template <typename R, bool ADD, int D, int RG>
 __global__ void __launch_bounds__(128) k_prolong2(const typename CT<R>::T* __restrict__ P, int Ls,
-                                                  const typename CT<R>::T* __restrict__ xc,
-                                                  typename CT<R>::T* __restrict__ xf, unsigned short* __restrict__ xf16,
-                                                  int bf, int nrhs, const int* __restrict__ active) {
+                                                  const typename CT<R>::T* xc,
+                                                  typename CT<R>::T* xf, unsigned short* __restrict__ xf16,
+                                                  int bf, int nrhs, const int* active) {
+  pdl_begin();
   typedef typename CT<R>::T C;
   constexpr int PAIRS = 8 * D, RS = 128 / PAIRS;  // dof pairs of an aggregate, rhs taken at once
   constexpr int ROWS = 8 * D;                     // rows of a chirality block
@@ -490,7 +492,7 @@ __global__ void __launch_bounds__(128) k_prolong2(const typename CT<R>::T* __res
   const size_t n = (size_t)Ls * Ls * D, nc = (size_t)Lc * Lc * 16;
   for (int q = tid; q < RG * 16; q += 128) {
     const int g = q >> 4, rhs = r0 + g;
-    if (rhs < nrhs && !(active && !active[rhs])) sc[g][q & 15] = __ldg(xc + rhs * nc + (size_t)a * 16 + (q & 15));
+    if (rhs < nrhs && !(active && !active[rhs])) sc[g][q & 15] = xc[rhs * nc + (size_t)a * 16 + (q & 15)];
   }
   const int pr = tid % PAIRS, js = pr / (D / 2), k = 2 * (pr % (D / 2)), rs = tid / PAIRS;
   const int c0 = D == 2 ? 0 : k >> 3, c1 = D == 2 ? 1 : c0;
@@ -553,7 +555,7 @@ void restrict_op(cudaStream_t stm, const typename CT<R>::T* P, int Ls, int d, in
     constexpr int RG = sizeof(R) == 4 ? 16 : 8, MM = sizeof(R) == 4 ? 2 : 1;
     constexpr int T = 16 / MM * (RG / MM), sm = (int)sizeof(C) * (2048 + RG * (256 + 16 / (int)sizeof(C)));
     ensure_max_smem((const void*)k_restrict16<R, RG, MM, MM>, sm);
-    MG_LAUNCH_W(bytes, flops, (k_restrict16<R, RG, MM, MM>), dim3(Lc * Lc, cdiv(nrhs, RG)), T, sm, stm, P, Ls, xf, xc,
+    MG_LAUNCH_P(bytes, flops, (k_restrict16<R, RG, MM, MM>), dim3(Lc * Lc, cdiv(nrhs, RG)), T, sm, stm, P, Ls, xf, xc,
                 half, nrhs, active);
     return;
   }
@@ -579,7 +581,7 @@ static void prolong_launch(cudaStream_t stm, const typename CT<R>::T* P, int Ls,
   const int Lc = Ls / agg;
   auto go = [&](auto dd, auto rg) {
     constexpr int D = decltype(dd)::value, RG = decltype(rg)::value;
-    MG_LAUNCH_W(bytes, flops, (k_prolong2<R, ADD, D, RG>), dim3(Lc * Lc, cdiv(nrhs, RG)), 128, 0, stm, P, Ls, xc, xf,
+    MG_LAUNCH_P(bytes, flops, (k_prolong2<R, ADD, D, RG>), dim3(Lc * Lc, cdiv(nrhs, RG)), 128, 0, stm, P, Ls, xc, xf,
                 xf16, bf, nrhs, active);
   };
   typedef std::integral_constant<int, 8> I8;

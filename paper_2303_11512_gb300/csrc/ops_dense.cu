@@ -545,8 +545,9 @@ struct DenseTile {
 };
 
 template <typename C, int RI, int NR>
-__global__ void __launch_bounds__(64) k_dense_apply(const C* __restrict__ A, int n, const C* __restrict__ x,
-                                                    C* __restrict__ y, int nrhs, const int* __restrict__ active) {
+__global__ void __launch_bounds__(64) k_dense_apply(const C* __restrict__ A, int n, const C* x,
+                                                    C* __restrict__ y, int nrhs, const int* active) {
+  pdl_begin();
   typedef DenseTile<C, RI, NR> DT;
   constexpr int KC = DT::KC, ST = DT::ST, TI = DT::TI, TR = DT::TR;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -615,7 +616,7 @@ void dense_apply(cudaStream_t st, const typename CT<R>::T* A, int n, const typen
     constexpr int RI = decltype(ri)::value, NR = decltype(nr)::value;
     constexpr int sm = (int)sizeof(DenseTile<C, RI, NR>);
     ensure_max_smem((const void*)k_dense_apply<C, RI, NR>, sm);
-    MG_LAUNCH_W(bytes, flops, (k_dense_apply<C, RI, NR>), dim3(cdiv(n, 8 * RI), cdiv(nrhs, 8 * NR)), 64, sm, st, A, n,
+    MG_LAUNCH_P(bytes, flops, (k_dense_apply<C, RI, NR>), dim3(cdiv(n, 8 * RI), cdiv(nrhs, 8 * NR)), 64, sm, st, A, n,
                 x, y, nrhs, active);
   };
   typedef std::integral_constant<int, 1> I1;

@@ -391,9 +391,10 @@ struct SapF {
 
 template <int RG, bool RESTRICT>
 __global__ void __launch_bounds__(64) k_sap_fine4_fp32(const float2* __restrict__ lk, float diag, int L,
-                                                       const float2* __restrict__ inv, const float2* __restrict__ f,
+                                                       const float2* __restrict__ inv, const float2* f,
                                                        const float2* x, float2* out, int color, int nrhs, int nitems,
-                                                       int known, const int* __restrict__ active) {
+                                                       int known, const int* active) {
+  pdl_begin();
   typedef SapF<RG, RESTRICT> S;
   constexpr int RP = S::RP, T = 64, NR = RG / 8, RSTEP = T / (4 * RG) ? T / (4 * RG) : 1;
   constexpr int RTH = T / 4 < RG ? T / 4 : RG;  // rhs that the CTA's threads fetch at once
@@ -713,7 +714,7 @@ void sap_half_fine(cudaStream_t st, const typename CT<R>::T* links, R diag, int 
       const int ntile = (nrhs + RG - 1) / RG;
       const dim3 grid(std::max(1, std::min(nb, (nsm * per_sm + ntile - 1) / ntile)), ntile);
       ensure_max_smem((const void*)k_sap_fine4_fp32<RG, false>, sm);
-      MG_LAUNCH_W(bytes, flops, (k_sap_fine4_fp32<RG, false>), grid, 64, sm, st, links, diag, L, inv, f, x, x, color,
+      MG_LAUNCH_P(bytes, flops, (k_sap_fine4_fp32<RG, false>), grid, 64, sm, st, links, diag, L, inv, f, x, x, color,
                   nrhs, nb, known, active);
     };
     if (nrhs <= 8)
@@ -755,7 +756,7 @@ void residual_restrict_fine(cudaStream_t st, const float2* links, float diag, in
     const int ntile = (nrhs + RG - 1) / RG;
     const dim3 grid(std::max(1, std::min(na, (nsm * per_sm + ntile - 1) / ntile)), ntile);
     ensure_max_smem((const void*)k_sap_fine4_fp32<RG, true>, sm);
-    MG_LAUNCH_W(bytes, flops, (k_sap_fine4_fp32<RG, true>), grid, 64, sm, st, links, diag, L, P, f, x, xc, 0, nrhs, na,
+    MG_LAUNCH_P(bytes, flops, (k_sap_fine4_fp32<RG, true>), grid, 64, sm, st, links, diag, L, P, f, x, xc, 0, nrhs, na,
                 SAP_X, active);
   };
   if (nrhs <= 8)

@@ -109,9 +109,10 @@ __host__ __device__ constexpr int tc_stage_bytes(int MODE, int BF, int KC, int N
 // item is multiplied.
 template <int MODE, int BF>
 __global__ void __launch_bounds__(TC_THREADS, 1)
-    k_tc(const __grid_constant__ CUtensorMap amap, const void* __restrict__ Wv, float* __restrict__ out,
-         const float* __restrict__ bvec, int Ls, int nitems, int bmode, int color, int nrhs, int vrows, int mm,
-         int stages, const int* __restrict__ active, int* err) {
+    k_tc(const __grid_constant__ CUtensorMap amap, const void* __restrict__ Wv, float* out,
+         const float* bvec, int Ls, int nitems, int bmode, int color, int nrhs, int vrows, int mm,
+         int stages, const int* active, int* err) {
+  pdl_begin();
   typedef TcCfg<MODE> CF;
   constexpr int KC = CF::KC, NW = CF::NW;
   const int MM = MODE == 0 ? mm : TC_M;           // MMA M
@@ -557,7 +558,7 @@ void launch_tc(cudaStream_t st, const float2* vin, const void* W, float* out, co
   const int tiles = (nrhs + tile - 1) / tile;
   const int gx = std::max(1, std::min(nitems, (nsm + tiles - 1) / tiles));
   dim3 grid(gx, tiles);
-  MG_LAUNCH_W(bytes, flops, k_tc_kernel, grid, TC_THREADS, sm, st, m, W, out, b, Ls, nitems, bmode, color, nrhs,
+  MG_LAUNCH_P(bytes, flops, k_tc_kernel, grid, TC_THREADS, sm, st, m, W, out, b, Ls, nitems, bmode, color, nrhs,
               vrows, mm, stages, active, err);
 }
 

@@ -103,9 +103,10 @@ __device__ __forceinline__ void tb_corner(int k, int Ls, int bmode, int color, i
 // the A operand of the SAP block update k_tcs)
 template <int BF, int O16>
 __global__ void __launch_bounds__(TB_THREADS, 1)
-    k_tcb(const __grid_constant__ CUtensorMap xmap, const unsigned char* __restrict__ W, void* __restrict__ out,
-          const float* __restrict__ bvec, int Ls, int nitems, int bmode, int color, int nrhs, int vrows_t,
-          const int* __restrict__ active, int* err) {
+    k_tcb(const __grid_constant__ CUtensorMap xmap, const unsigned char* __restrict__ W, void* out,
+          const float* bvec, int Ls, int nitems, int bmode, int color, int nrhs, int vrows_t,
+          const int* active, int* err) {
+  pdl_begin();
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* base = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   __shared__ __align__(8) uint64_t full_bar[TB_MAXST], empty_bar[TB_MAXST], xfull_bar[TB_MAXST];
@@ -387,8 +388,9 @@ constexpr int TS_SMEM = 1024 + TS_STAGES * TS_STAGE + TS_XBYTES;
 template <int BF>
 __global__ void __launch_bounds__(TS_THREADS, 1)
     k_tcs(const __grid_constant__ CUtensorMap rmap, const __grid_constant__ CUtensorMap xmap,
-          const unsigned char* __restrict__ Winv, float* __restrict__ x, uint16_t* __restrict__ x16, int Ls, int nitems,
-          int color, int nrhs, int xrows, const int* __restrict__ active, int* err) {
+          const unsigned char* __restrict__ Winv, float* x, uint16_t* x16, int Ls, int nitems,
+          int color, int nrhs, int xrows, const int* active, int* err) {
+  pdl_begin();
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* base = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   __shared__ __align__(8) uint64_t full_bar[TS_STAGES], empty_bar[TS_STAGES], xfull_bar[TS_STAGES];
@@ -672,7 +674,7 @@ void tc_block_stencil(cudaStream_t st, int bf, const void* W, int Ls, const void
   auto go = [&](auto* k_tcb_kernel) {
     ensure_max_smem((const void*)k_tcb_kernel, tb_smem_bytes(32) > tb_smem_bytes(64) ? tb_smem_bytes(32)
                                                                                       : tb_smem_bytes(64));
-    MG_LAUNCH_W(bytes, flops, k_tcb_kernel, grid, TB_THREADS, smem, st, xmap, (const unsigned char*)W, y,
+    MG_LAUNCH_P(bytes, flops, k_tcb_kernel, grid, TB_THREADS, smem, st, xmap, (const unsigned char*)W, y,
                 (const float*)b, Ls, nitems, bmode, color, nrhs, vrows_t, active, err);
   };
   if (bf == 2)
@@ -706,7 +708,7 @@ void tc_block_update(cudaStream_t st, int bf, const void* Winv, int Ls, const vo
   const dim3 grid = grid_of(nitems, nrhs);
   auto go = [&](auto* k_tcs_kernel) {
     ensure_max_smem((const void*)k_tcs_kernel, TS_SMEM);
-    MG_LAUNCH_W(bytes, flops, k_tcs_kernel, grid, TS_THREADS, TS_SMEM, st, rmap, xmap, (const unsigned char*)Winv,
+    MG_LAUNCH_P(bytes, flops, k_tcs_kernel, grid, TS_THREADS, TS_SMEM, st, rmap, xmap, (const unsigned char*)Winv,
                 (float*)x, (uint16_t*)x16, Ls, nitems, color, nrhs, xrows, active, err);
   };
   if (bf == 2)
