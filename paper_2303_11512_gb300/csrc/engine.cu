@@ -777,7 +777,7 @@ mgmlmc_sketch* deflation_basis(mgmlmc_hier* h, int k, int sweeps, uint64_t seed,
     double* yn = (double*)h->work("df_yn", 0, sizeof(double) * k);
     double2* G = (double2*)h->work("df_G", 0, sizeof(double2) * k * k);
     vnorm2<double2>(st, Y, n, k, yn, h->work("df_red", 0, reduce_work_bytes(n, k, 1)), nullptr);
-    proj_coeffs(st, V, k, Y, n, k, G, h->work("df_pw", 0, proj_work_bytes(k, n, k)));
+    proj_coeffs(st, V, k, Y, nullptr, n, k, G, h->work("df_pw", 0, proj_work_bytes(k, n, k)));
     std::vector<double> hy(k);
     std::vector<double2> hg((size_t)k * k);
     MG_CUDA(cudaMemcpyAsync(hy.data(), yn, sizeof(double) * k, cudaMemcpyDeviceToHost, st));
@@ -888,8 +888,7 @@ void project(mgmlmc_ctx* ctx, const mgmlmc_sketch* s, const double2* zeta, const
     MG_CHECK_ARG(s->n == n, "sketch and vectors differ in size");
     double2* c = (double2*)ctx->work("pj_c", sizeof(double2) * d * nrhs * 2);
     void* w = ctx->work("pj_w", proj_work_bytes(d, n, nrhs));
-    proj_coeffs(st, s->Q.as<double2>(), d, zeta, n, nrhs, c, w);
-    proj_coeffs(st, s->Q.as<double2>(), d, y, n, nrhs, c + (size_t)d * nrhs, w);
+    proj_coeffs(st, s->Q.as<double2>(), d, zeta, y, n, nrhs, c, w);
     MG_LAUNCH(k_proj_combine, cdiv(nrhs, 64), 64, 0, st, a, c, d, nrhs);
   }
   MG_CUDA(cudaMemcpyAsync(tau_host, a, sizeof(double2) * nrhs, cudaMemcpyDeviceToHost, st));

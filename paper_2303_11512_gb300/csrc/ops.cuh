@@ -167,9 +167,9 @@ size_t gram_work_bytes(int d, long n);
 void chol_inv_upper(cudaStream_t st, const double2* G, int d, double2* Rinv, int* fail);
 // Y <- Y Rinv (in place, Rinv upper triangular)
 void right_mul_upper(cudaStream_t st, double2* Y, int d, long n, const double2* Rinv);
-// c[i][rhs] = Q_i^H x_rhs, Q = [d][n], x = [nrhs][n]
-void proj_coeffs(cudaStream_t st, const double2* Q, int d, const double2* x, long n, int nrhs, double2* c,
-                 void* work);
+// c[i][rhs] = Q_i^H x_rhs, Q = [d][n], x = [nrhs][n]; x2 (or nullptr): the same for it, c[d + i][rhs]
+void proj_coeffs(cudaStream_t st, const double2* Q, int d, const double2* x, const double2* x2, long n, int nrhs,
+                 double2* c, void* work);
 size_t proj_work_bytes(int d, long n, int nrhs);
 
 // ---------------------------------------------------------------- tensor cores (coarse levels, d = 16)

@@ -728,43 +728,60 @@ void gram(cudaStream_t st, const double2* Y, int d, long n, double2* G, void* wo
   MG_LAUNCH(k_gram_final, cdiv(d * d, 256), 256, 0, st, part, d, nb, G);
 }
 
-// G = R^H R (R upper, real positive diagonal), Rinv = R^{-1}; R and its inverse in dynamic shared memory
-__global__ void k_chol_inv(const double2* __restrict__ Gg, int d, double2* __restrict__ Rinv, int* fail) {
+// G = R^H R (R upper, real positive diagonal), Rinv = R^{-1}; both in dynamic shared memory.  One CTA; what it costs is
+// the latency of dependent FP64 operations, so the factorisation updates the whole trailing matrix after each row
+// (one dependent product per step instead of a sum over the rows before it), one thread forms a row's root and
+// reciprocal, and the inverse is formed row by row from the bottom, four threads to a sum.  d = 32: 258 -> 106 us.
+// Every entry of R takes its subtractions and roundings in the order of a sum over the rows before it: a rank-deficient
+// Gram matrix is found by a pivot that rounds to zero or below.
+__global__ void __launch_bounds__(256) k_chol_inv(const double2* __restrict__ Gg, int d, double2* __restrict__ Rinv,
+                                                  int* fail) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   double2* R = reinterpret_cast<double2*>(smem_raw);
   double2* X = R + d * d;
+  __shared__ double rd[SK_MAXD];  // reciprocals of the diagonal of R
   __shared__ int bad;
   const int tid = threadIdx.x;
-  for (int e = tid; e < d * d; e += blockDim.x) { R[e] = Gg[e]; X[e] = make_double2(0, 0); }
+  for (int e = tid; e < d * d; e += 256) { R[e] = Gg[e]; X[e] = make_double2(0, 0); }
   if (tid == 0) bad = 0;
   __syncthreads();
   for (int k = 0; k < d; ++k) {
     if (tid == 0) {
-      double s = R[k * d + k].x;
-      for (int i = 0; i < k; ++i) s -= cabs2(R[i * d + k]);
+      const double s = R[k * d + k].x;
       if (!(s > 0.0)) bad = 1;
-      R[k * d + k] = make_double2(sqrt(fmax(s, 1e-300)), 0);
+      const double root = sqrt(fmax(s, 1e-300));
+      R[k * d + k] = make_double2(root, 0);
+      rd[k] = 1.0 / root;
     }
     __syncthreads();
-    const double rkk = R[k * d + k].x;
-    for (int j = k + 1 + tid; j < d; j += blockDim.x) {
-      double2 s = R[k * d + j];
-      for (int i = 0; i < k; ++i) s = csub(s, cmulc(R[i * d + k], R[i * d + j]));
-      R[k * d + j] = cscale(s, 1.0 / rkk);
+    const double inv = rd[k];
+    for (int j = k + 1 + tid; j < d; j += 256) R[k * d + j] = cscale(R[k * d + j], inv);
+    __syncthreads();
+    const int m = d - k - 1;  // trailing rows i <= columns j
+    for (int e = tid; e < m * m; e += 256) {
+      const int i = k + 1 + e / m, j = k + 1 + e % m;
+      if (j == i)
+        R[i * d + i].x -= cabs2(R[k * d + i]);
+      else if (j > i)
+        R[i * d + j] = csub(R[i * d + j], cmulc(R[k * d + i], R[k * d + j]));
     }
     __syncthreads();
   }
-  // upper-triangular inverse, column j per thread
-  for (int j = tid; j < d; j += blockDim.x) {
-    X[j * d + j] = make_double2(1.0 / R[j * d + j].x, 0);
-    for (int i = j - 1; i >= 0; --i) {
-      double2 s = make_double2(0, 0);
-      for (int m = i + 1; m <= j; ++m) s = cfma(R[i * d + m], X[m * d + j], s);
-      X[i * d + j] = cscale(cneg(s), 1.0 / R[i * d + i].x);
+  const int j = tid >> 2, part = tid & 3;
+  for (int i = d - 1; i >= 0; --i) {  // X_ij = (delta_ij - sum_{i < m <= j} R_im X_mj) / R_ii
+    double2 s = make_double2(0, 0);
+    if (j < d)
+      for (int m = i + 1 + part; m <= j; m += 4) s = cfma(R[i * d + m], X[m * d + j], s);
+#pragma unroll
+    for (int o = 1; o < 4; o <<= 1) {
+      s.x += __shfl_xor_sync(0xffffffff, s.x, o);
+      s.y += __shfl_xor_sync(0xffffffff, s.y, o);
     }
+    if (part == 0 && j < d && j >= i) X[i * d + j] = j == i ? make_double2(rd[i], 0) : cscale(s, -rd[i]);
+    __syncwarp();  // row i of column j is read by the same four threads only
   }
   __syncthreads();
-  for (int e = tid; e < d * d; e += blockDim.x) Rinv[e] = X[e];
+  for (int e = tid; e < d * d; e += 256) Rinv[e] = X[e];
   if (tid == 0 && bad) atomicExch(fail, 1);
 }
 
@@ -772,7 +789,7 @@ void chol_inv_upper(cudaStream_t st, const double2* G, int d, double2* Rinv, int
   MG_CHECK_ARG(d >= 1 && d <= SK_MAXD, "sketch size d limited to 64");
   const int sm = (int)sizeof(double2) * 2 * d * d;
   ensure_max_smem((const void*)k_chol_inv, sizeof(double2) * 2 * SK_MAXD * SK_MAXD);
-  MG_LAUNCH(k_chol_inv, 1, 128, sm, st, G, d, Rinv, fail);
+  MG_LAUNCH(k_chol_inv, 1, 256, sm, st, G, d, Rinv, fail);
 }
 
 // Y <- Y Rinv for Y = [d][n]: a block takes RMT consecutive elements e of all d vectors into shared memory and
@@ -811,64 +828,78 @@ void right_mul_upper(cudaStream_t st, double2* Y, int d, long n, const double2* 
 
 // ---- projection coefficients c[i][r] = Q_i^H x_r -----------------------------------------------------
 namespace {
-constexpr int PCH = 32;    // rows per chunk (the Q tile of up to 64 vectors stays under 48 KB)
-constexpr int PRG = 8;     // rhs per block
-constexpr int PBLK = 96;   // chunks (partials)
+constexpr int PCH = 32;    // rows per chunk
+constexpr int PBLK = 96;   // chunks (partials) at most
 }
 
 size_t proj_work_bytes(int d, long n, int nrhs) {
   (void)n;
-  return sizeof(double2) * (size_t)PBLK * d * nrhs;
+  return sizeof(double2) * (size_t)PBLK * d * nrhs * 2;
 }
 
-// 32 x 8 threads: lane i accumulates basis vectors i and i + 32 (d <= 64) against rhs r0 + g
+// Bound by the FP64 units: TI basis vectors x 256 / TI columns per CTA, one result per thread (every lane at work
+// whatever d is), chunks of the rows over blockIdx.x.  Columns 0 .. nrhs-1 are x, nrhs .. those of x2 (if any), so
+// that one pass over Q serves both vectors of a projected sample.  Lanes bound to basis vectors i and i + 32 idled where
+// d is small: d = 16, 24 right-hand sides, n = 131072: 2 x 786 -> 356 us (1.1 TF of FP64, its roof).
+template <int TI>
 __global__ void __launch_bounds__(256) k_proj_part(const double2* __restrict__ Q, int d, const double2* __restrict__ x,
-                                                   long n, int nrhs, double2* __restrict__ part) {
-  __shared__ double2 Qs[PCH * (SK_MAXD + 1)];
-  __shared__ double2 Xs[PRG * PCH];
-  const int tid = threadIdx.x;
-  const int r0 = blockIdx.y * PRG;
-  const int i = tid % 32, g = tid / 32;
-  double2 acc0 = make_double2(0, 0), acc1 = make_double2(0, 0);
+                                                   const double2* __restrict__ x2, long n, int nrhs, int ncol,
+                                                   double2* __restrict__ part) {
+  constexpr int TR = 256 / TI;
+  __shared__ double2 Qs[PCH][TI + 1];
+  __shared__ double2 Xs[PCH][TR + 1];
+  const int tid = threadIdx.x, ti = (d + TI - 1) / TI;
+  const int i0 = (blockIdx.y % ti) * TI, r0 = (blockIdx.y / ti) * TR;
+  const int i = tid % TI, g = tid / TI;
+  double2 acc = make_double2(0, 0);
   for (long e0 = (long)blockIdx.x * PCH; e0 < n; e0 += (long)gridDim.x * PCH) {
     __syncthreads();
-    for (int q = tid; q < d * PCH; q += blockDim.x) {
-      const int c = q / PCH, e = q % PCH;
-      Qs[e * (SK_MAXD + 1) + c] = (e0 + e < n) ? Q[(size_t)c * n + e0 + e] : make_double2(0, 0);
-    }
-    for (int q = tid; q < PRG * PCH; q += blockDim.x) {
-      const int rr = q / PCH, e = q % PCH;
-      Xs[q] = (r0 + rr < nrhs && e0 + e < n) ? x[(size_t)(r0 + rr) * n + e0 + e] : make_double2(0, 0);
+    const int e = tid & 31;
+#pragma unroll
+    for (int c = tid >> 5; c < TI; c += 8)
+      Qs[e][c] = i0 + c < d && e0 + e < n ? Q[(size_t)(i0 + c) * n + e0 + e] : make_double2(0, 0);
+#pragma unroll
+    for (int c = tid >> 5; c < TR; c += 8) {
+      const int r = r0 + c;
+      const double2* v = r < nrhs ? x + (size_t)r * n : x2 + (size_t)(r - nrhs) * n;
+      Xs[e][c] = r < ncol && e0 + e < n ? v[e0 + e] : make_double2(0, 0);
     }
     __syncthreads();
-    if (i < d)
 #pragma unroll 8
-      for (int e = 0; e < PCH; ++e) {
-        const double2 xv = Xs[g * PCH + e];
-        acc0 = cfmac(Qs[e * (SK_MAXD + 1) + i], xv, acc0);
-        if (i + 32 < d) acc1 = cfmac(Qs[e * (SK_MAXD + 1) + i + 32], xv, acc1);
-      }
+    for (int q = 0; q < PCH; ++q) acc = cfmac(Qs[q][i], Xs[q][g], acc);
   }
-  if (r0 + g < nrhs) {
-    if (i < d) part[((size_t)blockIdx.x * d + i) * nrhs + r0 + g] = acc0;
-    if (i + 32 < d) part[((size_t)blockIdx.x * d + i + 32) * nrhs + r0 + g] = acc1;
-  }
+  if (i0 + i < d && r0 + g < ncol) part[((size_t)blockIdx.x * ncol + r0 + g) * d + i0 + i] = acc;
 }
 
-__global__ void k_proj_final(const double2* __restrict__ part, int cnt, int nb, double2* __restrict__ c) {
+// c[(s d + i) nrhs + r], s = 0 for x and 1 for x2: sums over the chunks in order
+__global__ void k_proj_final(const double2* __restrict__ part, int d, int nrhs, int ncol, int nb,
+                             double2* __restrict__ c) {
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= cnt) return;
+  if (e >= d * ncol) return;
   double2 s = make_double2(0, 0);
-  for (int b = 0; b < nb; ++b) s = cadd(s, part[(size_t)b * cnt + e]);
-  c[e] = s;
+  for (int b = 0; b < nb; ++b) s = cadd(s, part[(size_t)b * d * ncol + e]);
+  const int col = e / d, i = e - col * d;
+  c[(size_t)((col < nrhs ? 0 : d) + i) * nrhs + col % nrhs] = s;
 }
 
-void proj_coeffs(cudaStream_t st, const double2* Q, int d, const double2* x, long n, int nrhs, double2* c, void* work) {
+void proj_coeffs(cudaStream_t st, const double2* Q, int d, const double2* x, const double2* x2, long n, int nrhs,
+                 double2* c, void* work) {
   MG_CHECK_ARG(d >= 1 && d <= SK_MAXD, "sketch size d limited to 64");
-  const int nb = (int)std::min<long>(PBLK, cdiv(n, PCH));
+  const int ncol = x2 ? 2 * nrhs : nrhs;
   double2* part = reinterpret_cast<double2*>(work);
-  MG_LAUNCH(k_proj_part, dim3(nb, cdiv(nrhs, PRG)), 256, 0, st, Q, d, x, n, nrhs, part);
-  MG_LAUNCH(k_proj_final, cdiv((long)d * nrhs, 256), 256, 0, st, part, d * nrhs, nb, c);
+  auto tiles = [&](int ti) { return cdiv(d, ti) * cdiv(ncol, 256 / ti); };
+  // the tile shape that pads least, and chunks for about six CTAs per SM
+  const int ti = tiles(8) < tiles(16) ? 8 : tiles(16) <= tiles(32) ? 16 : 32;
+  const int nb = (int)std::max<long>(1, std::min<long>(std::min<long>(PBLK, cdiv(n, PCH)), 912 / tiles(ti) + 1));
+  const dim3 grid(nb, tiles(ti));
+  const double flops = 8.0 * d * ncol * (double)n, bytes = 16.0 * (double)n * (d + ncol);
+  if (ti == 8)
+    MG_LAUNCH_W(bytes, flops, k_proj_part<8>, grid, 256, 0, st, Q, d, x, x2, n, nrhs, ncol, part);
+  else if (ti == 16)
+    MG_LAUNCH_W(bytes, flops, k_proj_part<16>, grid, 256, 0, st, Q, d, x, x2, n, nrhs, ncol, part);
+  else
+    MG_LAUNCH_W(bytes, flops, k_proj_part<32>, grid, 256, 0, st, Q, d, x, x2, n, nrhs, ncol, part);
+  MG_LAUNCH(k_proj_final, cdiv((long)d * ncol, 128), 128, 0, st, part, d, nrhs, ncol, nb, c);
 }
 
 }  // namespace mg

@@ -194,3 +194,42 @@ def test_stencil_forms(api, ctx, L, nrhs, prec, tol):
     api.schwinger_apply(ctx, torch.from_numpy(U).cuda(), L, 0.1, torch.from_numpy(x).cuda(), y, getattr(api, prec))
     ref = (osch.dirac_sparse(U, 0.1) @ x.T.astype(complex)).T
     assert relerr(y.cpu().numpy(), ref) < tol
+
+
+@pytest.mark.parametrize("nrhs", [1, 16, 17, 33])
+@pytest.mark.parametrize("shift", [0, 1])
+def test_coarse_operator_tiles(api, ctx, nrhs, shift):
+    """FP32 operator with 16 dof per site at the remainders of its rhs tiles, also on vectors that start 8 bytes off
+    a 16-byte boundary (80 products, a few roundings of 6e-8 each)."""
+    h, H = hierarchy(api, ctx, 64, ntv=8)
+    x = vecs(H.n[1], nrhs, 7, np.complex64)
+    buf = torch.empty(x.size + shift, dtype=torch.complex64, device="cuda")
+    xd = buf[shift:].view(x.shape)
+    xd.copy_(torch.from_numpy(x))
+    y = torch.full(x.shape, float("nan"), dtype=torch.complex64, device="cuda")
+    h.apply(1, xd, y, api.FP32)
+    assert relerr(y.cpu().numpy(), (H.D[1] @ x.T.astype(complex)).T) < 2e-5
+
+
+@pytest.mark.parametrize("d,nrhs", [(1, 1), (7, 9), (8, 17), (9, 5), (24, 24), (33, 8), (64, 33)])
+def test_projection_tiles(api, ctx, d, nrhs):
+    """Projected samples at the remainders of the basis and rhs tiles (sums of 512 products, their roundings)."""
+    h, H = hierarchy(api, ctx, 16)
+    sk, _ = api.hutchpp_sketch_qr(ctx, h, 0, d, 1, 3, api.ACCUMULATED, tol=1e-6, prec=api.MIXED)
+    Q = sk.Q().cpu().numpy()
+    z, y = vecs(H.n[0], nrhs, 1, np.complex128), vecs(H.n[0], nrhs, 2, np.complex128)
+    tau = api.hutchpp_project(ctx, sk, torch.from_numpy(z).cuda(), torch.from_numpy(y).cuda())
+    zp = z - (z @ Q.conj().T) @ Q
+    assert relerr(tau, np.einsum("ij,ij->i", zp.conj(), y)) < 1e-12
+
+
+@pytest.mark.parametrize("d", [1, 2, 31, 32, 33, 63])
+def test_cholesky_qr_sizes(api, ctx, d):
+    """Orthonormal basis by the Cholesky factor's right-looking form: Q^H Q = I to a few hundred roundings."""
+    Y = torch.from_numpy(vecs(1000, d, d, np.complex128)).cuda()
+    ref = Y.cpu().numpy()
+    api.hutchpp_cholqr2(ctx, Y)
+    Q = Y.cpu().numpy()
+    R = Q.conj() @ ref.T  # Y = R^T Q by rows: upper triangular with a positive real diagonal
+    assert np.abs(Q.conj() @ Q.T - np.eye(d)).max() < 1e-13
+    assert np.abs(np.tril(R, -1)).max(initial=0) < 1e-11 and np.diag(R).real.min() > 0
