@@ -137,7 +137,8 @@ int schwinger_apply(mgmlmc_ctx* ctx, const double* U, int L, double m0, const vo
     const double diag = m0 + 2.0;
     // Up to 64 K sites x rhs the operator reads U itself (twice the link bytes and 8 FP64 multiplications a site, but
     // one launch and no workspace: 10 us a call before, of which the operator 4); longer batches prepare the links
-    // once per call, in a workspace of the context.
+    // once per call, in a workspace of the context.  Inside a stream capture the workspace belongs to the capture
+    // (memory allocated there exists only while its graph runs), so it is not kept.
     if ((int64_t)L * L * nrhs <= 65536) {
       if (prec == MGMLMC_FP32)
         wilson_apply_raw<float>(st, (const double2*)U, (float)diag, L, (const float2*)x, (float2*)y, nrhs);
@@ -145,8 +146,17 @@ int schwinger_apply(mgmlmc_ctx* ctx, const double* U, int L, double m0, const vo
         wilson_apply_raw<double>(st, (const double2*)U, diag, L, (const double2*)x, (double2*)y, nrhs);
       return;
     }
-    double2* l64 = (double2*)ctx->work("sa_links64", sizeof(double2) * 2 * L * L);
-    float2* l32 = prec == MGMLMC_FP32 ? (float2*)ctx->work("sa_links32", sizeof(float2) * 2 * L * L) : nullptr;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    const bool own = cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone;
+    if (own) cudaGetLastError();
+    std::unique_lock<std::mutex> lock(ctx->links_mutex, std::defer_lock);
+    DBuf own64, own32;
+    if (!own) lock.lock();
+    DBuf &b64 = own ? own64 : ctx->links64, &b32 = own ? own32 : ctx->links32;
+    b64.ensure(sizeof(double2) * 2 * L * L, st);
+    if (prec == MGMLMC_FP32) b32.ensure(sizeof(float2) * 2 * L * L, st);
+    double2* l64 = b64.as<double2>();
+    float2* l32 = prec == MGMLMC_FP32 ? b32.as<float2>() : nullptr;
     prepare_links(st, (const double2*)U, L, l64, l32);
     if (prec == MGMLMC_FP32)
       wilson_apply<float>(st, l32, (float)diag, L, (const float2*)x, (float2*)y, nullptr, nrhs, nullptr);

@@ -222,8 +222,12 @@ struct DBuf {
   void alloc(size_t b, cudaStream_t s) {
     release();
     st = s;
+    if (b) {
+      const cudaError_t e = cudaMallocAsync(&p, b, s);
+      if (e != cudaSuccess) p = nullptr;  // a buffer that is kept stays empty, and the next call asks again
+      MG_CUDA(e);
+    }
     bytes = b;
-    if (b) MG_CUDA(cudaMallocAsync(&p, b, s));
   }
   void ensure(size_t b, cudaStream_t s) { if (b > bytes) alloc(b, s); }
   void release() {

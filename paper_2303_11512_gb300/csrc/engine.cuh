@@ -4,6 +4,7 @@
 
 #include <map>
 #include <memory>
+#include <mutex>
 #include <string>
 #include <tuple>
 #include <vector>
@@ -21,6 +22,8 @@ struct mgmlmc_ctx {
   double* pinned_d = nullptr;
   mg::KTimer timer;
   std::map<std::string, mg::DBuf> ws;  // workspaces of calls that have no hierarchy (projection)
+  mg::DBuf links64, links32;           // prepared links of schwinger_apply; launches that use them are issued under
+  std::mutex links_mutex;              // this lock, so that calls of several host threads stay whole on the stream
   void* work(const std::string& tag, size_t bytes) {
     auto& b = ws[tag];
     if (bytes > b.bytes) b.alloc(bytes, stream);

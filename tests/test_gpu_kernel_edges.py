@@ -233,3 +233,27 @@ def test_cholesky_qr_sizes(api, ctx, d):
     R = Q.conj() @ ref.T  # Y = R^T Q by rows: upper triangular with a positive real diagonal
     assert np.abs(Q.conj() @ Q.T - np.eye(d)).max() < 1e-13
     assert np.abs(np.tril(R, -1)).max(initial=0) < 1e-11 and np.diag(R).real.min() > 0
+
+
+def test_stencil_in_a_stream_capture(api):
+    """The first call of a context inside a stream capture keeps nothing of the capture's memory: calls after it, and
+    replays, give the same values as a call of another context."""
+    L, nrhs = 128, 8
+    U = torch.from_numpy(np.exp(1j * np.random.default_rng(0).uniform(-3, 3, (L, L, 2)))).cuda()
+    x = torch.from_numpy(vecs(2 * L * L, nrhs, 3, np.complex128)).cuda()
+    ref, y, z = (torch.zeros_like(x) for _ in range(3))
+    c = api.Context()
+    api.schwinger_apply(c, U, L, 0.1, x, ref, api.FP64)
+    c.close()
+    s = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    c = api.Context(s)
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=s):
+        api.schwinger_apply(c, U, L, 0.1, x, y, api.FP64)
+    api.schwinger_apply(c, U, L, 0.1, x, z, api.FP64)
+    with torch.cuda.stream(s):
+        g.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(z, ref) and torch.equal(y, ref)
+    c.close()
