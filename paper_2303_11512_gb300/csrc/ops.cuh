@@ -167,6 +167,9 @@ size_t gram_work_bytes(int d, long n);
 void chol_inv_upper(cudaStream_t st, const double2* G, int d, double2* Rinv, int* fail);
 // Y <- Y Rinv (in place, Rinv upper triangular)
 void right_mul_upper(cudaStream_t st, double2* Y, int d, long n, const double2* Rinv);
+// Kernels with tiles of 8 or more right-hand sides in grid.y (at most 65535) take longer batches in slices.
+constexpr int RHS_SLICE = 1 << 18;
+
 // c[i][rhs] = Q_i^H x_rhs, Q = [d][n], x = [nrhs][n]; x2 (or nullptr): the same for it, c[d + i][rhs]
 void proj_coeffs(cudaStream_t st, const double2* Q, int d, const double2* x, const double2* x2, long n, int nrhs,
                  double2* c, void* work);

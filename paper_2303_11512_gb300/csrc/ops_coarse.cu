@@ -174,6 +174,15 @@ void coarse_apply(cudaStream_t stm, const typename CT<R>::T* st, int Ls, int d, 
                   typename CT<R>::T* y, const typename CT<R>::T* b, int nrhs, const int* active) {
   typedef typename CT<R>::T C;
   MG_CHECK_ARG(d <= 64 && 256 % d == 0, "coarse dof must divide 256");
+  if (nrhs > RHS_SLICE) {
+    for (int r = 0; r < nrhs; r += RHS_SLICE) {
+      const int k = std::min(RHS_SLICE, nrhs - r);
+      const int* act = active ? active + r : nullptr;
+      const size_t n = (size_t)Ls * Ls * d;
+      coarse_apply<R>(stm, st, Ls, d, x + r * n, y + r * n, b ? b + r * n : nullptr, k, act);
+    }
+    return;
+  }
   const int G = 256 / d;
   size_t sm = sizeof(C) * (5 * d * d + G * 5 * d);
   const double ns = (double)Ls * Ls, cs = sizeof(C), ar = act_rhs(nrhs);
@@ -364,6 +373,15 @@ void sap_half_coarse(cudaStream_t stm, const typename CT<R>::T* st, int Ls, int 
   if (nrhs <= 0) return;
   const SapCoarseShape sh(bs, d);
   MG_CHECK_ARG(sh.bd <= 64, "coarse SAP blocks have at most 64 unknowns");
+  if (nrhs > RHS_SLICE) {
+    for (int r = 0; r < nrhs; r += RHS_SLICE) {
+      const int k = std::min(RHS_SLICE, nrhs - r);
+      const int* act = active ? active + r : nullptr;
+      const size_t n = (size_t)Ls * Ls * d;
+      sap_half_coarse<R>(stm, st, Ls, d, bs, inv, f + r * n, x + r * n, color, k, act, zero);
+    }
+    return;
+  }
   const size_t sm = sizeof(C) * (size_t)sh.complexes(sizeof(R) == 4);
   const int nb = (Ls / bs) * (Ls / bs) / 2;
   const double cs = sizeof(C), ar = act_rhs(nrhs), ext = zero ? 0.0 : sh.nslot * (double)d * d;
@@ -623,6 +641,15 @@ void restrict_op(cudaStream_t stm, const typename CT<R>::T* P, int Ls, int d, in
   typedef typename CT<R>::T C;
   if (nrhs <= 0) return;
   const int na = agg * agg, bsz = na * d / 2, dc = 2 * ntv;
+  if (nrhs > RHS_SLICE) {
+    for (int r = 0; r < nrhs; r += RHS_SLICE) {
+      const int k = std::min(RHS_SLICE, nrhs - r);
+      const int* act = active ? active + r : nullptr;
+      const size_t nf = (size_t)Ls * Ls * d;
+      restrict_op<R>(stm, P, Ls, d, agg, ntv, xf + r * nf, xc + r * (nf / (na * d) * dc), k, act, half);
+    }
+    return;
+  }
   const int Lc = Ls / agg;
   const double nag = (double)Lc * Lc, cs = sizeof(C), ar = act_rhs(nrhs);
   const double bytes = nag * (ar * (na * d * (half ? 0.5 : 1.0) + dc) * cs + 2.0 * bsz * ntv * cs);
@@ -688,6 +715,16 @@ void prolong_op(cudaStream_t stm, const typename CT<R>::T* P, int Ls, int d, int
   typedef typename CT<R>::T C;
   if (nrhs <= 0) return;
   const int na = agg * agg, bsz = na * d / 2, dc = 2 * ntv, fa = na * d;
+  if (nrhs > RHS_SLICE) {
+    for (int r = 0; r < nrhs; r += RHS_SLICE) {
+      const int k = std::min(RHS_SLICE, nrhs - r);
+      const int* act = active ? active + r : nullptr;
+      const size_t nf = (size_t)Ls * Ls * d;
+      prolong_op<R>(stm, P, Ls, d, agg, ntv, xc + r * (nf / fa * dc), xf + r * nf, add, k, act,
+                    xf16 ? (unsigned short*)xf16 + 2 * r * nf : nullptr, bf);
+    }
+    return;
+  }
   const int Lc = Ls / agg;
   const double nag = (double)Lc * Lc, cs = sizeof(C), ar = act_rhs(nrhs);
   const double bytes = nag * (ar * ((add ? 2.0 : 1.0) * fa + dc) * cs + 2.0 * bsz * ntv * cs) +

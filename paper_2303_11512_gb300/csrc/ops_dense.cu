@@ -611,6 +611,14 @@ void dense_apply(cudaStream_t st, const typename CT<R>::T* A, int n, const typen
                  typename CT<R>::T* y, int nrhs, const int* active) {
   typedef typename CT<R>::T C;
   if (nrhs <= 0) return;
+  if (nrhs > RHS_SLICE) {
+    for (int r = 0; r < nrhs; r += RHS_SLICE) {
+      const int k = std::min(RHS_SLICE, nrhs - r);
+      const int* act = active ? active + r : nullptr;
+      dense_apply<R>(st, A, n, x + (size_t)r * n, y + (size_t)r * n, k, act);
+    }
+    return;
+  }
   const double bytes = ((double)n * n + 2.0 * act_rhs(nrhs) * n) * sizeof(C), flops = 8.0 * n * (double)n * act_rhs(nrhs);
   auto go = [&](auto ri, auto nr) {
     constexpr int RI = decltype(ri)::value, NR = decltype(nr)::value;
@@ -838,7 +846,7 @@ size_t proj_work_bytes(int d, long n, int nrhs) {
 }
 
 // Bound by the FP64 units: TI basis vectors x 256 / TI columns per CTA, one result per thread (every lane at work
-// whatever d is), chunks of the rows over blockIdx.x.  Columns 0 .. nrhs-1 are x, nrhs .. those of x2 (if any), so
+// whatever d is), chunks of the rows over blockIdx.y.  Columns 0 .. nrhs-1 are x, nrhs .. those of x2 (if any), so
 // that one pass over Q serves both vectors of a projected sample.  Lanes bound to basis vectors i and i + 32 idled where
 // d is small: d = 16, 24 right-hand sides, n = 131072: 2 x 786 -> 356 us (1.1 TF of FP64, its roof).
 template <int TI>
@@ -849,10 +857,10 @@ __global__ void __launch_bounds__(256) k_proj_part(const double2* __restrict__ Q
   __shared__ double2 Qs[PCH][TI + 1];
   __shared__ double2 Xs[PCH][TR + 1];
   const int tid = threadIdx.x, ti = (d + TI - 1) / TI;
-  const int i0 = (blockIdx.y % ti) * TI, r0 = (blockIdx.y / ti) * TR;
+  const int i0 = (blockIdx.x % ti) * TI, r0 = (blockIdx.x / ti) * TR;
   const int i = tid % TI, g = tid / TI;
   double2 acc = make_double2(0, 0);
-  for (long e0 = (long)blockIdx.x * PCH; e0 < n; e0 += (long)gridDim.x * PCH) {
+  for (long e0 = (long)blockIdx.y * PCH; e0 < n; e0 += (long)gridDim.y * PCH) {
     __syncthreads();
     const int e = tid & 31;
 #pragma unroll
@@ -868,7 +876,7 @@ __global__ void __launch_bounds__(256) k_proj_part(const double2* __restrict__ Q
 #pragma unroll 8
     for (int q = 0; q < PCH; ++q) acc = cfmac(Qs[q][i], Xs[q][g], acc);
   }
-  if (i0 + i < d && r0 + g < ncol) part[((size_t)blockIdx.x * ncol + r0 + g) * d + i0 + i] = acc;
+  if (i0 + i < d && r0 + g < ncol) part[((size_t)blockIdx.y * ncol + r0 + g) * d + i0 + i] = acc;
 }
 
 // c[(s d + i) nrhs + r], s = 0 for x and 1 for x2: sums over the chunks in order
@@ -891,7 +899,7 @@ void proj_coeffs(cudaStream_t st, const double2* Q, int d, const double2* x, con
   // the tile shape that pads least, and chunks for about six CTAs per SM
   const int ti = tiles(8) < tiles(16) ? 8 : tiles(16) <= tiles(32) ? 16 : 32;
   const int nb = (int)std::max<long>(1, std::min<long>(std::min<long>(PBLK, cdiv(n, PCH)), 912 / tiles(ti) + 1));
-  const dim3 grid(nb, tiles(ti));
+  const dim3 grid(tiles(ti), nb);
   const double flops = 8.0 * d * ncol * (double)n, bytes = 16.0 * (double)n * (d + ncol);
   if (ti == 8)
     MG_LAUNCH_W(bytes, flops, k_proj_part<8>, grid, 256, 0, st, Q, d, x, x2, n, nrhs, ncol, part);

@@ -246,6 +246,14 @@ template <typename R>
 void wilson_apply(cudaStream_t st, const typename CT<R>::T* links, R diag, int L, const typename CT<R>::T* x,
                   typename CT<R>::T* y, const typename CT<R>::T* b, int nrhs, const int* active) {
   if (nrhs <= 0) return;
+  if (nrhs > 65535) {  // one row of the grid per rhs
+    for (int r = 0; r < nrhs; r += 65535) {
+      const size_t n = 2 * (size_t)L * L;
+      wilson_apply<R>(st, links, diag, L, x + r * n, y + r * n, b ? b + r * n : nullptr, std::min(65535, nrhs - r),
+                      active ? active + r : nullptr);
+    }
+    return;
+  }
   // algorithmic traffic: x read + y written once per site and rhs (+ b), links once per launch
   const double V = (double)L * L, sp = 2.0 * sizeof(typename CT<R>::T), ar = act_rhs(nrhs);
   const double bytes = ar * V * sp * (b ? 3 : 2) + V * sp;
@@ -690,6 +698,14 @@ void sap_half_fine(cudaStream_t st, const typename CT<R>::T* links, R diag, int 
                    int nrhs, const int* active, bool inv_transposed, int known) {
   MG_CHECK_ARG(bs == 4 || bs == 2, "fine SAP block side must be 2 or 4");
   if (nrhs <= 0) return;
+  if (nrhs > RHS_SLICE) {
+    for (int r = 0; r < nrhs; r += RHS_SLICE) {
+      const size_t n = 2 * (size_t)L * L;
+      sap_half_fine<R>(st, links, diag, L, bs, inv, f + r * n, x + r * n, color, std::min(RHS_SLICE, nrhs - r),
+                       active ? active + r : nullptr, inv_transposed, known);
+    }
+    return;
+  }
   const int nb = (L / bs) * (L / bs) / 2;
   // per block and rhs: f and the surrounding x read, x written on the block (bd complex each); inverse once per block
   const double bd = 2.0 * bs * bs, cs = sizeof(typename CT<R>::T), ar = act_rhs(nrhs);
@@ -744,6 +760,15 @@ void residual_restrict_fine(cudaStream_t st, const float2* links, float diag, in
                             const float2* f, float2* xc, int nrhs, const int* active) {
   MG_CHECK_ARG(L % 4 == 0, "4 x 4 aggregates");
   if (nrhs <= 0) return;
+  if (nrhs > RHS_SLICE) {
+    for (int r = 0; r < nrhs; r += RHS_SLICE) {
+      const int k = std::min(RHS_SLICE, nrhs - r);
+      const int* act = active ? active + r : nullptr;
+      const size_t n = 2 * (size_t)L * L;
+      residual_restrict_fine(st, links, diag, L, P, x + r * n, f + r * n, xc + r * (n / 2), k, act);
+    }
+    return;
+  }
   const int na = (L / 4) * (L / 4);
   const double ar = act_rhs(nrhs);
   const double bytes = na * (ar * (16 * 16 * 2 + 128.0) + 2048.0), flops = na * ar * (16 * 56.0 + 8.0 * 256);

@@ -257,3 +257,29 @@ def test_stencil_in_a_stream_capture(api):
     torch.cuda.synchronize()
     assert torch.equal(z, ref) and torch.equal(y, ref)
     c.close()
+
+
+def test_batches_beyond_the_grid(api, ctx):
+    """Operators, transfers and smoothers on more right-hand sides than one grid holds tiles of: the last ones equal a
+    batch of their own (the same sums, up to a few roundings of 6e-8 in another tile shape)."""
+    h, H = hierarchy(api, ctx, 16, ntv=8)
+    nrhs, k = 16 * 65535 + 5, 7
+    f = torch.zeros((nrhs, H.n[1]), dtype=torch.complex64, device="cuda")
+    f[-k:] = torch.from_numpy(vecs(H.n[1], k, 1, np.complex64)).cuda()
+    out, ref = torch.empty_like(f), torch.empty_like(f[-k:])
+    h.apply(1, f, out, api.FP32)
+    h.apply(1, f[-k:].clone(), ref, api.FP32)
+    assert relerr(out[-k:].cpu().numpy(), ref.cpu().numpy()) < 2e-6
+    del out
+    fine = torch.zeros((nrhs, H.n[0]), dtype=torch.complex64, device="cuda")
+    fref = torch.empty((k, H.n[0]), dtype=torch.complex64, device="cuda")
+    h.prolong(0, f, fine, api.FP32)
+    h.prolong(0, f[-k:].clone(), fref, api.FP32)
+    assert relerr(fine[-k:].cpu().numpy(), fref.cpu().numpy()) < 2e-6
+    h.restrict(0, fine, f, api.FP32)
+    h.restrict(0, fref, ref, api.FP32)
+    assert relerr(f[-k:].cpu().numpy(), ref.cpu().numpy()) < 2e-6
+    x, xref = torch.zeros_like(fine), torch.zeros_like(fref)
+    h.smooth(0, fine, x, api.FP32, 1)
+    h.smooth(0, fref, xref, api.FP32, 1)
+    assert relerr(x[-k:].cpu().numpy(), xref.cpu().numpy()) < 2e-6
