@@ -110,14 +110,15 @@ inline double act_rhs(int nrhs) { return (g_nact_hint >= 0 && g_nact_hint < nrhs
 // kernel wrote is not read through __restrict__ const pointers or __ldg, whose loads need not stay behind it); it
 // also lets the next kernel be placed.  Used by the kernels of a V-cycle, where a launch below PDL_BYTES takes 5 to
 // 12 us of which this hides about 2 (V(1,1) at L = 128 with 5 right-hand sides: 157 -> 129 us).  Larger launches lose
-// by it (V(2,2) at L = 512 with 32: 1.82 -> 1.93 ms with every launch, 1.79 with those below 24 MB, 1.81 below 8 MB),
-// and in a graph there is nothing left to hide.
+// by it (V(2,2) at L = 512 with 32: 1.82 -> 1.93 ms with every launch, 1.79 with those below 24 MB, 1.81 below 8 MB).
+// A stream capture, the library's own or a caller's, gets plain launches: in a graph there is nothing left to hide, and
+// some of these kernels follow a memset node, which a programmatic edge cannot start from.
 __device__ __forceinline__ void pdl_begin() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 constexpr double PDL_BYTES = 24e6;
-extern thread_local bool g_capturing;  // launches go into a graph
+extern thread_local bool g_capturing;  // launches go into a graph (looked up on entry of every call)
 template <typename... Par, typename... Arg>
 inline void launch_pdl(bool early, void (*kernel)(Par...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
                        Arg&&... arg) {

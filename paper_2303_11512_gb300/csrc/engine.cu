@@ -233,20 +233,23 @@ static void vcycle_maybe_graph(mgmlmc_hier* h, int l, const typename CT<R>::T* i
     if (!h->capture_stream) MG_CUDA(cudaStreamCreateWithFlags(&h->capture_stream, cudaStreamNonBlocking));
     cudaStream_t cs = h->capture_stream;
     MG_CUDA(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
+    const bool outer = g_capturing;
     h->capturing = g_capturing = true;
     h->ctx->stream = cs;  // the V-cycle's launches go to the capturing stream
     try {
       vcycle<R>(h, l, gin, gout, nrhs, active);
     } catch (...) {
       h->ctx->stream = st;
-      h->capturing = g_capturing = false;
+      h->capturing = false;
+      g_capturing = outer;
       cudaStreamEndCapture(cs, &graph);
       if (graph) cudaGraphDestroy(graph);
       cudaGetLastError();
       throw;
     }
     h->ctx->stream = st;
-    h->capturing = g_capturing = false;
+    h->capturing = false;
+    g_capturing = outer;
     MG_CUDA(cudaStreamEndCapture(cs, &graph));
     const int64_t captured = g_launch_counter ? *g_launch_counter - before : 0;
     if (g_launch_counter) *g_launch_counter = before;  // capturing issued nothing

@@ -131,6 +131,7 @@ struct LaunchScope {
     g_launch_counter = nullptr;
     g_timer = nullptr;
     g_nact_hint = -1;
+    g_capturing = false;
   }
 };
 
