@@ -242,5 +242,11 @@ struct DBuf {
 };
 
 inline unsigned cdiv(long a, long b) { return (unsigned)((a + b - 1) / b); }
+inline int sm_count() {  // of the current device
+  int dev = 0, n = 0;
+  MG_CUDA(cudaGetDevice(&dev));
+  MG_CUDA(cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev));
+  return n;
+}
 
 }  // namespace mg

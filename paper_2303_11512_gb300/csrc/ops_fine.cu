@@ -563,17 +563,24 @@ __global__ void __launch_bounds__(64) k_sap_fine4_fp32(const float2* __restrict_
 
 // FP64, 4 x 4 blocks: bound by the FP64 units (two FMAs a clock and SM).  The blocks of one colour do not couple, so
 // with E the hops that leave the block x_B + D_BB^{-1} (f - D x)_B = D_BB^{-1} (f - E x)_B: the hops inside the block
-// and the old x_B drop out.  One CTA of two warps per block, tiles of RG right-hand sides; a thread owns two sites
-// (4 complex rows) times RG / 8 rhs.
-template <int RG>
+// and the old x_B drop out.  One CTA of two warps per block and tile of at most 16 right-hand sides.  A lane owns a row
+// of the block and a warp takes every second live right-hand side of the tile, up to four at a time, so that neither the
+// remainder of a tile nor a right-hand side that has stopped costs FMAs, and the hops have loops of their own, in which
+// every lane has one.  With whole tiles of 8 and 16 in threads of 4 rows x 1 or 2 right-hand sides a sweep of one took
+// as long as of eight: at L = 512 with 1, 8, 9, 17, 64 right-hand sides 940, 943, 1860, 3645, 7390 us, now 193, 948,
+// 1118, 2035, 7410 (the products alone 107, 853, 960, 1810, 6825).  Which warp gets the odd one changes from block to
+// block, because a CTA's first warp lands in the same quarters of an SM.
+constexpr int SF64_TILE = 16;
 __global__ void __launch_bounds__(64) k_sap_fine4_fp64(const double2* __restrict__ lk, int L,
                                                        const double2* __restrict__ inv, const double2* __restrict__ f,
-                                                       double2* __restrict__ x, int color, int nrhs, int known,
+                                                       double2* __restrict__ x, int color, int nrhs, int tile, int known,
                                                        const int* __restrict__ active) {
-  constexpr int BD = 32, IS = BD + 1, RS = RG + 1, NR = RG / 8;
+  constexpr int BD = 32, IS = BD + 1;
   __shared__ double2 sinv[BD * IS];  // transposed
-  __shared__ double2 sres[BD * RS];
-  const int tid = threadIdx.x;
+  __shared__ double2 sres[SF64_TILE][BD];
+  __shared__ int srhs[SF64_TILE];  // live right-hand sides of the tile
+  __shared__ int scount;
+  const int tid = threadIdx.x, lane = tid & 31;
   const int nbx = L / 4, half = nbx / 2;
   const int BT = blockIdx.x / half;
   const int BX = 2 * (blockIdx.x - BT * half) + ((BT + color) & 1);
@@ -581,68 +588,66 @@ __global__ void __launch_bounds__(64) k_sap_fine4_fp64(const double2* __restrict
 #pragma unroll 4
   for (int e = tid; e < BD * BD; e += 64) sinv[(e % BD) * IS + e / BD] = I[e];
   const size_t n = 2 * (size_t)L * L;
-  const int g = tid & 7, rg = tid >> 3;  // row group and rhs group of the product
-  for (int r0 = blockIdx.y * RG; r0 < nrhs; r0 += gridDim.y * RG) {
-#pragma unroll 4
-    for (int q = tid; q < 16 * RG; q += 64) {
-      const int jx = q & 3, rr = (q >> 2) % RG, jt = (q >> 2) / RG;
-      const int rhs = r0 + rr;
-      if (rhs < nrhs && !(active && !active[rhs])) {
-        const int t = 4 * BT + jt, xx = 4 * BX + jx, s = t * L + xx;
-        const double2* X = x + rhs * n;
-        double2 o0, o1, a0, a1;
-        ld_sp(f + rhs * n, s, o0, o1);
-        if (known != SAP_ZERO && (jx == 0 || jx == 3)) {  // (1 -+ sigma_1) hop out of the block
-          const int s2 = jx == 3 ? (xx == L - 1 ? s + 1 - L : s + 1) : (xx == 0 ? s + L - 1 : s - 1);
-          ld_sp(X, s2, a0, a1);
-          const double2 w = jx == 3 ? __ldg(lk + 2 * s) : cconj(__ldg(lk + 2 * s2));
-          const double sg = jx == 3 ? -1.0 : 1.0;
-          const double2 u = cmul(w, cadd(a0, cscale(a1, sg)));
-          o0 = csub(o0, u);
-          o1 = csub(o1, cscale(u, sg));
-        }
-        if (known != SAP_ZERO && (jt == 0 || jt == 3)) {  // (1 -+ sigma_2) hop
-          const int s2 = jt == 3 ? (t == L - 1 ? xx : s + L) : (t == 0 ? s + L * (L - 1) : s - L);
-          ld_sp(X, s2, a0, a1);
-          const double2 w = jt == 3 ? __ldg(lk + 2 * s + 1) : cconj(__ldg(lk + 2 * s2 + 1));
-          const double sg = jt == 3 ? 1.0 : -1.0;
-          const double2 u = cmul(w, cadd(a0, cscale(cmuli(a1), sg)));
-          o0 = csub(o0, u);
-          o1 = cadd(o1, cscale(cmuli(u), sg));
-        }
-        const int j = 4 * jt + jx;
-        sres[(2 * j) * RS + rr] = o0;
-        sres[(2 * j + 1) * RS + rr] = o1;
+  const int first = (tid >> 5) ^ ((blockIdx.x * 0x9E3779B1u) >> 31);  // this warp's first slot
+  for (int r0 = blockIdx.y * tile; r0 < nrhs; r0 += gridDim.y * tile) {
+    if (tid < 32) {
+      const bool on = lane < tile && r0 + lane < nrhs && !(active && !active[r0 + lane]);
+      const unsigned m = __ballot_sync(0xffffffffu, on);
+      if (on) srhs[__popc(m & ((1u << lane) - 1))] = r0 + lane;
+      if (lane == 0) scount = __popc(m);
+    }
+    __syncthreads();
+    const int cnt = scount;
+    for (int q = tid; q < 32 * cnt; q += 64)
+      sres[q >> 5][q & 31] = __ldg(f + srhs[q >> 5] * n + 2 * ((size_t)(4 * BT + ((q >> 3) & 3)) * L + 4 * BX) + (q & 7));
+    if (known != SAP_ZERO) {
+      __syncthreads();
+      for (int q = tid; q < 8 * cnt; q += 64) {  // (1 -+ sigma_1) hops out of the block
+        const bool up = q & 1;
+        const int jt = (q >> 1) & 3, j = 4 * jt + (up ? 3 : 0), xx = 4 * BX + (up ? 3 : 0), s = (4 * BT + jt) * L + xx;
+        const int s2 = up ? (xx == L - 1 ? s + 1 - L : s + 1) : (xx == 0 ? s + L - 1 : s - 1);
+        double2 a0, a1;
+        ld_sp(x + srhs[q >> 3] * n, s2, a0, a1);
+        const double2 w = up ? __ldg(lk + 2 * s) : cconj(__ldg(lk + 2 * s2));
+        const double2 u = cmul(w, cadd(a0, up ? cneg(a1) : a1));
+        double2* o = sres[q >> 3] + 2 * j;
+        o[0] = csub(o[0], u);
+        o[1] = csub(o[1], up ? cneg(u) : u);
+      }
+      __syncthreads();
+      for (int q = tid; q < 8 * cnt; q += 64) {  // (1 -+ sigma_2) hops
+        const bool up = q & 4;
+        const int jx = q & 3, j = (up ? 12 : 0) + jx, t = 4 * BT + (up ? 3 : 0), xx = 4 * BX + jx, s = t * L + xx;
+        const int s2 = up ? (t == L - 1 ? xx : s + L) : (t == 0 ? s + L * (L - 1) : s - L);
+        double2 a0, a1;
+        ld_sp(x + srhs[q >> 3] * n, s2, a0, a1);
+        const double2 w = up ? __ldg(lk + 2 * s + 1) : cconj(__ldg(lk + 2 * s2 + 1));
+        const double2 u = cmul(w, cadd(a0, up ? cmuli(a1) : cmulmi(a1)));
+        double2* o = sres[q >> 3] + 2 * j;
+        o[0] = csub(o[0], u);
+        o[1] = cadd(o[1], up ? cmuli(u) : cmulmi(u));
       }
     }
     __syncthreads();
-    double2 acc[4][NR];
+    auto product = [&](int k0, auto nrc) {  // slots k0, k0 + 2, ..
+      constexpr int NR = decltype(nrc)::value;
+      double2 acc[NR];
 #pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-      for (int b = 0; b < NR; ++b) acc[a][b] = make_double2(0, 0);
+      for (int b = 0; b < NR; ++b) acc[b] = make_double2(0, 0);
 #pragma unroll 4
-    for (int j = 0; j < BD; ++j) {
-      const double2* mi = sinv + j * IS;
-      const double2 m[4] = {mi[2 * g], mi[2 * g + 1], mi[16 + 2 * g], mi[17 + 2 * g]};
-      double2 v[NR];
+      for (int j = 0; j < BD; ++j) {
+        const double2 m = sinv[j * IS + lane];
 #pragma unroll
-      for (int b = 0; b < NR; ++b) v[b] = sres[j * RS + rg * NR + b];
-#pragma unroll
-      for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int b = 0; b < NR; ++b) acc[a][b] = cfma(m[a], v[b], acc[a][b]);
-    }
-#pragma unroll
-    for (int b = 0; b < NR; ++b) {
-      const int rhs = r0 + rg * NR + b;
-      if (rhs < nrhs && !(active && !active[rhs])) {
-        double2* X = x + rhs * n;
-        const int s = (4 * BT + (g >> 2)) * L + 4 * BX + (g & 3);
-        st_sp(X, s, acc[0][b], acc[1][b]);
-        st_sp(X, s + 2 * L, acc[2][b], acc[3][b]);
+        for (int b = 0; b < NR; ++b) acc[b] = cfma(m, sres[k0 + 2 * b][j], acc[b]);
       }
-    }
+      const size_t o = 2 * ((size_t)(4 * BT + (lane >> 3)) * L + 4 * BX) + (lane & 7);
+#pragma unroll
+      for (int b = 0; b < NR; ++b) x[srhs[k0 + 2 * b] * n + o] = acc[b];
+    };
+    int k = first;
+    for (; k + 6 < cnt; k += 8) product(k, std::integral_constant<int, 4>());
+    for (; k + 2 < cnt; k += 4) product(k, std::integral_constant<int, 2>());
+    if (k < cnt) product(k, std::integral_constant<int, 1>());
     __syncthreads();
   }
 }
@@ -738,17 +743,13 @@ void sap_half_fine(cudaStream_t st, const typename CT<R>::T* links, R diag, int 
     else
       go(std::integral_constant<int, 16>());
   } else {
-    // lattices with few blocks spread the tiles of a batch over blockIdx.y; those with many keep the inverse in
-    // shared memory across the tiles
-    auto go = [&](auto rg) {
-      constexpr int RG = decltype(rg)::value;
-      const dim3 grid(nb, nb >= 4096 ? 1 : cdiv(nrhs, RG));
-      MG_LAUNCH_W(bytes, flops, k_sap_fine4_fp64<RG>, grid, 64, 0, st, links, L, inv, f, x, color, nrhs, known, active);
-    };
-    if (nrhs <= 8)
-      go(std::integral_constant<int, 8>());
-    else
-      go(std::integral_constant<int, 16>());
+    // lattices with few blocks spread a batch over blockIdx.y, in tiles as small as give every SM eight CTAs (at least
+    // two right-hand sides, one per warp); those with many keep the inverse in shared memory across the tiles
+    const int nsm = sm_count();
+    int tile = SF64_TILE;
+    while (tile > 2 && (long)nb * cdiv(nrhs, tile) < 8L * nsm) tile /= 2;
+    const dim3 grid(nb, nb >= 4096 ? 1 : cdiv(nrhs, tile));
+    MG_LAUNCH_W(bytes, flops, k_sap_fine4_fp64, grid, 64, 0, st, links, L, inv, f, x, color, nrhs, tile, known, active);
   }
 }
 template void sap_half_fine<float>(cudaStream_t, const float2*, float, int, int, const float2*, const float2*,
