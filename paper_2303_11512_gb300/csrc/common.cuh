@@ -104,6 +104,16 @@ inline double act_rhs(int nrhs) { return (g_nact_hint >= 0 && g_nact_hint < nrhs
 #define MG_LAUNCH(kernel, grid, block, smem, stream, ...) \
   MG_LAUNCH_W(0, 0, kernel, grid, block, smem, stream, __VA_ARGS__)
 
+// one complex number from global to shared memory, in flight until its group is waited for
+template <typename C>
+__device__ __forceinline__ void cp_async_elem(C* dst, const C* src) {
+  const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+  if constexpr (sizeof(C) == 16)
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
+  else
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d), "l"(src) : "memory");
+}
+
 // Programmatic dependent launch: a kernel that begins with pdl_begin() may be launched with MG_LAUNCH_P, and the GPU
 // then places its blocks while the last blocks of the kernel before it still run.  pdl_begin() waits until that
 // kernel has completed and its writes are visible, so nothing may be read or written before it (and what an earlier

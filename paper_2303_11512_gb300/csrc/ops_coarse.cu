@@ -252,12 +252,16 @@ void coarse_block_matrices(cudaStream_t stm, const double2* st, int Ls, int d, i
 
 // SAP half sweep.  The blocks of one colour do not couple, so with E the hops that leave the block
 // x_B + D_BB^{-1} (f - D x)_B = D_BB^{-1} (f - E x)_B: the hops inside the block and the old x_B drop out (of the 5
-// stencil blocks of a site in a 2 x 2 block 2 remain).  One CTA per block and tile of G right-hand sides; a thread
-// owns one row of the block (lanes: consecutive rows) and 4 right-hand sides.
+// stencil blocks of a site in a 2 x 2 block 2 remain).  One CTA per block and tile of at most G right-hand sides; a
+// thread owns one row of the block (lanes: consecutive rows) and every ng-th live right-hand side of the tile, up to 4:
+// the remainder of a tile and right-hand sides that have stopped are not computed.
 // FP64 is bound by its units (two FMAs a clock and SM, a share in each quarter): the rows of the inverse and the
 // stencil come straight from global memory (32 lines per load, which costs an eighth of the FMAs they feed) and the
 // CTA stays small, so that lattices with few blocks fill the chip (one 150 KB CTA of 4 rhs per SM before: 0.70 TF).
-// FP32 stages both transposed in shared memory.
+// FP32 stages both transposed in shared memory, by cp.async into rows padded by one.  Level 1 at L = 512 with 1, 8, 9,
+// 64 right-hand sides, a sweep in FP64 1585, 1590, 3038, 12050 us with whole tiles of 8, now 222, 1590, 1733, 12050; in
+// FP32 230, 254, 433, 1760 us with a transposing store that met in one bank, now 72, 117, 166, 789 (tiles of 16: 89,
+// 144, 168, 888).
 constexpr int SC_T = 128, SC_R = 4;
 struct SapCoarseShape {
   int bs, d, bd, ng, G, GP, nslot;
@@ -269,7 +273,7 @@ struct SapCoarseShape {
     nslot = 4 * bs;
   }
   __host__ __device__ int complexes(bool stage) const {
-    return bd * GP + nslot * d * GP + (stage ? bd * bd + nslot * d * d : 0);
+    return bd * GP + nslot * d * GP + (stage ? bd * (bd + 1) + nslot * d * (d + 1) : 0);
   }
 };
 
@@ -282,17 +286,19 @@ __global__ void __launch_bounds__(SC_T) k_sap_coarse(const typename CT<R>::T* __
   typedef typename CT<R>::T C;
   constexpr bool STAGE = sizeof(R) == 4;
   const SapCoarseShape sh(BS ? BS : bs_, DT ? DT : d_);
-  const int bs = sh.bs, d = sh.d, bd = sh.bd, G = sh.G, GP = sh.GP, dd = d * d;
+  const int bs = sh.bs, d = sh.d, bd = sh.bd, ng = sh.ng, GP = sh.GP, dd = d * d;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  C* sres = reinterpret_cast<C*>(smem_raw);      // [row][rhs]
-  C* sx = sres + bd * GP;                        // [slot][k][rhs]: x on the sites around the block
-  C* sinv = sx + sh.nslot * d * GP;              // [column][row] (FP32)
-  C* sst = sinv + bd * bd;                       // [slot][k][row of the site] (FP32)
+  C* sres = reinterpret_cast<C*>(smem_raw);      // [row][group][its rhs]
+  C* sx = sres + bd * GP;                        // [slot][k][group][its rhs]: x on the sites around the block
+  C* sinv = sx + sh.nslot * d * GP;              // [column][row] (FP32), rows of bd + 1
+  C* sst = sinv + bd * (bd + 1);                 // [slot][k][row of the site] (FP32), rows of d + 1
+  __shared__ int srhs[SC_T / 2 * SC_R];          // live right-hand sides of the tile: number k is the (k / ng)-th of
+  __shared__ int scount;                         // group k % ng
   const int tid = threadIdx.x;
   const int nbx = Ls / bs, half = nbx / 2;
   const int BT = blockIdx.x / half;
   const int BX = 2 * (blockIdx.x - BT * half) + ((BT + color) & 1);
-  const int t0 = BT * bs, x0 = BX * bs, r0 = blockIdx.y * G;
+  const int t0 = BT * bs, x0 = BX * bs, r0 = blockIdx.y * sh.G;
   const size_t n = (size_t)Ls * Ls * d;
   const C* I = inv + (size_t)(BT * nbx + BX) * bd * bd;
   // slot: the -x, +x neighbours by row, then the -t, +t neighbours by column; the block's site and direction of each
@@ -302,67 +308,93 @@ __global__ void __launch_bounds__(SC_T) k_sap_coarse(const typename CT<R>::T* __
   };
   auto slot_dir = [&](int s) { const int e = s / bs; return e == 0 ? 2 : e == 1 ? 1 : e == 2 ? 4 : 3; };
   auto site_of = [&](int j) { return (t0 + j / bs) * Ls + x0 + j % bs; };
-  if (!zero) {
-    for (int q = tid; q < sh.nslot * G * d; q += SC_T) {
-      const int k = q % d, g = (q / d) % G, s = q / (d * G), rhs = r0 + g;
-      if (rhs < nrhs && !(active && !active[rhs]))
-        sx[(s * d + k) * GP + g] = x[rhs * n + (size_t)nbr_site(site_of(slot_site(s)), slot_dir(s), Ls) * d + k];
-    }
-  }
   if (STAGE) {
-    for (int e = tid; e < bd * bd; e += SC_T) sinv[(e % bd) * bd + e / bd] = I[e];
+    for (int e = tid; e < bd * bd; e += SC_T) cp_async_elem(sinv + (e % bd) * (bd + 1) + e / bd, I + e);
     if (!zero)
       for (int e = tid; e < sh.nslot * dd; e += SC_T) {
         const int s = e / dd, r = e - s * dd;
-        sst[s * dd + (r % d) * d + r / d] = st[((size_t)site_of(slot_site(s)) * 5 + slot_dir(s)) * dd + r];
+        cp_async_elem(sst + (s * d + r % d) * (d + 1) + r / d,
+                      st + ((size_t)site_of(slot_site(s)) * 5 + slot_dir(s)) * dd + r);
       }
   }
-  const int row = tid % bd, grp = tid / bd, j = row / d, i = row - j * d;
-  const bool mine = grp < sh.ng;
-  const int site = site_of(j);
-  C acc[SC_R];
-  bool on[SC_R];
-#pragma unroll
-  for (int b = 0; b < SC_R; ++b) {
-    const int rhs = r0 + grp * SC_R + b;
-    on[b] = mine && rhs < nrhs && !(active && !active[rhs]);
-    acc[b] = on[b] ? f[rhs * n + (size_t)site * d + i] : czero<C>();
+  if (tid < 32) {
+    int k = 0;
+    for (int b = 0; b < sh.G; b += 32) {
+      const int rhs = r0 + b + tid;
+      const bool on = b + tid < sh.G && rhs < nrhs && !(active && !active[rhs]);
+      const unsigned m = __ballot_sync(0xffffffffu, on);
+      if (on) srhs[k + __popc(m & ((1u << tid) - 1))] = rhs;
+      k += __popc(m);
+    }
+    if (tid == 0) scount = k;
   }
   __syncthreads();
-  if (mine) {
-    if (!zero) {
+  const int cnt = scount;
+  if (!zero) {
+    for (int q = tid; q < sh.nslot * cnt * d; q += SC_T) {
+      const int k = q % d, g = (q / d) % cnt, s = q / (d * cnt);
+      cp_async_elem(sx + (s * d + k) * GP + (g % ng) * SC_R + g / ng,
+                    x + srhs[g] * n + (size_t)nbr_site(site_of(slot_site(s)), slot_dir(s), Ls) * d + k);
+    }
+  }
+  asm volatile("cp.async.commit_group;" ::: "memory");
+  const int row = tid % bd, grp = tid / bd, j = row / d, i = row - j * d;
+  const bool mine = grp < ng;
+  const int site = site_of(j);
+  const int own = mine ? (cnt - grp + ng - 1) / ng : 0;         // right-hand sides of this thread
+  const int most = __reduce_max_sync(0xffffffffu, own);         // and of its warp: blocks below 32 rows share one
+  auto each = [&](auto&& f) {  // with the number of right-hand sides of the warp at compile time
+    if (most == 1) f(std::integral_constant<int, 1>());
+    else if (most == 2) f(std::integral_constant<int, 2>());
+    else if (most == 3) f(std::integral_constant<int, 3>());
+    else if (most == 4) f(std::integral_constant<int, 4>());
+  };
+  C fv[SC_R];
+#pragma unroll
+  for (int b = 0; b < SC_R; ++b)
+    fv[b] = b < own ? f[srhs[grp + b * ng] * n + (size_t)site * d + i] : czero<C>();
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+  __syncthreads();
+  each([&](auto nb) {
+    constexpr int NB = decltype(nb)::value;
+    if (!zero && mine) {
       const int jt = j / bs, jx = j % bs;
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
         if (!(e == 0 ? jx == 0 : e == 1 ? jx == bs - 1 : e == 2 ? jt == 0 : jt == bs - 1)) continue;
         const int s = e * bs + (e < 2 ? jt : jx);
-        const C* w = STAGE ? sst + s * dd + i : st + ((size_t)site * 5 + slot_dir(s)) * dd + (size_t)i * d;
+        const C* w = STAGE ? sst + s * d * (d + 1) + i : st + ((size_t)site * 5 + slot_dir(s)) * dd + (size_t)i * d;
         const C* xv = sx + s * d * GP + grp * SC_R;
 #pragma unroll 8
         for (int k = 0; k < d; ++k) {
-          const C m = cneg(STAGE ? w[k * d] : w[k]);
+          const C m = cneg(STAGE ? w[k * (d + 1)] : w[k]);
 #pragma unroll
-          for (int b = 0; b < SC_R; ++b) acc[b] = cfma(m, xv[k * GP + b], acc[b]);
+          for (int b = 0; b < NB; ++b) fv[b] = cfma(m, xv[k * GP + b], fv[b]);
         }
       }
     }
+    if (mine)
 #pragma unroll
-    for (int b = 0; b < SC_R; ++b) sres[row * GP + grp * SC_R + b] = acc[b];
-  }
+      for (int b = 0; b < NB; ++b) sres[row * GP + grp * SC_R + b] = fv[b];
+  });
   __syncthreads();
   if (!mine) return;
+  each([&](auto nb) {
+    constexpr int NB = decltype(nb)::value;
+    C acc[NB];
 #pragma unroll
-  for (int b = 0; b < SC_R; ++b) acc[b] = czero<C>();
-  const C* rv = sres + grp * SC_R;
+    for (int b = 0; b < NB; ++b) acc[b] = czero<C>();
+    const C* rv = sres + grp * SC_R;
 #pragma unroll 8
-  for (int c = 0; c < bd; ++c) {
-    const C m = STAGE ? sinv[c * bd + row] : __ldg(I + (size_t)row * bd + c);
+    for (int c = 0; c < bd; ++c) {
+      const C m = STAGE ? sinv[c * (bd + 1) + row] : __ldg(I + (size_t)row * bd + c);
 #pragma unroll
-    for (int b = 0; b < SC_R; ++b) acc[b] = cfma(m, rv[c * GP + b], acc[b]);
-  }
+      for (int b = 0; b < NB; ++b) acc[b] = cfma(m, rv[c * GP + b], acc[b]);
+    }
 #pragma unroll
-  for (int b = 0; b < SC_R; ++b)
-    if (on[b]) x[(size_t)(r0 + grp * SC_R + b) * n + (size_t)site * d + i] = acc[b];
+    for (int b = 0; b < NB; ++b)
+      if (b < own) x[srhs[grp + b * ng] * n + (size_t)site * d + i] = acc[b];
+  });
 }
 
 template <typename R>
@@ -388,15 +420,16 @@ void sap_half_coarse(cudaStream_t stm, const typename CT<R>::T* st, int Ls, int 
   const double bytes = nb * (ar * (zero ? 2.0 : 3.0) * sh.bd * cs + ((double)sh.bd * sh.bd + ext) * cs);
   const double flops = nb * ar * 8.0 * (ext + (double)sh.bd * sh.bd);
   const dim3 grid(nb, cdiv(nrhs, sh.G));
-  if (bs == 2 && d == 16) {
-    ensure_max_smem((const void*)k_sap_coarse<R, 2, 16>, 120 * 1024);
-    MG_LAUNCH_W(bytes, flops, (k_sap_coarse<R, 2, 16>), grid, SC_T, sm, stm, st, Ls, d, bs, inv, f, x, color, nrhs,
-                zero, active);
-  } else {
-    ensure_max_smem((const void*)k_sap_coarse<R, 0, 0>, 120 * 1024);
-    MG_LAUNCH_W(bytes, flops, (k_sap_coarse<R, 0, 0>), grid, SC_T, sm, stm, st, Ls, d, bs, inv, f, x, color, nrhs,
-                zero, active);
-  }
+  auto go = [&](auto* kernel) {
+    ensure_max_smem((const void*)kernel, 120 * 1024);
+    MG_LAUNCH_W(bytes, flops, kernel, grid, SC_T, sm, stm, st, Ls, d, bs, inv, f, x, color, nrhs, zero, active);
+  };
+  // 2 x 2 blocks of 2, 4 and 8 test vectors per chirality at compile time: with 4 (L = 512, level 1, 1 and 64 FP32
+  // right-hand sides) the index divisions of the runtime form made a sweep 42 and 350 us instead of 24 and 210
+  if (bs == 2 && d == 16) go(&k_sap_coarse<R, 2, 16>);
+  else if (bs == 2 && d == 8) go(&k_sap_coarse<R, 2, 8>);
+  else if (bs == 2 && d == 4) go(&k_sap_coarse<R, 2, 4>);
+  else go(&k_sap_coarse<R, 0, 0>);
 }
 template void sap_half_coarse<float>(cudaStream_t, const float2*, int, int, int, const float2*, const float2*,
                                      float2*, int, int, const int*, bool);

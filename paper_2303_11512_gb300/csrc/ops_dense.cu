@@ -527,15 +527,6 @@ template void invert_large<float2>(cudaStream_t, float2*, int, int*, void*, int*
 // hence 2 x 2 (32 bytes for 16 FMAs).  FP64: each quarter of an SM has its own share of the two FMAs a clock, so the
 // results are spread over as many warps as there are, one a thread.  n = 1024 with 8, 32, 64 rhs: FP32 32, 33, 43 ->
 // 23, 30, 33 us, FP64 275, 275, 523 -> 151, 270, 537 us (tiles of 16 x 16 results and a barrier every 16 columns before).
-template <typename C>
-__device__ __forceinline__ void cp_async_elem(C* dst, const C* src) {
-  const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
-  if constexpr (sizeof(C) == 16)
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
-  else
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d), "l"(src) : "memory");
-}
-
 template <typename C, int RI, int NR>
 struct DenseTile {
   static constexpr int KC = 32, ST = sizeof(C) == 8 ? 8 : 4, TI = 8 * RI, TR = 8 * NR;

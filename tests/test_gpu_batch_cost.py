@@ -60,9 +60,10 @@ def micros(fn, reps=20, best=5):
     return min(out)
 
 
-# level, lattice side, hierarchy, batch, larger batch, most that their times may differ by: FP64 units bound both, so
-# the times go as the batches do (0.125, 0.56 and 0.53 here)
-SMOOTH = [(0, 256, {}, 1, 8, 0.6), (0, 256, {}, 9, 16, 0.8), (0, 256, {}, 17, 32, 0.8)]
+# level, lattice side, hierarchy, batch, larger batch, largest ratio of their times: FP64 units bound both, so the times
+# go as the batches do (1/8, 9/16 and 17/32)
+SMOOTH = [(0, 256, {}, 1, 8, 0.6), (0, 256, {}, 9, 16, 0.8), (0, 256, {}, 17, 32, 0.8),
+          (1, 256, {}, 1, 8, 0.6), (1, 256, {}, 9, 16, 0.8), (1, 256, dict(ntv=4), 17, 32, 0.8)]
 
 
 @pytest.mark.parametrize("level,L,kw,few,many,ratio", SMOOTH)
@@ -85,3 +86,33 @@ def test_fine_smoother_by_rhs(api, ctx, L, nrhs):
     for k in range(nrhs):
         h.smooth(0, f[k:k + 1], ref[k:k + 1], api.FP64, 2)
     assert torch.equal(x, ref)
+
+
+@pytest.mark.parametrize("ntv,nrhs", [(8, 2), (8, 3), (8, 7), (8, 13), (4, 5), (4, 18), (2, 11), (2, 37), (1, 70)])
+@pytest.mark.parametrize("prec", ["FP32", "FP64"])
+def test_coarse_smoother_by_rhs(api, ctx, ntv, nrhs, prec):
+    """Sweeps on level 1 with 2 x 2 blocks of 8 to 64 unknowns (one to sixteen groups of rows in a CTA): batches that
+    leave its groups uneven give the bits of one right-hand side at a time, also through the V-cycle's zero start."""
+    h = hierarchy(api, ctx, 64, ntv=ntv)
+    pr, dt = getattr(api, prec), torch.complex64 if prec == "FP32" else torch.complex128
+    f, x = (vecs(h.n[1], nrhs, s, dt) for s in (1, 2))
+    ref = x.clone()
+    h.smooth(1, f, x, pr, 2)
+    for k in range(nrhs):
+        h.smooth(1, f[k:k + 1], ref[k:k + 1], pr, 2)
+    assert torch.equal(x, ref)
+
+
+def test_stopped_right_hand_sides(api, ctx):
+    """Solves in which some right-hand sides never start (zero) or stop early beside others, FP64 and mixed: every
+    solution satisfies the residual, whatever slots of a tile are live."""
+    h = hierarchy(api, ctx, 64)
+    b = vecs(h.n[0], 21, 5, torch.complex128)
+    b[[0, 3, 4, 17]] = 0
+    x = torch.empty_like(b)
+    for prec in (api.FP64, api.MIXED):
+        api.fgmres_batched(ctx, h, 0, b, x, tol=1e-10, prec=prec)
+        r = torch.empty_like(b)
+        h.apply(0, x, r, api.FP64)
+        norm = torch.linalg.vector_norm
+        assert (norm(b - r, dim=1) <= 1.1e-10 * norm(b, dim=1)).all() and not x[[0, 3, 4, 17]].any()
