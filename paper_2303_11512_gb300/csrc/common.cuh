@@ -128,6 +128,13 @@ __device__ __forceinline__ void pdl_begin() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 constexpr double PDL_BYTES = 24e6;
+// FP64 kernels that keep their units busy for more than some 14 us are launched plainly: blocks placed beside the last
+// ones of the kernel before come to lie unevenly on the SMs, and the fullest SM decides.
+constexpr double PDL_FLOPS64 = 1.7e7;
+template <typename R>
+inline bool early_launch(double bytes, double flops) {
+  return bytes < PDL_BYTES && (sizeof(R) == 4 || flops < PDL_FLOPS64);
+}
 extern thread_local bool g_capturing;  // launches go into a graph (looked up on entry of every call)
 template <typename... Par, typename... Arg>
 inline void launch_pdl(bool early, void (*kernel)(Par...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
@@ -144,7 +151,7 @@ inline void launch_pdl(bool early, void (*kernel)(Par...), dim3 grid, dim3 block
   cfg.numAttrs = early ? 1 : 0;
   MG_CUDA(cudaLaunchKernelEx(&cfg, kernel, static_cast<Par>(arg)...));
 }
-#define MG_LAUNCH_P(bytes, flops, kernel, grid, block, smem, stream, ...)          \
+#define MG_LAUNCH_PE(early, bytes, flops, kernel, grid, block, smem, stream, ...)  \
   do {                                                                             \
     ::mg::KTimer* t_ = ::mg::g_timer;                                              \
     cudaEvent_t a_ = nullptr, b_ = nullptr;                                        \
@@ -153,13 +160,15 @@ inline void launch_pdl(bool early, void (*kernel)(Par...), dim3 grid, dim3 block
       b_ = t_->get();                                                              \
       MG_CUDA(cudaEventRecord(a_, (stream)));                                      \
     }                                                                              \
-    ::mg::launch_pdl((bytes) < PDL_BYTES && !::mg::g_capturing, kernel, (grid), (block), (smem), (stream), __VA_ARGS__);      \
+    ::mg::launch_pdl((early) && !::mg::g_capturing, kernel, (grid), (block), (smem), (stream), __VA_ARGS__); \
     if (a_) {                                                                      \
       MG_CUDA(cudaEventRecord(b_, (stream)));                                      \
       t_->recs.push_back({#kernel, __PRETTY_FUNCTION__, (double)(bytes), (double)(flops), a_, b_}); \
     }                                                                              \
     if (::mg::g_launch_counter) ++*::mg::g_launch_counter;                         \
   } while (0)
+#define MG_LAUNCH_P(bytes, flops, kernel, grid, block, smem, stream, ...) \
+  MG_LAUNCH_PE((bytes) < ::mg::PDL_BYTES, bytes, flops, kernel, grid, block, smem, stream, __VA_ARGS__)
 
 // ---------------------------------------------------------------- complex
 template <typename R> struct CT;

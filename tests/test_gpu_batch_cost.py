@@ -116,3 +116,27 @@ def test_stopped_right_hand_sides(api, ctx):
         h.apply(0, x, r, api.FP64)
         norm = torch.linalg.vector_norm
         assert (norm(b - r, dim=1) <= 1.1e-10 * norm(b, dim=1)).all() and not x[[0, 3, 4, 17]].any()
+
+
+@pytest.mark.parametrize("few,many,ratio", [(1, 8, 0.6), (9, 16, 0.85)])
+def test_restriction_cost(api, ctx, few, many, ratio):
+    """FP64 restriction of `few` vectors of 16 dof per site against one of `many`."""
+    h = hierarchy(api, ctx, 512)
+    f, c = (vecs(h.n[l], many, l, torch.complex128) for l in (1, 2))
+    t = [micros(lambda: h.restrict(1, f[:k], c[:k], api.FP64)) for k in (few, many)]
+    assert t[0] < ratio * t[1], t
+
+
+@pytest.mark.parametrize("L,nrhs", [(64, 3), (64, 5), (64, 37), (128, 13), (128, 50)])
+@pytest.mark.parametrize("prec", ["FP32", "FP64"])
+def test_restriction_by_rhs(api, ctx, L, nrhs, prec):
+    """Restriction from level 1 in tiles of 4, 8 and 16 right-hand sides with their remainders: the bits of one
+    right-hand side at a time."""
+    h = hierarchy(api, ctx, L)
+    pr, dt = getattr(api, prec), torch.complex64 if prec == "FP32" else torch.complex128
+    f = vecs(h.n[1], nrhs, 1, dt)
+    c, ref = (torch.full((nrhs, h.n[2]), float("nan"), dtype=dt, device="cuda") for _ in range(2))
+    h.restrict(1, f, c, pr)
+    for k in range(nrhs):
+        h.restrict(1, f[k:k + 1], ref[k:k + 1], pr)
+    assert torch.equal(c, ref)
