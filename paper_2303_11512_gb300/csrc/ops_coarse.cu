@@ -606,8 +606,12 @@ __global__ void __launch_bounds__(16 / MM * (RG / RR))
 }
 
 // xf (+)= P xc.  A thread keeps the rows of P of its two consecutive dofs in registers (D = 16: one chirality; D = 2:
-// both spins of a site) and takes the right-hand sides of the tile in turn; xc comes from shared memory.  D = 16 with
-// xf16: the planar 16-bit copy is written alongside.
+// both spins of a site; FP64 with D = 2 of one dof, so that a warp has one right-hand side and an odd one costs no more)
+// and takes right-hand sides of the tile in turn, up to the last one; xc comes from shared memory.
+// D = 2: a row of P serves the 8 threads of its site, so P goes through shared memory too (rows padded: their 16-byte
+// reads fall into different banks); reading it from global memory in every thread was 16 loads for one or two results.
+// L = 512 with 1, 8, 32 right-hand sides: FP32 20, 66, 108 -> 19, 22, 57 us, FP64 60, 226, 882 -> 33, 224, 876.
+// D = 16 with xf16: the planar 16-bit copy is written alongside.
 template <typename R, bool ADD, int D, int RG>
 __global__ void __launch_bounds__(128) k_prolong2(const typename CT<R>::T* __restrict__ P, int Ls,
                                                   const typename CT<R>::T* xc,
@@ -615,44 +619,65 @@ __global__ void __launch_bounds__(128) k_prolong2(const typename CT<R>::T* __res
                                                   int bf, int nrhs, const int* active) {
   pdl_begin();
   typedef typename CT<R>::T C;
-  constexpr int PAIRS = 8 * D, RS = 128 / PAIRS;  // dof pairs of an aggregate, rhs taken at once
-  constexpr int ROWS = 8 * D;                     // rows of a chirality block
+  constexpr int DPT = D == 2 && sizeof(R) == 8 ? 1 : 2;  // dofs per thread
+  constexpr int TPR = 16 * D / DPT, RS = 128 / TPR;      // threads per rhs, rhs taken at once
+  constexpr int ROWS = 8 * D;                            // rows of a chirality block
+  constexpr int PP = 8 + 16 / (int)sizeof(C);            // padded row of P
   __shared__ __align__(16) C sc[RG][16];
+  __shared__ __align__(16) C sp[D == 2 ? 32 * PP : 1];
   const int Lc = Ls / 4, a = blockIdx.x, AT = a / Lc, AX = a - AT * Lc, r0 = blockIdx.y * RG, tid = threadIdx.x;
+  const int cnt = min(RG, nrhs - r0);
   const size_t n = (size_t)Ls * Ls * D, nc = (size_t)Lc * Lc * 16;
-  for (int q = tid; q < RG * 16; q += 128) {
-    const int g = q >> 4, rhs = r0 + g;
-    if (rhs < nrhs && !(active && !active[rhs])) sc[g][q & 15] = xc[rhs * nc + (size_t)a * 16 + (q & 15)];
-  }
-  const int pr = tid % PAIRS, js = pr / (D / 2), k = 2 * (pr % (D / 2)), rs = tid / PAIRS;
-  const int c0 = D == 2 ? 0 : k >> 3, c1 = D == 2 ? 1 : c0;
   const C* Pa = P + (size_t)a * 2 * ROWS * 8;
-  const C* p0 = Pa + (c0 * ROWS + (D == 2 ? js : js * 8 + (k & 7))) * 8;
-  const C* p1 = Pa + (c1 * ROWS + (D == 2 ? js : js * 8 + (k & 7) + 1)) * 8;
-  C w[2][8];
+  if constexpr (D == 2) {
+    constexpr int CPR = 8 * (int)sizeof(C) / 16;  // 16-byte chunks of a row
+    for (int q = tid; q < 32 * CPR; q += 128)
+      cp_async16c(reinterpret_cast<char*>(sp + q / CPR * PP) + q % CPR * 16, reinterpret_cast<const char*>(Pa) + q * 16);
+  }
+  for (int q = tid; q < cnt * 16; q += 128) {
+    const int rhs = r0 + (q >> 4);
+    if (!(active && !active[rhs])) cp_async_elem(&sc[q >> 4][q & 15], xc + rhs * nc + (size_t)a * 16 + (q & 15));
+  }
+  asm volatile("cp.async.commit_group;" ::: "memory");
+  const int dof = DPT * (tid % TPR), js = dof / D, k = dof % D, rs = tid / TPR;  // first dof of the thread
+  const int c0 = D == 2 ? k : k >> 3;                                            // its chirality
+  constexpr int CS = D == 2 ? 1 : 0;                                             // step of the chirality to the next
+  C w[DPT][8];
+  if constexpr (D == 16) {
 #pragma unroll
-  for (int m = 0; m < 8; ++m) {
-    w[0][m] = __ldg(p0 + m);
-    w[1][m] = __ldg(p1 + m);
+    for (int u = 0; u < DPT; ++u)
+#pragma unroll
+      for (int m = 0; m < 8; m += 2) load2(Pa + (c0 * ROWS + js * 8 + (k & 7) + u) * 8 + m, w[u] + m);
   }
   const size_t off = ((size_t)(4 * AT + (js >> 2)) * Ls + 4 * AX + (js & 3)) * D + k;
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
   __syncthreads();
+  if constexpr (D == 2) {
+#pragma unroll
+    for (int u = 0; u < DPT; ++u)
+#pragma unroll
+      for (int m = 0; m < 8; m += 2) load2(sp + ((c0 + u) * 16 + js) * PP + m, w[u] + m);
+  }
 #pragma unroll 4
-  for (int g = rs; g < RG; g += RS) {
+  for (int g = rs; g < cnt; g += RS) {
     const int rhs = r0 + g;
-    if (rhs >= nrhs || (active && !active[rhs])) continue;
+    if (active && !active[rhs]) continue;
     C* px = xf + rhs * n + off;
-    C v[2], acc[2];
-    if (ADD) load2(px, v);
-    acc[0] = acc[1] = czero<C>();
+    C v[DPT], acc[DPT];
+    if constexpr (ADD && DPT == 2) load2(px, v);
+    if constexpr (ADD && DPT == 1) v[0] = px[0];
 #pragma unroll
-    for (int m = 0; m < 8; ++m) {
-      acc[0] = cfma(w[0][m], sc[g][c0 * 8 + m], acc[0]);
-      acc[1] = cfma(w[1][m], sc[g][c1 * 8 + m], acc[1]);
-    }
+    for (int u = 0; u < DPT; ++u) acc[u] = czero<C>();
 #pragma unroll
-    for (int u = 0; u < 2; ++u) v[u] = ADD ? cadd(v[u], acc[u]) : acc[u];
-    store2(px, v);
+    for (int m = 0; m < 8; ++m)
+#pragma unroll
+      for (int u = 0; u < DPT; ++u) acc[u] = cfma(w[u][m], sc[g][(c0 + u * CS) * 8 + m], acc[u]);
+#pragma unroll
+    for (int u = 0; u < DPT; ++u) v[u] = ADD ? cadd(v[u], acc[u]) : acc[u];
+    if constexpr (DPT == 2)
+      store2(px, v);
+    else
+      px[0] = v[0];
     if constexpr (sizeof(R) == 4 && D == 16) {
       if (xf16) {  // Re parts of the site's 16 dofs, then the Im parts
         unsigned* p16 = reinterpret_cast<unsigned*>(xf16 + 2 * (rhs * n + off - k) + k);
@@ -667,6 +692,11 @@ __global__ void __launch_bounds__(128) k_prolong2(const typename CT<R>::T* __res
       }
     }
   }
+}
+
+// right-hand sides on the fullest SM where every aggregate has a CTA per tile of rg of them
+static long fullest_sm(int aggs, int nrhs, int rg, int nsm) {
+  return (long)cdiv((long)aggs * (nrhs / rg), nsm) * rg + (long)cdiv(aggs, nsm) * (nrhs % rg);
 }
 
 template <typename R>
@@ -703,8 +733,8 @@ void restrict_op(cudaStream_t stm, const typename CT<R>::T* P, int Ls, int d, in
     // FP64 with few aggregates: the tile whose fullest SM has the fewer right-hand sides (64 aggregates with 32, 48, 64:
     // 37, 52, 72 us in tiles of 4, 8, 4; 51, 52, 72 before)
     const int aggs = Lc * Lc, nsm = sm_count();
-    auto fullest = [&](int rg) { return cdiv((long)aggs * (nrhs / rg), nsm) * rg + cdiv(aggs, nsm) * (nrhs % rg); };
-    const bool small = nrhs <= 4 || (sizeof(R) == 8 && aggs * cdiv(nrhs, 8) < 4 * nsm && fullest(4) < fullest(8));
+    const bool small = nrhs <= 4 || (sizeof(R) == 8 && aggs * cdiv(nrhs, 8) < 4 * nsm &&
+                                     fullest_sm(aggs, nrhs, 4, nsm) < fullest_sm(aggs, nrhs, 8, nsm));
     typedef std::integral_constant<int, 1> I1;
     if (small)
       go(std::integral_constant<int, 4>(), I1());
@@ -736,18 +766,22 @@ static void prolong_launch(cudaStream_t stm, const typename CT<R>::T* P, int Ls,
   const int Lc = Ls / agg;
   auto go = [&](auto dd, auto rg) {
     constexpr int D = decltype(dd)::value, RG = decltype(rg)::value;
-    MG_LAUNCH_P(bytes, flops, (k_prolong2<R, ADD, D, RG>), dim3(Lc * Lc, cdiv(nrhs, RG)), 128, 0, stm, P, Ls, xc, xf,
-                xf16, bf, nrhs, active);
+    MG_LAUNCH_PE(early_launch<R>(bytes, flops), bytes, flops, (k_prolong2<R, ADD, D, RG>),
+                 dim3(Lc * Lc, cdiv(nrhs, RG)), 128, 0, stm, P, Ls, xc, xf, xf16, bf, nrhs, active);
   };
   typedef std::integral_constant<int, 8> I8;
   typedef std::integral_constant<int, 32> I32;
   const bool aligned = ((uintptr_t)xf & 15) == 0;  // 16-byte accesses; other vectors take the general kernel
+  const int aggs = Lc * Lc, nsm = sm_count();
+  // tiles of 8 or 32: FP64 the one whose fullest SM has the fewer right-hand sides (8 while that leaves SMs without a
+  // tile); FP32 8 for few aggregates, which spreads a batch over more CTAs
+  const bool tile8 = nrhs <= 8 || (sizeof(R) == 4 ? d == 16 && aggs * cdiv(nrhs, 32) < 4 * nsm
+                                                  : aggs * cdiv(nrhs, 8) <= nsm ||
+                                                        fullest_sm(aggs, nrhs, 8, nsm) < fullest_sm(aggs, nrhs, 32, nsm));
   if (agg == 4 && ntv == 8 && d == 2 && aligned) {
-    nrhs <= 8 ? go(std::integral_constant<int, 2>(), I8()) : go(std::integral_constant<int, 2>(), I32());
+    tile8 ? go(std::integral_constant<int, 2>(), I8()) : go(std::integral_constant<int, 2>(), I32());
   } else if (agg == 4 && ntv == 8 && d == 16 && aligned) {
-    // few aggregates: tiles of 8 rhs spread a batch over more CTAs
-    nrhs <= 8 || Lc * Lc * cdiv(nrhs, 32) < 152 * 4 ? go(std::integral_constant<int, 16>(), I8())
-                                                   : go(std::integral_constant<int, 16>(), I32());
+    tile8 ? go(std::integral_constant<int, 16>(), I8()) : go(std::integral_constant<int, 16>(), I32());
   } else {
     const int na = agg * agg, bsz = na * d / 2, dc = 2 * ntv, G = std::max(1, 256 / (na * d));
     const size_t sm = sizeof(C) * ((size_t)2 * bsz * ntv + (size_t)G * dc);

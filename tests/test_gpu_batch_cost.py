@@ -140,3 +140,30 @@ def test_restriction_by_rhs(api, ctx, L, nrhs, prec):
     for k in range(nrhs):
         h.restrict(1, f[k:k + 1], ref[k:k + 1], pr)
     assert torch.equal(c, ref)
+
+
+@pytest.mark.parametrize("level,L,prec,few,many,ratio", [(0, 512, "FP32", 8, 32, 0.5), (1, 256, "FP64", 9, 16, 0.85)])
+def test_prolongation_cost(api, ctx, level, L, prec, few, many, ratio):
+    """Prolongation of `few` vectors against one of `many`: on the fine level bound by memory (8 right-hand sides move a
+    third of the bytes of 32), from 16 dof per site by the FP64 units."""
+    h = hierarchy(api, ctx, L)
+    pr, dt = getattr(api, prec), torch.complex64 if prec == "FP32" else torch.complex128
+    f, c = (vecs(h.n[l], many, l, dt) for l in (level, level + 1))
+    t = [micros(lambda: h.prolong(level, c[:k], f[:k], pr)) for k in (few, many)]
+    assert t[0] < ratio * t[1], t
+
+
+@pytest.mark.parametrize("L,nrhs", [(64, 2), (64, 7), (64, 9), (64, 35), (128, 13), (128, 41)])
+@pytest.mark.parametrize("prec", ["FP32", "FP64"])
+def test_prolongation_by_rhs(api, ctx, L, nrhs, prec):
+    """Prolongation to levels 0 and 1 in tiles of 8 and 32 right-hand sides with their remainders: the bits of one
+    right-hand side at a time."""
+    h = hierarchy(api, ctx, L)
+    pr, dt = getattr(api, prec), torch.complex64 if prec == "FP32" else torch.complex128
+    for l in range(2):
+        c = vecs(h.n[l + 1], nrhs, 1, dt)
+        f, ref = (torch.full((nrhs, h.n[l]), float("nan"), dtype=dt, device="cuda") for _ in range(2))
+        h.prolong(l, c, f, pr)
+        for k in range(nrhs):
+            h.prolong(l, c[k:k + 1], ref[k:k + 1], pr)
+        assert torch.equal(f, ref)
