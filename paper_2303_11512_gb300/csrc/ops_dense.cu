@@ -525,11 +525,13 @@ template void invert_large<float2>(cudaStream_t, float2*, int, int*, void*, int*
 // the results only: blocks of 64 threads with RI rows x NR right-hand sides each, tiles of A and x staged ST chunks of
 // 32 columns deep by cp.async (L2 answers in about 1 us).  In FP32 the bytes that shared memory returns come next,
 // hence 2 x 2 (32 bytes for 16 FMAs).  FP64: each quarter of an SM has its own share of the two FMAs a clock, so the
-// results are spread over as many warps as there are, one a thread.  n = 1024 with 8, 32, 64 rhs: FP32 32, 33, 43 ->
-// 23, 30, 33 us, FP64 275, 275, 523 -> 151, 270, 537 us (tiles of 16 x 16 results and a barrier every 16 columns before).
+// results are spread over as many warps as there are, one a thread; warps without a right-hand side multiply nothing,
+// and three stages let eight CTAs into an SM, so that 64 right-hand sides need no second wave.  n = 1024 with 8, 17, 32,
+// 64 rhs: FP32 31, 31, 31, 41 -> 20, 26, 26, 40 us, FP64 273, 273, 275, 521 -> 146, 206, 269, 488 us (tiles of 16 x 16
+// results and a barrier every 16 columns before).
 template <typename C, int RI, int NR>
 struct DenseTile {
-  static constexpr int KC = 32, ST = sizeof(C) == 8 ? 8 : 4, TI = 8 * RI, TR = 8 * NR;
+  static constexpr int KC = 32, ST = sizeof(C) == 8 ? 8 : 3, TI = 8 * RI, TR = 8 * NR;
   static constexpr int AP = TI + 16 / (int)sizeof(C), XP = TR + 16 / (int)sizeof(C);  // padded, rows 16-byte aligned
   C As[ST][KC][AP];  // [column][row]
   C Xs[ST][KC][XP];  // [column][rhs]
@@ -580,6 +582,7 @@ __global__ void __launch_bounds__(64) k_dense_apply(const C* __restrict__ A, int
 #pragma unroll
         for (int b = 0; b < NR; ++b) acc[a][b] = cfma(m[a], v[b], acc[a][b]);
     };
+    if (sizeof(C) == 16 && r0 + tr * NR >= nrhs) continue;  // no right-hand side: FP64 units are the bound
     if (cols == KC) {
 #pragma unroll 8
       for (int j = 0; j < KC; ++j) column(j);
@@ -615,8 +618,10 @@ void dense_apply(cudaStream_t st, const typename CT<R>::T* A, int n, const typen
     constexpr int RI = decltype(ri)::value, NR = decltype(nr)::value;
     constexpr int sm = (int)sizeof(DenseTile<C, RI, NR>);
     ensure_max_smem((const void*)k_dense_apply<C, RI, NR>, sm);
-    MG_LAUNCH_P(bytes, flops, (k_dense_apply<C, RI, NR>), dim3(cdiv(n, 8 * RI), cdiv(nrhs, 8 * NR)), 64, sm, st, A, n,
-                x, y, nrhs, active);
+    const dim3 grid(cdiv(n, 8 * RI), cdiv(nrhs, 8 * NR));
+    // FP64, three CTAs per SM and more: an early launch would place them unevenly (32 rhs: 390 us)
+    const bool early = bytes < PDL_BYTES && (sizeof(R) == 4 || (long)grid.x * grid.y < 3L * sm_count());
+    MG_LAUNCH_PE(early, bytes, flops, (k_dense_apply<C, RI, NR>), grid, 64, sm, st, A, n, x, y, nrhs, active);
   };
   typedef std::integral_constant<int, 1> I1;
   typedef std::integral_constant<int, 2> I2;

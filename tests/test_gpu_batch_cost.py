@@ -167,3 +167,27 @@ def test_prolongation_by_rhs(api, ctx, L, nrhs, prec):
         for k in range(nrhs):
             h.prolong(l, c[k:k + 1], ref[k:k + 1], pr)
         assert torch.equal(f, ref)
+
+
+def test_coarsest_apply_cost(api, ctx):
+    """FP64 inverse of a coarsest level of 1024 unknowns, applied one call behind the other: 32 right-hand sides load
+    the SMs evenly (twice the 16 that give every SM at most two tiles), and 64 need no second wave."""
+    h = hierarchy(api, ctx, 128)
+    top = h.levels - 1
+    b, x = (vecs(h.n[top], 64, s, torch.complex128) for s in (1, 2))
+    t = [micros(lambda: h.vcycle(top, b[:k], x[:k], api.FP64)) for k in (16, 32, 64)]
+    assert h.n[top] == 1024 and t[1] < 2.2 * t[0] and t[2] < 1.9 * t[1], t
+
+
+@pytest.mark.parametrize("nrhs", [3, 11, 20, 33])
+@pytest.mark.parametrize("prec", ["FP32", "FP64"])
+def test_coarsest_apply_by_rhs(api, ctx, nrhs, prec):
+    """Warps of a tile without a right-hand side skip their products: the bits of one right-hand side at a time."""
+    h = hierarchy(api, ctx, 64)
+    top, pr, dt = h.levels - 1, getattr(api, prec), torch.complex64 if prec == "FP32" else torch.complex128
+    b = vecs(h.n[top], nrhs, 1, dt)
+    x, ref = (torch.full_like(b, float("nan")) for _ in range(2))
+    h.vcycle(top, b, x, pr)
+    for k in range(nrhs):
+        h.vcycle(top, b[k:k + 1], ref[k:k + 1], pr)
+    assert torch.equal(x, ref)
