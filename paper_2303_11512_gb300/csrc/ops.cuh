@@ -15,6 +15,8 @@ void prepare_links(cudaStream_t st, const double2* U, int L, double2* l64, float
 // *bad = 1 if some link of U is NaN or infinite (bad is not cleared)
 void check_links(cudaStream_t st, const double2* U, int L, int* bad);
 // y = D x, or y = b - D x when b != nullptr.
+// form of the FP32 operator for a batch and the tuned rhs per thread: 0 per site, else rhs per thread, walking along t
+int wilson_variant(int L, int nrhs, int rpt);
 template <typename R>
 void wilson_apply(cudaStream_t st, const typename CT<R>::T* links, R diag, int L,
                   const typename CT<R>::T* x, typename CT<R>::T* y, const typename CT<R>::T* b,

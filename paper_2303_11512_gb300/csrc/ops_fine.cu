@@ -155,16 +155,18 @@ __global__ void __launch_bounds__(256) k_wilson(LK lk, R diag, int L, const type
 // FP32, long batches: a thread walks WT time slices of its column, for RPT right-hand sides (blockIdx.y * RPT + j),
 // with the spinors of the last, this and the next slice in registers, so that a spinor comes from L2 (1 + 2 / WT)
 // times instead of three times and a link 1 / RPT times; its x neighbours are L1 hits of the same row.  One thread
-// per site and rhs moved 80 bytes of L2 traffic per site and rhs for 32 of DRAM (5.0 TB/s at L = 512, 256 rhs).
+// per site and rhs moved 80 bytes of L2 traffic per site and rhs for 32 of DRAM (5.0 TB/s at L = 512, 256 rhs).  The
+// columns of all slice groups are numbered through, so that lattices whose side is no multiple of a block leave no lanes
+// idle.
 constexpr int WT = 8;
 template <bool RES, int RPT>
-__global__ void __launch_bounds__(128) k_wilson_walk(const float2* __restrict__ lk, float diag, int L, int xblocks,
+__global__ void __launch_bounds__(128) k_wilson_walk(const float2* __restrict__ lk, float diag, int L,
                                                      const float2* __restrict__ x, float2* __restrict__ y,
                                                      const float2* __restrict__ b, const int* __restrict__ active,
                                                      int nrhs) {
-  const int V = L * L, tb = blockIdx.x / xblocks, xx = (blockIdx.x - tb * xblocks) * 128 + threadIdx.x;
+  const int V = L * L, i = blockIdx.x * 128 + threadIdx.x, tb = i / L, xx = i - tb * L;
   const int t0 = tb * WT, t1 = min(t0 + WT, L);
-  if (xx >= L) return;
+  if (t0 >= L) return;
   const float4* X[RPT];
   bool on[RPT];
   float4 prev[RPT], cur[RPT];
@@ -242,6 +244,18 @@ static void wilson_sites(cudaStream_t st, LK lk, R diag, int L, const typename C
     MG_LAUNCH_W(bytes, flops, (k_wilson<R, false, LK>), grid, bt, 0, st, lk, diag, L, x, y, b, active);
 }
 
+// FP32: 0 one thread per site, else right-hand sides per thread of the walking form, the tuned number or 1 where that
+// would leave the chip short of threads.  The line, with one rhs per thread, per site against walking: L = 512 with 4,
+// 12, 49, 244 rhs 17.5, 30.8, 86.2, 378 against 15.6, 31.4, 84.2, 357 us; L = 136 with 52, 173, 3460 rhs 12.5, 26.7, 371
+// against 12.3, 24.7, 366; below 64 columns a warp lies across slice groups and the per-site form wins (L = 16, 24, 48
+// with 12.8 M sites x rhs: 73.9, 81.4, 78.0 against 88.0, 94.6, 82.6).  At L = 512 with 256 rhs the walk takes 375 us (86 %
+// of the copy bandwidth) with one rhs per thread, 392 with two, 477 with four, 413 with 16 slices and one rhs.
+int wilson_variant(int L, int nrhs, int rpt) {
+  const double threads = (double)L * L * nrhs / WT, least = 1024.0 * sm_count();
+  if (L < 64 || threads < least) return 0;
+  return threads / rpt >= least ? rpt : 1;
+}
+
 template <typename R>
 void wilson_apply(cudaStream_t st, const typename CT<R>::T* links, R diag, int L, const typename CT<R>::T* x,
                   typename CT<R>::T* y, const typename CT<R>::T* b, int nrhs, const int* active) {
@@ -259,20 +273,15 @@ void wilson_apply(cudaStream_t st, const typename CT<R>::T* links, R diag, int L
   const double bytes = ar * V * sp * (b ? 3 : 2) + V * sp;
   const double flops = ar * V * (b ? 56.0 : 52.0);
   if constexpr (sizeof(R) == 4) {
-    // the walking form needs L * L / WT threads per rhs to fill the chip; at L = 512 with 256 rhs it takes 375 us (86 %
-    // of the copy bandwidth) with one rhs per thread, 392 with two, 477 with four, 413 with 16 slices and one rhs, and
-    // one thread per site 418 us
-    const int rpt = tune_lookup(TUNE_WILSON32, L, nrhs, 0, 1);
-    if (V * nrhs / (WT * rpt) >= 152.0 * 1024) {
-      const int xb = cdiv(L, 128);
-      const dim3 grid(xb * cdiv(L, WT), cdiv(nrhs, rpt));
+    if (const int rpt = wilson_variant(L, nrhs, tune_lookup(TUNE_WILSON32, L, nrhs, 0, 1))) {
+      const dim3 grid(cdiv((long)L * cdiv(L, WT), 128), cdiv(nrhs, rpt));
 #define MG_WILSON_LAUNCH(RPT_)                                                                                        \
   do {                                                                                                                \
     if (b)                                                                                                            \
-      MG_LAUNCH_W(bytes, flops, (k_wilson_walk<true, RPT_>), grid, 128, 0, st, links, diag, L, xb, x, y, b, active,   \
+      MG_LAUNCH_W(bytes, flops, (k_wilson_walk<true, RPT_>), grid, 128, 0, st, links, diag, L, x, y, b, active,       \
                   nrhs);                                                                                              \
     else                                                                                                              \
-      MG_LAUNCH_W(bytes, flops, (k_wilson_walk<false, RPT_>), grid, 128, 0, st, links, diag, L, xb, x, y, b, active,  \
+      MG_LAUNCH_W(bytes, flops, (k_wilson_walk<false, RPT_>), grid, 128, 0, st, links, diag, L, x, y, b, active,      \
                   nrhs);                                                                                              \
   } while (0)
       if (rpt == 4)

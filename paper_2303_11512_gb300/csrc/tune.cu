@@ -106,6 +106,7 @@ void autotune(mgmlmc_hier* h, const std::vector<int>& nrhs_list, bool force) {
         int best = 1;
         float tbest = 1e30f;
         for (int v : {1, 2, 4}) {
+          if (v > 1 && wilson_variant(L0.side, bucket, v) != v) continue;  // runs as variant 1 does
           tune_store(TUNE_WILSON32, L0.side, bucket, 0, v, 0.f);
           const float t = time_us(st, [&] {
             wilson_apply<float>(st, L0.links32.as<float2>(), (float)L0.diag, L0.side, x.as<float2>(), y.as<float2>(),

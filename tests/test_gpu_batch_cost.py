@@ -191,3 +191,45 @@ def test_coarsest_apply_by_rhs(api, ctx, nrhs, prec):
     for k in range(nrhs):
         h.vcycle(top, b[k:k + 1], ref[k:k + 1], pr)
     assert torch.equal(x, ref)
+
+
+@pytest.mark.parametrize("L,nrhs", [(24, 22222), (72, 12346), (136, 3460)])
+def test_stencil_lanes(api, ctx, L, nrhs):
+    """FP32 operator on sides that are no multiple of its blocks: memory bounds it, so a batch takes the time that as
+    many sites take at L = 512, up to a tenth (with idle lanes 1.16 to 1.23 times as long)."""
+    t = []
+    for side, k in ((L, nrhs), (512, max(1, round(nrhs * L * L / 512 ** 2)))):
+        U = torch.from_numpy(np.exp(1j * np.random.default_rng(0).uniform(-3, 3, (side, side, 2)))).cuda()
+        x = vecs(2 * side * side, k, 1, torch.complex64)
+        y = torch.empty_like(x)
+        t.append(micros(lambda: api.schwinger_apply(ctx, U, side, 0.1, x, y, api.FP32)) / (k * side * side))
+    assert t[0] < 1.1 * t[1], t
+
+
+@pytest.mark.parametrize("L,nrhs,rpt", [(142, 63, 1), (136, 76, 1), (130, 161, 2), (200, 65, 2), (130, 323, 4),
+                                        (256, 101, 4), (142, 63, 4), (48, 700, 2)])
+def test_stencil_walk_forms(api, ctx, L, nrhs, rpt):
+    """The walking form with 1, 2 and 4 right-hand sides per thread set in the table, sides that are no multiple of its
+    128 columns or 8 slices, batches that leave a thread short, a setting that would leave the chip short of threads
+    (taken as 1) and a side below its smallest: against the FP64 form of the same call (nine terms, a few roundings of
+    6e-8 each), and which kernel ran."""
+    U = torch.from_numpy(np.exp(1j * np.random.default_rng(L).uniform(-3, 3, (L, L, 2)))).cuda()
+    x = vecs(2 * L * L, nrhs, 3, torch.complex64)
+    y = torch.full_like(x, float("nan"))
+    x64 = x.to(torch.complex128)
+    ref = torch.empty_like(x64)
+    api.schwinger_apply(ctx, U, L, 0.1, x64, ref, api.FP64)
+    bucket = 8
+    while bucket < min(nrhs, 256):
+        bucket *= 2
+    try:
+        api.tune_set([dict(kind=0, side=L, bucket=bucket, format=0, variant=rpt)])
+        ctx.timing(True, "k_wilson")
+        api.schwinger_apply(ctx, U, L, 0.1, x, y, api.FP32)
+        ran = " ".join(ctx.timing_report())
+    finally:
+        ctx.timing(False)
+        api.tune_clear()
+    eff = 0 if L < 64 else rpt if L * L * nrhs / 8 / rpt >= 1024 * torch.cuda.get_device_properties(0).multi_processor_count else 1
+    assert ("k_wilson_walk" in ran) == (eff > 0), (ran, eff)
+    assert (y - ref).abs().max() < 2e-6 * ref.abs().max()
