@@ -44,7 +44,7 @@ __device__ __forceinline__ int nbr_site(int s, int dir, int Ls) {
 }
 
 // ---- coarse stencil apply -----------------------------------------------------
-// FP64, other block sizes than 16, and FP32 vectors off a 16-byte boundary.
+// FP64, other block sizes than 16, FP32 vectors off a 16-byte boundary and small batches on few sites.
 // CTA per site: the 5 stencil blocks (transposed in shared memory) are applied to the
 // rhs in groups of 256 / d; DT = d at compile time (0: runtime d).
 template <typename R, bool RES, int DT>
@@ -189,7 +189,11 @@ void coarse_apply(cudaStream_t stm, const typename CT<R>::T* st, int Ls, int d, 
   const double bytes = ar * ns * d * cs * (b ? 3 : 2) + ns * 5.0 * d * d * cs;
   const double flops = ar * ns * 8.0 * 5.0 * d * d;
   if constexpr (sizeof(R) == 4) {
-    if (d == 16 && ((uintptr_t)x & 15) == 0) {  // 16-byte copies; other vectors take the general kernel
+    // 16-byte copies: other vectors take the general kernel, as do lattices of less than a site per SM up to 16
+    // right-hand sides, where its 256 threads per site are the shorter chain (8 x 8 sites with 1, 16: 4.9, 6.2 us
+    // against 6.2, 8.2; 16 x 16 sites 5.9, 8.2 against 6.2, 8.2)
+    const bool few = Ls * Ls < sm_count() && nrhs <= 16;
+    if (d == 16 && ((uintptr_t)x & 15) == 0 && !few) {
       auto go = [&](auto rg, auto ri) {
         constexpr int RG = decltype(rg)::value, RI = decltype(ri)::value, smb = (80 + 5 * RG) * 18 * 8;
         ensure_max_smem((const void*)k_coarse_apply16<false, RG, RI>, smb);

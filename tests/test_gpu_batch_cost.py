@@ -233,3 +233,21 @@ def test_stencil_walk_forms(api, ctx, L, nrhs, rpt):
     eff = 0 if L < 64 else rpt if L * L * nrhs / 8 / rpt >= 1024 * torch.cuda.get_device_properties(0).multi_processor_count else 1
     assert ("k_wilson_walk" in ran) == (eff > 0), (ran, eff)
     assert (y - ref).abs().max() < 2e-6 * ref.abs().max()
+
+
+@pytest.mark.parametrize("level,nrhs,tiled", [(2, 1, False), (2, 16, False), (2, 17, True), (1, 1, True), (1, 16, True)])
+def test_coarse_operator_forms(api, ctx, level, nrhs, tiled):
+    """FP32 operator with 16 dof per site: 8 x 8 sites with up to 16 right-hand sides take the kernel of 256 threads per
+    site, 16 x 16 sites and larger batches the tiled one (80 products, a few roundings of 6e-8 each)."""
+    h = hierarchy(api, ctx, 128 if level == 2 else 64)
+    x = vecs(h.n[level], nrhs, 1, torch.complex64)
+    y, ref = torch.empty_like(x), torch.empty_like(x, dtype=torch.complex128)
+    h.apply(level, x.to(torch.complex128), ref, api.FP64)
+    try:
+        ctx.timing(True, "k_coarse_apply")
+        h.apply(level, x, y, api.FP32)
+        ran = " ".join(ctx.timing_report())
+    finally:
+        ctx.timing(False)
+    assert ("k_coarse_apply16" in ran) == tiled, ran
+    assert (y - ref).abs().max() < 2e-5 * ref.abs().max()
