@@ -245,8 +245,8 @@ int mg_tc_status(mgmlmc_ctx* ctx, mgmlmc_hier* h);
  * direct solve of Section 3.1: tau_L of Algorithm 2 is the trace of D_L^{-1}):
  * Gauss-Jordan elimination with partial pivoting (largest |A_ik|, ties to the
  * smallest row), by block columns: a cluster eliminates 8 columns, the grid
- * applies them.  A: device, row-major, complex128 (prec MGMLMC_FP64) or complex64
- * (MGMLMC_FP32), 1 <= n <= 8192.
+ * applies them (n <= 32: one CTA in shared memory).  A: device, row-major,
+ * complex128 (prec MGMLMC_FP64) or complex64 (MGMLMC_FP32), 1 <= n <= 8192.
  * barrier_polls: 0 = as above (no software barrier).  Otherwise one cooperative
  * kernel whose CTAs meet at a grid barrier per column, with the same pivots:
  * positive = poll limit of every barrier wait (a wait that expires returns

@@ -80,7 +80,7 @@ void invert_small_batched(cudaStream_t st, C* A, int nmat, int bd, int* fail);
 // in-place inverse of one n x n matrix (large n); work: invert_large_work_bytes(n); fail set on a zero pivot;
 // C = double2 / float2
 size_t invert_large_work_bytes(int n);
-// polls: 0 = by block columns (n > 32); otherwise one cooperative kernel with a grid barrier per column, > 0: poll
+// polls: 0 = by block columns (n <= 32: in one CTA); otherwise one cooperative kernel with a grid barrier per column, > 0: poll
 // limit of each wait (timeout set when one expires), < 0: bounded-wait self-test (the barrier expects one arrival more
 // than the grid has, so every wait runs out after -polls polls)
 template <typename C>

@@ -138,7 +138,6 @@ template void invert_small_batched<float2>(cudaStream_t, float2*, int, int, int*
 // barrier per column.  The barrier spins on a generation counter with an iteration limit (timeout flag, all
 // CTAs then leave).  Columns are unscrambled afterwards by the recorded swaps in reverse order.
 constexpr int GJ_T = 512;
-constexpr long GJ_SPIN = 1L << 28;  // default polls of the generation counter (well over a second)
 
 // `expect` arrivals release the barrier (the grid size; one more in the bounded-wait self-test, where nothing
 // releases it and every wait runs out after `polls` polls)
@@ -482,8 +481,10 @@ static void invert_blocked(cudaStream_t st, C* A, int n, int* piv, void* work, i
 
 template <typename C>
 void invert_large(cudaStream_t st, C* A, int n, int* piv, void* work, int* fail, int* timeout, long polls) {
-  // below 33 rows the launches of the block columns take longer than the barriers (0.2 against 0.13 ms at n = 8)
+  // up to 32 rows one CTA in shared memory, with the same pivots (the launches of the block columns would take longer:
+  // 0.2 ms at n = 8); the cooperative kernel only where a poll limit of its barrier is asked for
   if (polls == 0 && n > 32) return invert_blocked<C>(st, A, n, piv, work, fail, timeout);
+  if (polls == 0) return invert_small_batched<C>(st, A, 1, n, fail);
   int dev = 0, nsm = 0, per = 0;
   MG_CUDA(cudaGetDevice(&dev));
   MG_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
@@ -499,8 +500,7 @@ void invert_large(cudaStream_t st, C* A, int n, int* piv, void* work, int* fail,
   int* slot_i = (int*)(slot_v + 2048);
   unsigned* bar = (unsigned*)(slot_i + 2048);
   MG_CUDA(cudaMemsetAsync(bar, 0, 2 * sizeof(unsigned), st));
-  // polls == 0: the default limit; polls < 0: bounded-wait self-test (one arrival more than the grid has)
-  long lim = polls == 0 ? GJ_SPIN : polls > 0 ? polls : -polls;
+  long lim = polls > 0 ? polls : -polls;  // < 0: bounded-wait self-test (one arrival more than the grid has)
   unsigned expect = (unsigned)grid + (polls < 0 ? 1u : 0u);
   void* args[] = {&A, &A1, &n, &piv, &slot_v, &slot_i, &bar, &fail, &timeout, &lim, &expect};
   KTimer* t = g_timer;

@@ -283,3 +283,27 @@ def test_batches_beyond_the_grid(api, ctx):
     h.smooth(0, fine, x, api.FP32, 1)
     h.smooth(0, fref, xref, api.FP32, 1)
     assert relerr(x[-k:].cpu().numpy(), xref.cpu().numpy()) < 2e-6
+
+
+@pytest.mark.parametrize("n", [1, 2, 7, 31, 32, 33])
+@pytest.mark.parametrize("prec,eps", [("FP64", 1.1e-16), ("FP32", 6e-8)])
+def test_dense_inverse_without_barrier(api, ctx, n, prec, eps):
+    """Without a poll limit no size runs the kernel that spins on a grid barrier (n <= 32: one CTA, 33 on: block
+    columns); the inverse of a matrix whose rows have to be swapped, against the identity as above, and a singular one."""
+    rs = np.random.default_rng(n)
+    A = (rs.standard_normal((n, n)) + 1j * rs.standard_normal((n, n))).astype(
+        np.complex128 if prec == "FP64" else np.complex64)
+    if n > 1:
+        A[0, 0] = 0
+    B = torch.from_numpy(A).cuda()
+    try:
+        ctx.timing(True)
+        api.mg_dense_inverse(ctx, B, getattr(api, prec))
+        ran = " ".join(ctx.timing_report())
+    finally:
+        ctx.timing(False)
+    assert "k_gj_coop" not in ran and ("k_gj_panel" in ran) == (n > 32), ran
+    A = A.astype(complex)
+    assert np.abs(B.cpu().numpy() @ A - np.eye(n)).max() < 4 * n * eps * np.linalg.cond(A)
+    with pytest.raises(Exception):
+        api.mg_dense_inverse(ctx, torch.zeros((n, n), dtype=B.dtype, device="cuda"), getattr(api, prec))
