@@ -384,6 +384,7 @@ void fgmres_core(mgmlmc_hier* h, int l, const typename CT<R>::T* b, typename CT<
         // every right-hand side that has stopped
         MG_CUDA(cudaEventSynchronize(ctx->flag_event[j & 1]));
         if (ctx->pinned[j - 2] == 0) break;
+        g_nact_hint = ctx->pinned[j - 2];
       }
       op_apply<R>(h, l, Zj, Vj1, nullptr, nrhs, s.iact);
       kry_step<C>(st, s.V, vs, j + 1, Vj1, n, s.gm, s.red);

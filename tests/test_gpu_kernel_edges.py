@@ -307,3 +307,39 @@ def test_dense_inverse_without_barrier(api, ctx, n, prec, eps):
     assert np.abs(B.cpu().numpy() @ A - np.eye(n)).max() < 4 * n * eps * np.linalg.cond(A)
     with pytest.raises(Exception):
         api.mg_dense_inverse(ctx, torch.zeros((n, n), dtype=B.dtype, device="cuda"), getattr(api, prec))
+
+
+def free_field(L, periodic=False):
+    U = np.ones((L, L, 2), dtype=complex)
+    if periodic:
+        U[L - 1, :, 1] = -1  # undoes the antiperiodic sign
+    return U
+
+
+def test_reported_bytes_follow_the_stopped(api, ctx):
+    """Unpreconditioned solve of seven plane waves of the free field, each done in two steps, beside a random vector of
+    many: the report bills the operator for the right-hand sides that go on, at most two steps late."""
+    L, nrhs = 32, 8
+    U = free_field(L)
+    h = api.mg_setup(ctx, torch.from_numpy(U).cuda(), L, 0.2, ntv=1, setup_sweeps=1, tensor_cores=0, levels=2)
+    try:
+        t, x = np.meshgrid(np.arange(L), np.arange(L), indexing="ij")
+        b = vecs(2 * L * L, nrhs, 1, np.complex128)
+        for k in range(nrhs - 1):
+            wave = np.exp(2j * np.pi * ((k + 0.5) * t + 3 * k * x) / L)
+            b[k] = (wave[..., None] * np.array([0.3, 0.7 + 0.2j])).reshape(-1)
+        bd = torch.from_numpy(b).cuda()
+        xd = torch.empty_like(bd)
+        ctx.timing(True, "k_wilson")
+        st = api.fgmres_batched(ctx, h, 0, bd, xd, precond=0, m=64, tol=1e-10, prec=api.FP64, maxit=60,
+                                raise_on_nonconvergence=False)
+        rep = ctx.timing_report()
+        ctx.timing(False)
+        steps = int(st["its"].max())
+        assert steps >= 20 and sorted(st["its"])[-2] <= 3, st["its"]
+        full = 32.0 * L * L * (2 * nrhs + 1)  # bytes of one application to the whole batch
+        used = sum(r["bytes"] for r in rep.values()) / full
+        assert used < 4 + 0.25 * steps, (used, steps)
+    finally:
+        ctx.timing(False)
+        h.close()
