@@ -2,7 +2,10 @@
 // w = D z_j against the basis V_0 .. V_j, the norm, the Givens update of the Hessenberg column and the next basis
 // vector, per right-hand side:
 //   h1 = V^H w,  w' = w - V h1,  h2 = V^H w',  hn^2 = |w'|^2 - |h2|^2,  v_{j+1} = (w' - V h2) / hn.
-// (hn is |w' - V h2| by Pythagoras; h2 is of the order of the rounding of h1, so nothing cancels.)
+// hn is |w' - V h2| by Pythagoras: h2 is of the order of the rounding of h1, so nothing cancels while w' is much larger
+// than that.  When w lies in the span of the basis up to rounding, w' is rounding itself and may lie in the span too: from
+// |h2|^2 > |w'|^2 / 4 on the Krylov space counts as spent, the right-hand side's cycle ends with this column and the true
+// residual decides (the difference could be 0 or of either sign, and v_{j+1} would be rounding of any length).
 //
 // Two forms.  Long vectors: three passes over V, each one launch; the block that finishes last for a right-hand
 // side adds the partial sums in a fixed order (bitwise repeatable) and, after the second pass, does the Givens
@@ -67,10 +70,11 @@ __device__ __forceinline__ void givens_load(const KryGm& g, int j, int r, Givens
     v.s[i] = g.sn[(size_t)i * g.nrhs + r];
   }
 }
+__device__ __forceinline__ bool kry_spent(double w2, double h22) { return 4 * h22 > w2; }
 // Givens update of column j for right-hand side r by one thread; v.col: h1 + h2 (j + 1 entries, overwritten); hn2 =
-// |w' - V h2|^2 (negative by rounding counts as 0).  FP64 latency is what it costs: reciprocal square roots in place
+// |w' - V h2|^2 (negative by rounding counts as 0); spent: see above, the right-hand side's cycle ends here.  FP64 latency is what it costs: reciprocal square roots in place
 // of square roots and divisions, and the stop test on squares.
-__device__ void givens_column(const KryGm& g, int j, int r, Givens& v, double hn2) {
+__device__ void givens_column(const KryGm& g, int j, int r, Givens& v, double hn2, bool spent) {
   const int nrhs = g.nrhs, m = g.m;
   double2* col = v.col;
   double2 a = col[0];
@@ -107,7 +111,7 @@ __device__ void givens_column(const KryGm& g, int j, int r, Givens& v, double hn
   g.its[r] = it;
   g.kvec[r] = j + 1;
   g.hn[r] = hh;
-  if (res2 <= goal * goal || it >= g.maxit || hh == 0.0 || j + 1 == m || !(res2 == res2))
+  if (res2 <= goal * goal || it >= g.maxit || hh == 0.0 || spent || j + 1 == m || !(res2 == res2))
     g.iact[r] = 0;
   else
     atomicAdd(g.count + j, 1);
@@ -297,9 +301,13 @@ __global__ void __launch_bounds__(KT, sizeof(C) == 16 && KM > 8 ? 2 : 1)
   }
   __syncthreads();
   if (threadIdx.x == 0) {
-    double hn2 = tot[k].x;
-    for (int i = 0; i < k; ++i) hn2 -= tot[i].x * tot[i].x + tot[i].y * tot[i].y;
-    givens_column(gm, k - 1, rhs, gv, hn2);
+    double hn2 = tot[k].x, h22 = 0;
+    for (int i = 0; i < k; ++i) {
+      const double q = tot[i].x * tot[i].x + tot[i].y * tot[i].y;
+      hn2 -= q;
+      h22 += q;
+    }
+    givens_column(gm, k - 1, rhs, gv, hn2, kry_spent(tot[k].x, h22));
   }
 }
 
@@ -363,8 +371,7 @@ __global__ void __launch_bounds__(32) k_kry_givens(KryGm gm, int k) {
   h2n = warp_sum1(h2n);
   __syncwarp();
   if (l == 0) {
-    const double hn2 = gm.wn2[r] - h2n;
-    givens_column(gm, k - 1, r, gv, hn2);
+    givens_column(gm, k - 1, r, gv, gm.wn2[r] - h2n, kry_spent(gm.wn2[r], h2n));
   }
 }
 
@@ -527,11 +534,12 @@ __global__ void __launch_bounds__(T) k_kry_small(const C* __restrict__ V, long v
   cluster_totals(2 * k + 1, hp2, reinterpret_cast<double*>(h2));
   double h2n = 0;
   for (int i = l; i < k; i += 32) h2n += h2[i].x * h2[i].x + h2[i].y * h2[i].y;
-  const double hn2 = h2[k].x - warp_sum1(h2n);
+  h2n = warp_sum1(h2n);
+  const double hn2 = h2[k].x - h2n;
   if (rank == 0 && wi == 0) {
     for (int i = l; i < k; i += 32) gv.col[i] = cadd(h1[i], h2[i]);
     __syncwarp();
-    if (l == 0) givens_column(gm, k - 1, rhs, gv, hn2);
+    if (l == 0) givens_column(gm, k - 1, rhs, gv, hn2, kry_spent(h2[k].x, h2n));
   }
   if (hn2 > 0) {
     update(h2);

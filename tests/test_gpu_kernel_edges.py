@@ -343,3 +343,32 @@ def test_reported_bytes_follow_the_stopped(api, ctx):
     finally:
         ctx.timing(False)
         h.close()
+
+
+@pytest.mark.parametrize("L", [16, 32, 64, 128])
+@pytest.mark.parametrize("prec", ["FP32", "FP64"])
+def test_spent_krylov_space(api, ctx, L, prec):
+    """An eigenvector (the constant spinor of the periodic free field) spends its Krylov space in one step, up to a
+    residue of rounding that lies in the span: the cycle ends there, in the one-launch form (up to 16384 entries) and in
+    the three-pass form, and the true residual decides.  Plane waves of two spin components spend it in two."""
+    dt, eps = (np.complex64, 6e-8) if prec == "FP32" else (np.complex128, 1.1e-16)
+    t, x = np.meshgrid(np.arange(L), np.arange(L), indexing="ij")
+    for m0 in (0.2, 0.37, 0.61):
+        for periodic in (True, False):
+            U = free_field(L, periodic)
+            h = api.mg_setup(ctx, torch.from_numpy(U).cuda(), L, m0, ntv=1, setup_sweeps=1, tensor_cores=0,
+                             levels=2 if L <= 64 else 0)
+            try:
+                D = osch.dirac_sparse(U, m0)
+                wave = np.ones((L, L)) if periodic else np.exp(2j * np.pi * (2.5 * t + 3 * x) / L)
+                b = (wave[..., None] * np.array([1, 1] if periodic else [0.3, 0.7 + 0.2j])).reshape(1, -1).astype(dt)
+                bd = torch.from_numpy(b).cuda()
+                xd = torch.empty_like(bd)
+                st = api.fgmres_batched(ctx, h, 0, bd, xd, precond=0, m=30, tol=1e-300, maxit=12, prec=getattr(api, prec),
+                                        raise_on_nonconvergence=False)
+                res = np.linalg.norm(b[0] - D @ xd.cpu().numpy()[0].astype(complex)) / np.linalg.norm(b)
+                assert res < 100 * eps, res
+                if periodic:
+                    assert st["its"][0] == st["outer"], st
+            finally:
+                h.close()
