@@ -251,3 +251,15 @@ def test_coarse_operator_forms(api, ctx, level, nrhs, tiled):
         ctx.timing(False)
     assert ("k_coarse_apply16" in ran) == tiled, ran
     assert (y - ref).abs().max() < 2e-5 * ref.abs().max()
+
+
+def test_projection_chunks(api, ctx):
+    """A projected sample's sums run over the same chunks of its rows whatever the batch: its bits do not depend on the
+    other samples (one chunk of all rows for long batches would change them)."""
+    h = hierarchy(api, ctx, 64)
+    sk, _ = api.hutchpp_sketch_qr(ctx, h, 0, 8, 1, 3, api.ACCUMULATED, tol=1e-6, prec=api.MIXED)
+    z, y = (vecs(h.n[0], 3000, s, torch.complex128) for s in (1, 2))
+    tau = api.hutchpp_project(ctx, sk, z, y)
+    for k in (0, 1500, 2999):
+        assert api.hutchpp_project(ctx, sk, z[k:k + 1], y[k:k + 1])[0] == tau[k]
+    sk.close()
