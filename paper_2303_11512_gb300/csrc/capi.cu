@@ -15,11 +15,6 @@ int guarded(mgmlmc_ctx* ctx, F&& f) {
   LaunchScope scope(ctx);
   try {
     MG_CUDA(cudaSetDevice(ctx->device));
-    // a caller's stream capture turns launches into graph nodes (an error: the legacy stream beside another capture)
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    const bool known = cudaStreamIsCapturing(ctx->stream, &cap) == cudaSuccess;
-    g_capturing = !known || cap != cudaStreamCaptureStatusNone;
-    if (!known) cudaGetLastError();
     f();
     ctx->err.clear();
     return MGMLMC_OK;
@@ -151,7 +146,7 @@ int schwinger_apply(mgmlmc_ctx* ctx, const double* U, int L, double m0, const vo
         wilson_apply_raw<double>(st, (const double2*)U, diag, L, (const double2*)x, (double2*)y, nrhs);
       return;
     }
-    const bool own = g_capturing;
+    const bool own = in_capture(st);
     std::unique_lock<std::mutex> lock(ctx->links_mutex, std::defer_lock);
     DBuf own64, own32;
     if (!own) lock.lock();

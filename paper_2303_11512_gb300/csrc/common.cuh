@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
 #include <cstdio>
 #include <cstring>
 #include <mutex>
@@ -135,7 +136,18 @@ template <typename R>
 inline bool early_launch(double bytes, double flops) {
   return bytes < PDL_BYTES && (sizeof(R) == 4 || flops < PDL_FLOPS64);
 }
-extern thread_local bool g_capturing;  // launches go into a graph (looked up on entry of every call)
+// Launches of this call go into a graph: 1 yes, 0 no, -1 not looked up yet.  Looked up where it matters and at most once
+// a call (200 ns), because the smallest calls take 5 us.
+extern thread_local int g_capturing;
+inline bool in_capture(cudaStream_t stream) {
+  if (g_capturing < 0) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    const bool known = cudaStreamIsCapturing(stream, &cap) == cudaSuccess;
+    if (!known) cudaGetLastError();  // the legacy stream beside another capture
+    g_capturing = !known || cap != cudaStreamCaptureStatusNone;
+  }
+  return g_capturing != 0;
+}
 template <typename... Par, typename... Arg>
 inline void launch_pdl(bool early, void (*kernel)(Par...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
                        Arg&&... arg) {
@@ -160,7 +172,7 @@ inline void launch_pdl(bool early, void (*kernel)(Par...), dim3 grid, dim3 block
       b_ = t_->get();                                                              \
       MG_CUDA(cudaEventRecord(a_, (stream)));                                      \
     }                                                                              \
-    ::mg::launch_pdl((early) && !::mg::g_capturing, kernel, (grid), (block), (smem), (stream), __VA_ARGS__); \
+    ::mg::launch_pdl((early) && !::mg::in_capture(stream), kernel, (grid), (block), (smem), (stream), __VA_ARGS__); \
     if (a_) {                                                                      \
       MG_CUDA(cudaEventRecord(b_, (stream)));                                      \
       t_->recs.push_back({#kernel, __PRETTY_FUNCTION__, (double)(bytes), (double)(flops), a_, b_}); \
@@ -261,10 +273,15 @@ struct DBuf {
 };
 
 inline unsigned cdiv(long a, long b) { return (unsigned)((a + b - 1) / b); }
-inline int sm_count() {  // of the current device
-  int dev = 0, n = 0;
+inline int sm_count() {  // of the current device (the attribute is looked up once per device: calls are microseconds)
+  static std::atomic<int> known[64];
+  int dev = 0;
   MG_CUDA(cudaGetDevice(&dev));
-  MG_CUDA(cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev));
+  int n = dev < 64 ? known[dev].load(std::memory_order_relaxed) : 0;
+  if (!n) {
+    MG_CUDA(cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev));
+    if (dev < 64) known[dev].store(n, std::memory_order_relaxed);
+  }
   return n;
 }
 

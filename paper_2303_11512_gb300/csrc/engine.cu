@@ -14,7 +14,7 @@ namespace mg {
 thread_local int64_t* g_launch_counter = nullptr;
 thread_local KTimer* g_timer = nullptr;
 thread_local int g_nact_hint = -1;
-thread_local bool g_capturing = false;
+thread_local int g_capturing = -1;
 
 // ---------------------------------------------------------------- helpers
 template <typename R> static inline const typename CT<R>::T* links_of(const LevelData& L) {
@@ -233,8 +233,9 @@ static void vcycle_maybe_graph(mgmlmc_hier* h, int l, const typename CT<R>::T* i
     if (!h->capture_stream) MG_CUDA(cudaStreamCreateWithFlags(&h->capture_stream, cudaStreamNonBlocking));
     cudaStream_t cs = h->capture_stream;
     MG_CUDA(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
-    const bool outer = g_capturing;
-    h->capturing = g_capturing = true;
+    const int outer = g_capturing;
+    h->capturing = true;
+    g_capturing = 1;
     h->ctx->stream = cs;  // the V-cycle's launches go to the capturing stream
     try {
       vcycle<R>(h, l, gin, gout, nrhs, active);

@@ -126,12 +126,13 @@ struct LaunchScope {
     g_launch_counter = &c->launches;
     g_timer = c->timer.on ? &c->timer : nullptr;
     g_nact_hint = -1;
+    g_capturing = -1;
   }
   ~LaunchScope() {
     g_launch_counter = nullptr;
     g_timer = nullptr;
     g_nact_hint = -1;
-    g_capturing = false;
+    g_capturing = -1;
   }
 };
 
