@@ -525,24 +525,23 @@ template void invert_large<float2>(cudaStream_t, float2*, int, int*, void*, int*
 // the results only: blocks of 64 threads with RI rows x NR right-hand sides each, tiles of A and x staged ST chunks of
 // 32 columns deep by cp.async (L2 answers in about 1 us).  In FP32 the bytes that shared memory returns come next,
 // hence 2 x 2 (32 bytes for 16 FMAs).  FP64: each quarter of an SM has its own share of the two FMAs a clock, so the
-// results are spread over as many warps as there are, one a thread; warps without a right-hand side multiply nothing,
-// and three stages let eight CTAs into an SM, so that 64 right-hand sides need no second wave.  n = 1024 with 8, 17, 32,
-// 64 rhs: FP32 31, 31, 31, 41 -> 20, 26, 26, 40 us, FP64 273, 273, 275, 521 -> 146, 206, 269, 488 us (tiles of 16 x 16
-// results and a barrier every 16 columns before).
-template <typename C, int RI, int NR>
+// results are spread over as many warps as there are, one a thread, and warps without a right-hand side multiply nothing.
+// n = 1024 with 8, 17, 32, 64 rhs: FP32 31, 31, 31, 41 -> 20, 26, 26, 40 us, FP64 273, 273, 275, 521 -> 146, 183, 270, 488
+// us (tiles of 16 x 16 results and a barrier every 16 columns before).
+template <typename C, int RI, int NR, int ST>
 struct DenseTile {
-  static constexpr int KC = 32, ST = sizeof(C) == 8 ? 8 : 3, TI = 8 * RI, TR = 8 * NR;
+  static constexpr int KC = 32, TI = 8 * RI, TR = 8 * NR;
   static constexpr int AP = TI + 16 / (int)sizeof(C), XP = TR + 16 / (int)sizeof(C);  // padded, rows 16-byte aligned
   C As[ST][KC][AP];  // [column][row]
   C Xs[ST][KC][XP];  // [column][rhs]
 };
 
-template <typename C, int RI, int NR>
+template <typename C, int RI, int NR, int ST>
 __global__ void __launch_bounds__(64) k_dense_apply(const C* __restrict__ A, int n, const C* x,
                                                     C* __restrict__ y, int nrhs, const int* active) {
   pdl_begin();
-  typedef DenseTile<C, RI, NR> DT;
-  constexpr int KC = DT::KC, ST = DT::ST, TI = DT::TI, TR = DT::TR;
+  typedef DenseTile<C, RI, NR, ST> DT;
+  constexpr int KC = DT::KC, TI = DT::TI, TR = DT::TR;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   DT& t = *reinterpret_cast<DT*>(smem_raw);
   const int tid = threadIdx.x, i0 = blockIdx.x * TI, r0 = blockIdx.y * TR;
@@ -614,23 +613,30 @@ void dense_apply(cudaStream_t st, const typename CT<R>::T* A, int n, const typen
     return;
   }
   const double bytes = ((double)n * n + 2.0 * act_rhs(nrhs) * n) * sizeof(C), flops = 8.0 * n * (double)n * act_rhs(nrhs);
-  auto go = [&](auto ri, auto nr) {
-    constexpr int RI = decltype(ri)::value, NR = decltype(nr)::value;
-    constexpr int sm = (int)sizeof(DenseTile<C, RI, NR>);
-    ensure_max_smem((const void*)k_dense_apply<C, RI, NR>, sm);
+  auto go = [&](auto ri, auto nr, auto stages) {
+    constexpr int RI = decltype(ri)::value, NR = decltype(nr)::value, ST = decltype(stages)::value;
+    constexpr int sm = (int)sizeof(DenseTile<C, RI, NR, ST>);
+    ensure_max_smem((const void*)k_dense_apply<C, RI, NR, ST>, sm);
     const dim3 grid(cdiv(n, 8 * RI), cdiv(nrhs, 8 * NR));
-    // FP64, three CTAs per SM and more: an early launch would place them unevenly (32 rhs: 390 us)
-    const bool early = bytes < PDL_BYTES && (sizeof(R) == 4 || (long)grid.x * grid.y < 3L * sm_count());
-    MG_LAUNCH_PE(early, bytes, flops, (k_dense_apply<C, RI, NR>), grid, 64, sm, st, A, n, x, y, nrhs, active);
+    // FP64: more CTAs than SMs are launched plainly, because beside the last blocks of the kernel before they come to lie
+    // unevenly (V-cycle on level 1 at L = 128, n = 1024, with 16 right-hand sides 1164 us, 778 so)
+    const bool early = bytes < PDL_BYTES && (sizeof(R) == 4 || grid.x * grid.y <= (unsigned)sm_count());
+    MG_LAUNCH_PE(early, bytes, flops, (k_dense_apply<C, RI, NR, ST>), grid, 64, sm, st, A, n, x, y, nrhs, active);
   };
   typedef std::integral_constant<int, 1> I1;
   typedef std::integral_constant<int, 2> I2;
-  if constexpr (sizeof(R) == 8)
-    go(I1(), I1());
-  else if (nrhs <= 8)
-    go(I2(), I1());
-  else
-    go(I2(), I2());
+  if constexpr (sizeof(R) == 8) {
+    // six CTAs in an SM with four stages, eight with three: those where they spare a second wave (n = 1024 with 64
+    // right-hand sides 533, 488 us)
+    const long ctas = (long)cdiv(n, 8) * cdiv(nrhs, 8), nsm = sm_count();
+    if (ctas > 6 * nsm && ctas <= 7 * nsm)
+      go(I1(), I1(), std::integral_constant<int, 3>());
+    else
+      go(I1(), I1(), std::integral_constant<int, 4>());
+  } else {
+    typedef std::integral_constant<int, 8> I8;
+    nrhs <= 8 ? go(I2(), I1(), I8()) : go(I2(), I2(), I8());
+  }
 }
 template void dense_apply<float>(cudaStream_t, const float2*, int, const float2*, float2*, int, const int*);
 template void dense_apply<double>(cudaStream_t, const double2*, int, const double2*, double2*, int, const int*);
