@@ -296,8 +296,8 @@ __global__ void __launch_bounds__(SC_T) k_sap_coarse(const typename CT<R>::T* __
   C* sx = sres + bd * GP;                        // [slot][k][group][its rhs]: x on the sites around the block
   C* sinv = sx + sh.nslot * d * GP;              // [column][row] (FP32), rows of bd + 1
   C* sst = sinv + bd * (bd + 1);                 // [slot][k][row of the site] (FP32), rows of d + 1
-  __shared__ int srhs[SC_T / 2 * SC_R];          // live right-hand sides of the tile: number k is the (k / ng)-th of
-  __shared__ int scount;                         // group k % ng
+  __shared__ unsigned char srhs[SC_T / 2 * SC_R];  // live right-hand sides of the tile (r0 + this): number k is the
+  __shared__ int scount;                           // (k / ng)-th of group k % ng.  Bytes: 8 FP64 CTAs fit an SM
   const int tid = threadIdx.x;
   const int nbx = Ls / bs, half = nbx / 2;
   const int BT = blockIdx.x / half;
@@ -327,7 +327,7 @@ __global__ void __launch_bounds__(SC_T) k_sap_coarse(const typename CT<R>::T* __
       const int rhs = r0 + b + tid;
       const bool on = b + tid < sh.G && rhs < nrhs && !(active && !active[rhs]);
       const unsigned m = __ballot_sync(0xffffffffu, on);
-      if (on) srhs[k + __popc(m & ((1u << tid) - 1))] = rhs;
+      if (on) srhs[k + __popc(m & ((1u << tid) - 1))] = (unsigned char)(b + tid);
       k += __popc(m);
     }
     if (tid == 0) scount = k;
@@ -338,7 +338,7 @@ __global__ void __launch_bounds__(SC_T) k_sap_coarse(const typename CT<R>::T* __
     for (int q = tid; q < sh.nslot * cnt * d; q += SC_T) {
       const int k = q % d, g = (q / d) % cnt, s = q / (d * cnt);
       cp_async_elem(sx + (s * d + k) * GP + (g % ng) * SC_R + g / ng,
-                    x + srhs[g] * n + (size_t)nbr_site(site_of(slot_site(s)), slot_dir(s), Ls) * d + k);
+                    x + (r0 + srhs[g]) * n + (size_t)nbr_site(site_of(slot_site(s)), slot_dir(s), Ls) * d + k);
     }
   }
   asm volatile("cp.async.commit_group;" ::: "memory");
@@ -356,7 +356,7 @@ __global__ void __launch_bounds__(SC_T) k_sap_coarse(const typename CT<R>::T* __
   C fv[SC_R];
 #pragma unroll
   for (int b = 0; b < SC_R; ++b)
-    fv[b] = b < own ? f[srhs[grp + b * ng] * n + (size_t)site * d + i] : czero<C>();
+    fv[b] = b < own ? f[(r0 + srhs[grp + b * ng]) * n + (size_t)site * d + i] : czero<C>();
   asm volatile("cp.async.wait_group 0;" ::: "memory");
   __syncthreads();
   each([&](auto nb) {
@@ -397,7 +397,7 @@ __global__ void __launch_bounds__(SC_T) k_sap_coarse(const typename CT<R>::T* __
     }
 #pragma unroll
     for (int b = 0; b < NB; ++b)
-      if (b < own) x[srhs[grp + b * ng] * n + (size_t)site * d + i] = acc[b];
+      if (b < own) x[(r0 + srhs[grp + b * ng]) * n + (size_t)site * d + i] = acc[b];
   });
 }
 
@@ -424,16 +424,20 @@ void sap_half_coarse(cudaStream_t stm, const typename CT<R>::T* st, int Ls, int 
   const double bytes = nb * (ar * (zero ? 2.0 : 3.0) * sh.bd * cs + ((double)sh.bd * sh.bd + ext) * cs);
   const double flops = nb * ar * 8.0 * (ext + (double)sh.bd * sh.bd);
   const dim3 grid(nb, cdiv(nrhs, sh.G));
-  auto go = [&](auto* kernel) {
-    ensure_max_smem((const void*)kernel, 120 * 1024);
-    MG_LAUNCH_W(bytes, flops, kernel, grid, SC_T, sm, stm, st, Ls, d, bs, inv, f, x, color, nrhs, zero, active);
+  auto go = [&](auto bsc, auto dc) {
+    constexpr int BS = decltype(bsc)::value, DT = decltype(dc)::value;
+    ensure_max_smem((const void*)k_sap_coarse<R, BS, DT>, 120 * 1024);
+    MG_LAUNCH_W(bytes, flops, (k_sap_coarse<R, BS, DT>), grid, SC_T, sm, stm, st, Ls, d, bs, inv, f, x, color, nrhs, zero,
+                active);
   };
+  typedef std::integral_constant<int, 2> I2;
+  typedef std::integral_constant<int, 0> I0;
   // 2 x 2 blocks of 2, 4 and 8 test vectors per chirality at compile time: with 4 (L = 512, level 1, 1 and 64 FP32
   // right-hand sides) the index divisions of the runtime form made a sweep 42 and 350 us instead of 24 and 210
-  if (bs == 2 && d == 16) go(&k_sap_coarse<R, 2, 16>);
-  else if (bs == 2 && d == 8) go(&k_sap_coarse<R, 2, 8>);
-  else if (bs == 2 && d == 4) go(&k_sap_coarse<R, 2, 4>);
-  else go(&k_sap_coarse<R, 0, 0>);
+  if (bs == 2 && d == 16) go(I2(), std::integral_constant<int, 16>());
+  else if (bs == 2 && d == 8) go(I2(), std::integral_constant<int, 8>());
+  else if (bs == 2 && d == 4) go(I2(), std::integral_constant<int, 4>());
+  else go(I0(), I0());
 }
 template void sap_half_coarse<float>(cudaStream_t, const float2*, int, int, int, const float2*, const float2*,
                                      float2*, int, int, const int*, bool);

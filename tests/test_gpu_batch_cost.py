@@ -263,3 +263,19 @@ def test_projection_chunks(api, ctx):
     for k in (0, 1500, 2999):
         assert api.hutchpp_project(ctx, sk, z[k:k + 1], y[k:k + 1])[0] == tau[k]
     sk.close()
+
+
+def test_kernel_names_in_the_report(api, ctx):
+    """Every launch of FP32 and FP64 cycles, sweeps and solves is reported under its kernel's name."""
+    h = hierarchy(api, ctx, 128)
+    try:
+        ctx.timing(True)
+        for pr, dt in ((api.FP32, torch.complex64), (api.FP64, torch.complex128)):
+            b, x = (vecs(h.n[0], 3, s, dt) for s in (1, 2))
+            h.vcycle(0, b, x, pr)
+            api.fgmres_batched(ctx, h, 0, b, x, precond=0, m=4, tol=1e-30, maxit=4, prec=pr,
+                               raise_on_nonconvergence=False)
+        names = list(ctx.timing_report())
+    finally:
+        ctx.timing(False)
+    assert any("k_sap_coarse" in n for n in names) and all(n.lstrip("(").startswith("k_") for n in names), names
