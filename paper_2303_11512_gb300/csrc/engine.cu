@@ -285,14 +285,15 @@ struct GmState {
 };
 
 template <typename R>
-static GmState<R> gm_state(mgmlmc_hier* h, int l, int nrhs, int m) {
+static GmState<R> gm_state(mgmlmc_hier* h, int l, int nrhs, int m, bool precond) {
   typedef typename CT<R>::T C;
   GmState<R> s;
   const long n = h->lv[l].n;
   const char* tg = sizeof(R) == 8 ? "gm64" : "gm32";
   char* b = (char*)h->work(std::string(tg) + "_V", l, sizeof(C) * n * nrhs * (m + 1));
   s.V = (C*)b;
-  s.Z = (C*)h->work(std::string(tg) + "_Z", l, sizeof(C) * n * nrhs * m);
+  // without a preconditioner z_j = v_j
+  s.Z = precond ? (C*)h->work(std::string(tg) + "_Z", l, sizeof(C) * n * nrhs * m) : s.V;
   size_t ints = (size_t)nrhs * 6 + m + 1;  // count: one per step, then one for the start of a cycle
   int* ip = (int*)h->work(std::string(tg) + "_i", l, sizeof(int) * ints);
   s.act = ip; s.cact = ip + nrhs; s.iact = ip + 2 * nrhs; s.kvec = ip + 3 * nrhs; s.its = ip + 4 * nrhs;
@@ -330,10 +331,9 @@ void fgmres_core(mgmlmc_hier* h, int l, const typename CT<R>::T* b, typename CT<
   cudaStream_t st = ctx->stream;
   const long n = h->lv[l].n;
   MG_CHECK_ARG(m >= 1 && m <= 64, "FGMRES restart length must be 1..64");
-  GmState<R> s = gm_state<R>(h, l, nrhs, m);
+  GmState<R> s = gm_state<R>(h, l, nrhs, m, precond != 0);
   s.gm.tol = tol;
   s.gm.maxit = maxit;
-  const C* Z = precond ? s.Z : s.V;  // without a preconditioner z_j = v_j
   int* const started = s.count + m;
   const long vs = n * nrhs;
   const unsigned nb = cdiv(nrhs, 64);
@@ -358,7 +358,7 @@ void fgmres_core(mgmlmc_hier* h, int l, const typename CT<R>::T* b, typename CT<
     for (int j = 0; j < m; ++j) {
       C* Vj = s.V + (size_t)j * vs;
       C* Vj1 = s.V + (size_t)(j + 1) * vs;
-      C* Zj = const_cast<C*>(Z) + (size_t)j * vs;
+      C* Zj = s.Z + (size_t)j * vs;
       if (precond) {
         vcycle_maybe_graph<R>(h, l, Vj, Zj, nrhs, s.iact);
         if constexpr (sizeof(R) == 4) {
@@ -401,7 +401,7 @@ void fgmres_core(mgmlmc_hier* h, int l, const typename CT<R>::T* b, typename CT<
     }
     g_nact_hint = nstart;
     kry_trisolve(st, s.gm, s.cact, s.y);
-    vcombine<C>(st, Z, vs, jdone, s.y, x, n, nrhs, s.cact);
+    vcombine<C>(st, s.Z, vs, jdone, s.y, x, n, nrhs, s.cact);
     g_nact_hint = -1;
   }
   g_nact_hint = -1;

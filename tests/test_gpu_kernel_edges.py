@@ -372,3 +372,24 @@ def test_spent_krylov_space(api, ctx, L, prec):
                     assert st["its"][0] == st["outer"], st
             finally:
                 h.close()
+
+
+def test_unpreconditioned_memory(api):
+    """A solve without preconditioner holds one basis of m + 1 batches: 33 of 34 MB here, and 32 more with a second."""
+    L, nrhs, m = 128, 64, 32
+    c = api.Context()
+    h = api.mg_setup(c, torch.from_numpy(free_field(L)).cuda(), L, 0.5, ntv=1, setup_sweeps=1, tensor_cores=0)
+    try:
+        b = torch.from_numpy(vecs(2 * L * L, nrhs, 1, np.complex128)).cuda()
+        x = torch.empty_like(b)
+        api.fgmres_batched(c, h, 0, b, x, precond=0, m=1, tol=0.9, prec=api.FP64)
+        torch.cuda.synchronize()
+        before = torch.cuda.mem_get_info()[0]
+        api.fgmres_batched(c, h, 0, b, x, precond=0, m=m, tol=1e-3, prec=api.FP64)
+        torch.cuda.synchronize()
+        used = before - torch.cuda.mem_get_info()[0]
+        batch = 16 * 2 * L * L * nrhs
+        assert used < 1.3 * (m + 1) * batch, used / batch
+    finally:
+        h.close()
+        c.close()
