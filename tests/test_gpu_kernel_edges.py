@@ -393,3 +393,24 @@ def test_unpreconditioned_memory(api):
     finally:
         h.close()
         c.close()
+
+
+@pytest.mark.parametrize("L,level,ntv,prec,tol", [(16, 0, 8, "FP32", 2e-5), (16, 0, 8, "FP64", 1e-12),
+                                                  (64, 1, 8, "FP32", 2e-5), (64, 1, 4, "FP64", 1e-12)])
+def test_cycles_beyond_one_slice(api, ctx, L, level, ntv, prec, tol):
+    """V-cycles and sweeps of more right-hand sides than the tiled kernels take in one slice (256 K): smoothers of both
+    levels, fused residual and restriction, operator, transfers and coarsest apply in both precisions; the last
+    right-hand sides equal a batch of their own (the same sums, in FP32 up to roundings in another tile shape)."""
+    h, H = hierarchy(api, ctx, L, ntv=ntv)
+    pr, dt = getattr(api, prec), torch.complex64 if prec == "FP32" else torch.complex128
+    nrhs, k = (1 << 18) + 5, 7
+    f = torch.zeros((nrhs, H.n[level]), dtype=dt, device="cuda")
+    f[-k:] = torch.from_numpy(vecs(H.n[level], k, 1, np.complex128)).cuda().to(dt)
+    x = torch.zeros_like(f)
+    ref = torch.zeros_like(f[-k:])
+    for call in (lambda b, y: h.smooth(level, b, y, pr, 1), lambda b, y: h.vcycle(level, b, y, pr)):
+        call(f, x)
+        call(f[-k:].clone(), ref)
+        assert relerr(x[-k:].cpu().numpy(), ref.cpu().numpy()) < tol and not x[:-k].any()
+    del f, x
+    torch.cuda.empty_cache()
