@@ -105,14 +105,19 @@ inline double act_rhs(int nrhs) { return (g_nact_hint >= 0 && g_nact_hint < nrhs
 #define MG_LAUNCH(kernel, grid, block, smem, stream, ...) \
   MG_LAUNCH_W(0, 0, kernel, grid, block, smem, stream, __VA_ARGS__)
 
-// one complex number from global to shared memory, in flight until its group is waited for
+// 16 bytes from global to shared memory, in flight until their group is waited for
+__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
+}
+// one complex number
 template <typename C>
 __device__ __forceinline__ void cp_async_elem(C* dst, const C* src) {
-  const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
   if constexpr (sizeof(C) == 16)
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
+    cp_async16(dst, src);
   else
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d), "l"(src) : "memory");
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
 }
 
 // Programmatic dependent launch: a kernel that begins with pdl_begin() may be launched with MG_LAUNCH_P, and the GPU

@@ -16,10 +16,6 @@
 
 namespace mg {
 
-__device__ __forceinline__ void cp_async16c(void* dst, const void* src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
-               : "memory");
-}
 // two consecutive complex numbers (16-byte aligned in FP32)
 __device__ __forceinline__ void load2(const float2* p, float2* v) {
   const float4 q = *reinterpret_cast<const float4*>(p);
@@ -113,11 +109,11 @@ __global__ void __launch_bounds__(64) k_coarse_apply16(const float2* __restrict_
   for (int q = tid; q < 5 * RG * 8; q += 64) {
     const int c = q & 7, g = (q >> 3) % RG, dir = (q >> 3) / RG, rhs = r0 + g;
     if (rhs < nrhs && !(active && !active[rhs]))
-      cp_async16c(sx + (dir * RG + g) * XP + 2 * c, x + rhs * n + (size_t)nbr_site(s, dir, Ls) * 16 + 2 * c);
+      cp_async16(sx + (dir * RG + g) * XP + 2 * c, x + rhs * n + (size_t)nbr_site(s, dir, Ls) * 16 + 2 * c);
   }
 #pragma unroll 5
   for (int q = tid; q < 640; q += 64)
-    cp_async16c(sw + (q >> 3) * XP + 2 * (q & 7), st + (size_t)s * 1280 + 2 * q);
+    cp_async16(sw + (q >> 3) * XP + 2 * (q & 7), st + (size_t)s * 1280 + 2 * q);
   asm volatile("cp.async.commit_group;" ::: "memory");
   asm volatile("cp.async.wait_group 0;" ::: "memory");
   __syncthreads();
@@ -496,14 +492,13 @@ __global__ void __launch_bounds__(256) k_restrict(const typename CT<R>::T* __res
   }
 }
 
-template <typename R, bool ADD, int DT, int AT, int NT>
-__global__ void __launch_bounds__(256) k_prolong(const typename CT<R>::T* __restrict__ P, int Ls, int d_, int agg_,
-                                                 int ntv_, const typename CT<R>::T* __restrict__ xc,
+template <typename R, bool ADD>
+__global__ void __launch_bounds__(256) k_prolong(const typename CT<R>::T* __restrict__ P, int Ls, int d, int agg,
+                                                 int ntv, const typename CT<R>::T* __restrict__ xc,
                                                  typename CT<R>::T* __restrict__ xf,
                                                  unsigned short* __restrict__ xf16, int bf, int nrhs,
                                                  const int* __restrict__ active) {
   typedef typename CT<R>::T C;
-  const int d = DT ? DT : d_, agg = AT ? AT : agg_, ntv = NT ? NT : ntv_;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int hd = d / 2, na = agg * agg, bsz = na * hd, dc = 2 * ntv, fa = na * d;
   const int G = max(1, 256 / fa);
@@ -573,12 +568,12 @@ __global__ void __launch_bounds__(16 / MM * (RG / RR))
   const char* Pa = reinterpret_cast<const char*>(P + (size_t)a * 2048);
   constexpr int CPS = 16 * (int)sizeof(C) / 16;  // 16-byte chunks of a site
   for (int q = tid; q < 2048 * (int)sizeof(C) / 16; q += T)
-    cp_async16c(reinterpret_cast<char*>(sP) + q * 16, Pa + q * 16);
+    cp_async16(reinterpret_cast<char*>(sP) + q * 16, Pa + q * 16);
   for (int q = tid; q < RG * 16 * CPS; q += T) {
     const int c = q % CPS, js = (q / CPS) & 15, g = q / (16 * CPS), rhs = r0 + g;
     if (rhs < nrhs && !(active && !active[rhs]) && !(half && (((js >> 3) + (js >> 1)) & 1))) {
       const size_t site = (size_t)(4 * AT + (js >> 2)) * Ls + 4 * AX + (js & 3);
-      cp_async16c(reinterpret_cast<char*>(sx + g * XP + js * 16) + c * 16,
+      cp_async16(reinterpret_cast<char*>(sx + g * XP + js * 16) + c * 16,
                   reinterpret_cast<const char*>(xf + rhs * n + site * 16) + c * 16);
     }
   }
@@ -640,7 +635,7 @@ __global__ void __launch_bounds__(128) k_prolong2(const typename CT<R>::T* __res
   if constexpr (D == 2) {
     constexpr int CPR = 8 * (int)sizeof(C) / 16;  // 16-byte chunks of a row
     for (int q = tid; q < 32 * CPR; q += 128)
-      cp_async16c(reinterpret_cast<char*>(sp + q / CPR * PP) + q % CPR * 16, reinterpret_cast<const char*>(Pa) + q * 16);
+      cp_async16(reinterpret_cast<char*>(sp + q / CPR * PP) + q % CPR * 16, reinterpret_cast<const char*>(Pa) + q * 16);
   }
   for (int q = tid; q < cnt * 16; q += 128) {
     const int rhs = r0 + (q >> 4);
@@ -793,8 +788,8 @@ static void prolong_launch(cudaStream_t stm, const typename CT<R>::T* P, int Ls,
   } else {
     const int na = agg * agg, bsz = na * d / 2, dc = 2 * ntv, G = std::max(1, 256 / (na * d));
     const size_t sm = sizeof(C) * ((size_t)2 * bsz * ntv + (size_t)G * dc);
-    set_smem_attr(k_prolong<R, ADD, 0, 0, 0>);
-    MG_LAUNCH_W(bytes, flops, (k_prolong<R, ADD, 0, 0, 0>), Lc * Lc, 256, sm, stm, P, Ls, d, agg, ntv, xc, xf,
+    set_smem_attr(k_prolong<R, ADD>);
+    MG_LAUNCH_W(bytes, flops, (k_prolong<R, ADD>), Lc * Lc, 256, sm, stm, P, Ls, d, agg, ntv, xc, xf,
                 xf16, bf, nrhs, active);
   }
 }

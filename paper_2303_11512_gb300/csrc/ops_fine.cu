@@ -236,7 +236,7 @@ template <typename R, typename LK>
 static void wilson_sites(cudaStream_t st, LK lk, R diag, int L, const typename CT<R>::T* x, typename CT<R>::T* y,
                          const typename CT<R>::T* b, int nrhs, const int* active, double bytes, double flops) {
   // blocks of 64 threads where 256 would leave most SMs without one (FP64: two FMAs a clock and SM bound it)
-  const int bt = (long)L * L * nrhs >= 152L * 256 * 2 ? 256 : 64;
+  const int bt = (long)L * L * nrhs >= 512L * sm_count() ? 256 : 64;
   const dim3 grid(cdiv((long)L * L, bt), nrhs);
   if (b)
     MG_LAUNCH_W(bytes, flops, (k_wilson<R, true, LK>), grid, bt, 0, st, lk, diag, L, x, y, b, active);
@@ -374,15 +374,6 @@ void fine_block_matrices(cudaStream_t st, const double2* l64, double diag, int L
 // nothing (SAP_ZERO: x counts as zero, the first half sweep of a cycle), or the other colour only (SAP_OTHER: x
 // counts as zero on this colour, the second half sweep).
 
-__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
-               : "memory");
-}
-__device__ __forceinline__ void cp_async8(void* dst, const void* src) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
-               : "memory");
-}
-
 // FP32, 4 x 4 blocks.  An item is one block; blockIdx.y picks the tile of RG right-hand sides, which a CTA keeps.
 // Two warps per CTA and one shared-memory stage (21 KB at RG = 16, ten CTAs per SM, each in another phase):
 //   fetch     f on the block, x on the block and on the 16 sites around it, the inverse, all by cp.async
@@ -438,10 +429,10 @@ __global__ void __launch_bounds__(64) k_sap_fine4_fp32(const float2* __restrict_
         cp_async16(reinterpret_cast<char*>(s.inv) + (tid + q * T) * 16, I + (tid + q * T) * 16);
       if (tid < 20) {
         const int i = tid / 5, j = tid - 5 * i;
-        cp_async8(&s.lx[tid], lk + 2 * ((t0 + i) * L + (j ? x0 + j - 1 : xm)));
+        cp_async_elem(&s.lx[tid], lk + 2 * ((t0 + i) * L + (j ? x0 + j - 1 : xm)));
       } else if (tid >= 32 && tid < 52) {
         const int i = (tid - 32) >> 2, j = tid & 3;
-        cp_async8(&s.lt[tid - 32], lk + 2 * ((i ? t0 + i - 1 : tm) * L + x0 + j) + 1);
+        cp_async_elem(&s.lt[tid - 32], lk + 2 * ((i ? t0 + i - 1 : tm) * L + x0 + j) + 1);
       }
 #pragma unroll
       for (int k = 0; k < RG / RTH; ++k) {
@@ -733,9 +724,7 @@ void sap_half_fine(cudaStream_t st, const typename CT<R>::T* links, R diag, int 
   }
   if constexpr (sizeof(R) == 4) {
     MG_CHECK_ARG(inv_transposed, "the FP32 fine smoother reads transposed block inverses");
-    int dev = 0, nsm = 152;
-    MG_CUDA(cudaGetDevice(&dev));
-    MG_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+    const int nsm = sm_count();
     // tile of right-hand sides: 8 where that takes the batch, else 16.  A tile of 32 needs fewer reads of the
     // inverse per FMA but leaves 6 CTAs per SM instead of 10: 115 us against 100 at L = 512, 32 rhs.
     auto go = [&](auto rg) {
@@ -782,9 +771,7 @@ void residual_restrict_fine(cudaStream_t st, const float2* links, float diag, in
   const int na = (L / 4) * (L / 4);
   const double ar = act_rhs(nrhs);
   const double bytes = na * (ar * (16 * 16 * 2 + 128.0) + 2048.0), flops = na * ar * (16 * 56.0 + 8.0 * 256);
-  int dev = 0, nsm = 152;
-  MG_CUDA(cudaGetDevice(&dev));
-  MG_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+  const int nsm = sm_count();
   auto go = [&](auto rg) {
     constexpr int RG = decltype(rg)::value, sm = (int)sizeof(SapF<RG, true>);
     constexpr int per_sm = std::min(16, 227 * 1024 / (sm + 1024));

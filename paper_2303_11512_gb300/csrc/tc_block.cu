@@ -74,10 +74,7 @@ __device__ __forceinline__ uint32_t tb_pack(float a, float b) {
   return BF == 2 ? f16x2_rn(a, b) : bf16x2_rn(a, b);
 }
 
-// 16-byte global -> shared copy without a register round trip (completion by commit / wait groups)
-__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
-}
+// completion of cp.async copies (no register round trip) by groups
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait1() { asm volatile("cp.async.wait_group 1;" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait0() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
