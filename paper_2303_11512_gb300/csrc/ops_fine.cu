@@ -248,8 +248,9 @@ static void wilson_sites(cudaStream_t st, LK lk, R diag, int L, const typename C
 // would leave the chip short of threads.  The line, with one rhs per thread, per site against walking: L = 512 with 4,
 // 12, 49, 244 rhs 17.5, 30.8, 86.2, 378 against 15.6, 31.4, 84.2, 357 us; L = 136 with 52, 173, 3460 rhs 12.5, 26.7, 371
 // against 12.3, 24.7, 366; below 64 columns a warp lies across slice groups and the per-site form wins (L = 16, 24, 48
-// with 12.8 M sites x rhs: 73.9, 81.4, 78.0 against 88.0, 94.6, 82.6).  At L = 512 with 256 rhs the walk takes 375 us (86 %
-// of the copy bandwidth) with one rhs per thread, 392 with two, 477 with four, 413 with 16 slices and one rhs.
+// with 12.8 M sites x rhs: 73.9, 81.4, 78.0 against 88.0, 94.6, 82.6).  At L = 512 with 244 rhs the walk takes 357 us with
+// one rhs per thread, 389 with two, 505 with four; with 256 rhs 367 us alone (0.88 of the copy bandwidth), 413 against 375
+// in an earlier form with 16 slices instead of 8.
 int wilson_variant(int L, int nrhs, int rpt) {
   const double threads = (double)L * L * nrhs / WT, least = 1024.0 * sm_count();
   if (L < 64 || threads < least) return 0;
