@@ -777,10 +777,11 @@ static void prolong_launch(cudaStream_t stm, const typename CT<R>::T* P, int Ls,
   const bool aligned = ((uintptr_t)xf & 15) == 0;  // 16-byte accesses; other vectors take the general kernel
   const int aggs = Lc * Lc, nsm = sm_count();
   // tiles of 8 or 32: FP64 the one whose fullest SM has the fewer right-hand sides (8 while that leaves SMs without a
-  // tile); FP32 8 for few aggregates, which spreads a batch over more CTAs
+  // tile; of equals 8 for even numbers of whole tiles: 256 fine aggregates with 16, 24 right-hand sides 10.5, 18.1 us in
+  // tiles of 8 and 13.9, 14.2 in tiles of 32); FP32 8 for few aggregates, which spreads a batch over more CTAs
+  const long f8 = fullest_sm(aggs, nrhs, 8, nsm), f32 = fullest_sm(aggs, nrhs, 32, nsm);
   const bool tile8 = nrhs <= 8 || (sizeof(R) == 4 ? d == 16 && aggs * cdiv(nrhs, 32) < 4 * nsm
-                                                  : aggs * cdiv(nrhs, 8) <= nsm ||
-                                                        fullest_sm(aggs, nrhs, 8, nsm) < fullest_sm(aggs, nrhs, 32, nsm));
+                                                  : aggs * cdiv(nrhs, 8) <= nsm || f8 < f32 || (f8 == f32 && nrhs % 16 == 0));
   if (agg == 4 && ntv == 8 && d == 2 && aligned) {
     tile8 ? go(std::integral_constant<int, 2>(), I8()) : go(std::integral_constant<int, 2>(), I32());
   } else if (agg == 4 && ntv == 8 && d == 16 && aligned) {
