@@ -47,6 +47,7 @@ int mgmlmc_ctx_create(void* stream, mgmlmc_ctx** out) {
   if (!c) return MGMLMC_ERR_OOM;
   c->stream = (cudaStream_t)stream;
   if (cudaGetDevice(&c->device) != cudaSuccess ||
+      cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, c->device) != cudaSuccess ||
       cudaMallocHost((void**)&c->pinned, 64 * sizeof(int) + 64) != cudaSuccess ||
       cudaEventCreateWithFlags(&c->flag_event[0], cudaEventDisableTiming) != cudaSuccess ||
       cudaEventCreateWithFlags(&c->flag_event[1], cudaEventDisableTiming) != cudaSuccess) {

@@ -4,7 +4,6 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
-#include <atomic>
 #include <cstdio>
 #include <cstring>
 #include <mutex>
@@ -278,15 +277,14 @@ struct DBuf {
 };
 
 inline unsigned cdiv(long a, long b) { return (unsigned)((a + b - 1) / b); }
-inline int sm_count() {  // of the current device (the attribute is looked up once per device: calls are microseconds)
-  static std::atomic<int> known[64];
-  int dev = 0;
+// SMs of the device of this thread's current call (a thread's variable that every call sets, because the smallest calls
+// take 5 us); looked up outside of any
+extern thread_local int g_sms;
+inline int sm_count() {
+  if (g_sms > 0) return g_sms;
+  int dev = 0, n = 0;
   MG_CUDA(cudaGetDevice(&dev));
-  int n = dev < 64 ? known[dev].load(std::memory_order_relaxed) : 0;
-  if (!n) {
-    MG_CUDA(cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev));
-    if (dev < 64) known[dev].store(n, std::memory_order_relaxed);
-  }
+  MG_CUDA(cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev));
   return n;
 }
 

@@ -15,6 +15,7 @@ thread_local int64_t* g_launch_counter = nullptr;
 thread_local KTimer* g_timer = nullptr;
 thread_local int g_nact_hint = -1;
 thread_local int g_capturing = -1;
+thread_local int g_sms = 0;
 
 // ---------------------------------------------------------------- helpers
 template <typename R> static inline const typename CT<R>::T* links_of(const LevelData& L) {

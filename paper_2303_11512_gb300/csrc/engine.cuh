@@ -14,7 +14,7 @@
 
 struct mgmlmc_ctx {
   cudaStream_t stream = 0;
-  int device = 0;
+  int device = 0, sms = 0;
   std::string err;
   int64_t launches = 0;
   int* pinned = nullptr;  // small pinned host buffer for flags (64 ints, then pinned_d)
@@ -127,12 +127,12 @@ struct LaunchScope {
     g_timer = c->timer.on ? &c->timer : nullptr;
     g_nact_hint = -1;
     g_capturing = -1;
+    g_sms = c->sms;
   }
   ~LaunchScope() {
     g_launch_counter = nullptr;
     g_timer = nullptr;
     g_nact_hint = -1;
-    g_capturing = -1;
   }
 };
 
